@@ -125,7 +125,7 @@ struct dgswe_ctx {
   int np = 0, rv = 0, gv = 0;      // modes, record and geometry sizes (16-byte units)
   long long E = 0, N = 0;          // padded element count, node count
   std::vector<long long> eoff, noff;
-  DevBuf rec[3], nbr, geo, nodes, node_xy, xy64, hbn, rain_e, rain_node, node_scen, lim, scen, tile_scen, tile_meta, xy0,
+  DevBuf rec[3], nbr, geo, nodes, node_xy, xy64, hbn, rain_e, rain_node, node_scen, lim, rain_rec, scen, tile_scen, tile_meta, xy0,
       ledger, ctl,
       einv, grids, rivers, scratch,
       gather_buf, edges, slots;
@@ -140,7 +140,7 @@ struct dgswe_ctx {
   int block = 128, waves = 1, split = 1;
   bool autotune = true;
   bool graphs = true;  // replay steps from CUDA graphs (else direct launches)
-  bool grid_rain = false;  // some scenario has gridded rain: a node kernel runs before each stage
+  bool grid_rain = false;  // gridded rain without element records: a node kernel runs before each stage
   int feat = FT_ALL;       // features of the run (Feature bits): selects the tile-kernel instantiation
   long long nn_total = 0;
   int grid = 0;
@@ -155,7 +155,7 @@ struct dgswe_ctx {
     DevBuf* bufs[] = {&rec[0], &rec[1], &rec[2], &nbr, &geo, &nodes, &node_xy, &xy64, &hbn, &rain_e, &scen,
                       &tile_scen, &tile_meta, &xy0, &ledger, &ctl, &einv, &grids, &rivers, &scratch, &gather_buf,
                       &edges, &slots,
-                      &rain_node, &node_scen, &lim};
+                      &rain_node, &node_scen, &lim, &rain_rec};
     for (DevBuf* b : bufs) b->alloc(0);
     if (g1) cudaGraphExecDestroy(g1);
     if (gK) cudaGraphExecDestroy(gK);
@@ -584,8 +584,21 @@ static int build_layout(dgswe_h h) {
     }
   }
   h->nn_total = N;
-  h->grid_rain = false;
-  for (size_t s = 0; s < ns; ++s) h->grid_rain = h->grid_rain || h->sc[s].rain_kind == 3;
+  // gridded rain: element means of every record, where they fit (at most 8 GiB and a quarter of the
+  // free memory: 25 hourly records of 8M triangles are 0.8 GB); else a node kernel interpolates the
+  // grid at every stage
+  size_t rr_elems = 0, free_b = 0, total_b = 0;
+  std::vector<size_t> rr_off(ns, 0);
+  for (size_t s = 0; s < ns; ++s)
+    if (h->sc[s].rain_kind == 3) {
+      rr_off[s] = rr_elems;
+      rr_elems += (size_t)h->sc[s].gnt * h->sc[s].m.ne;
+    }
+  const size_t rr_bytes = (mx ? 4 : 8) * rr_elems;
+  CU(cudaMemGetInfo(&free_b, &total_b));
+  const bool records = rr_elems > 0 && rr_bytes <= std::min<size_t>((size_t)8 << 30, free_b / 4);
+  if (h->rain_rec.alloc(records ? rr_bytes : 0)) return fail(DGSWE_ENOMEM, "device allocation of %zu bytes failed", rr_bytes);
+  h->grid_rain = rr_elems > 0 && !records;
   CU(cudaMemset(h->ctl.p, 0, sizeof(Ctl)));
   // per-scenario parameter blocks (dt filled in later)
   std::vector<ScenDev> sd(ns);
@@ -599,6 +612,8 @@ static int build_layout(dgswe_h h) {
     D.rain_kind = S.rain_kind;
     D.gnx = S.gnx; D.gny = S.gny; D.gnt = S.gnt;
     D.grid = S.rain_kind == 3 ? h->grids.as<float>() + grid_off[s] : nullptr;
+    D.rrec = (records && S.rain_kind == 3) ? static_cast<const void*>(h->rain_rec.as<char>() + (mx ? 4 : 8) * rr_off[s]) : nullptr;
+    D.rstride = S.m.ne;
     D.nseg = (int32_t)S.tamp.size();
     D.rnseg = S.rnseg;
     D.rnt = S.rnt;
@@ -653,6 +668,15 @@ static int build_layout(dgswe_h h) {
   CU(cudaMemset(h->ledger.p, 0, 16 * (size_t)h->wslots * ns));
   h->wcur = 0;
   CU(cudaMemcpy(h->scen.p, sd.data(), sizeof(ScenDev) * ns, cudaMemcpyHostToDevice));
+  for (size_t s = 0; s < ns; ++s) {
+    if (!sd[s].rrec) continue;
+    cudaError_t ce = mx ? launch_rain_records<Mixed>(h->scen.as<ScenDev>(), (int)s, h->nodes.as<int4>(), h->xy64.as<double>(),
+                                                     h->sc[s].m.ne, sd[s].rstride, h->rain_rec.as<float>() + rr_off[s], h->stream)
+                        : launch_rain_records<Fp64>(h->scen.as<ScenDev>(), (int)s, h->nodes.as<int4>(), h->xy64.as<double>(),
+                                                    h->sc[s].m.ne, sd[s].rstride, h->rain_rec.as<double>() + rr_off[s], h->stream);
+    if (ce != cudaSuccess) return fail(DGSWE_ECUDA, "rain record launch: %s", cudaGetErrorString(ce));
+    h->launches++;
+  }
   h->led_rain.assign(ns, 0.0);
   h->led_bdry.assign(ns, 0.0);
   h->V0.assign(ns, 0.0);

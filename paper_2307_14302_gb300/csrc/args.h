@@ -142,6 +142,10 @@ cudaError_t launch_limiter(const StageArgs<Pol>& a, long long ne, cudaStream_t s
 // gridded rain (rain_kind 3) interpolated to every node at the stage time: a.rain_node[0, nn)
 template <class Pol>
 cudaError_t launch_node_rain(const StageArgs<Pol>& a, long long nn, cudaStream_t s);
+// gridded rain of every record averaged to the elements of one scenario: rrec[record][element], m/s
+template <class Pol>
+cudaError_t launch_rain_records(const ScenDev* scen, int sc, const int4* nodes, const double* xy64, long long ne,
+                                long long stride, typename PolT<Pol>::T* rrec, cudaStream_t s);
 // partial FP64 sums of A*mean(zeta) and A*mean(H) over [begin, end): partials[4*block]
 template <class Pol>
 cudaError_t launch_volume(int p, const uint4* rec, const uint4* geo, long long begin, long long end,

@@ -101,6 +101,8 @@ struct ScenDev {
   double rt0, ridt;                // first record time, 1 / record interval
   const double* river;             // [rnt][rnseg] m^2/s into the domain
   const float* grid;               // [gnt][gny][gnx] mm/h
+  const void* rrec;                // [gnt][rstride] element rain of every grid record (T), or null (node kernel)
+  long long rstride;               // elements per record of rrec
   ForcingT<float> f;
   ForcingT<double> d;
 };

@@ -883,6 +883,7 @@ __global__ void DG_TILE_BOUNDS tile_kernel(const StageArgs<Pol> a) {
   const ScenDev* Sp = a.scen;
   double t64 = 0.0;
   int rain_kind = 0, press = 0;
+  RainRec<T> rr = {nullptr, nullptr, T(0)};  // gridded rain: the two records around the stage time
   uint32_t ph = 0;  // parity of the next completion: bit 0 buffer 0, bit 1 buffer 1
   if (gw < a.ntiles) issue(gw, 0);
 
@@ -913,6 +914,14 @@ __global__ void DG_TILE_BOUNDS tile_kernel(const StageArgs<Pol> a) {
       t64 = Sp->d.t0 + stepd * Sp->d.dt;  // stage time, formed in FP64
       rain_kind = ft_rain(FT) >= 0 ? ft_rain(FT) : Sp->rain_kind;
       press = (FT & FT_PRESS) ? Sp->press : 0;
+      if (rain_kind == 3) {
+        rr.r0 = nullptr;
+        if (Sp->rrec) {
+          rr = rain_records<T>(*Sp, t64);
+          rr.r0 -= Sp->elem_begin;
+          rr.r1 -= Sp->elem_begin;
+        }
+      }
     }
     const ScenDev& S = *Sp;
     const int e0 = tile * TILE, e = e0 + lane;
@@ -993,8 +1002,18 @@ __global__ void DG_TILE_BOUNDS tile_kernel(const StageArgs<Pol> a) {
     T Rz[NP], Rx[NP], Ry[NP];
     T Re = 0;
     if (valid) {
-      // gridded rain: node indices now (coalesced), their nodal rates after the area integrals
-      const int4 nd = (rain_kind == 3) ? __ldg(a.nodes + e) : make_int4(0, 0, 0, 0);
+      // gridded rain: the element's two records now, blended after the area integrals; without
+      // records the node indices now, their nodal rates then
+      T re0 = T(0), re1 = T(0);
+      int4 nd = make_int4(0, 0, 0, 0);
+      if (rain_kind == 3) {
+        if (rr.r0) {
+          re0 = __ldg(rr.r0 + e);
+          re1 = __ldg(rr.r1 + e);
+        } else {
+          nd = __ldg(a.nodes + e);
+        }
+      }
       Elem<P, Pol> E;
       {
         Raw<RV> r;
@@ -1033,7 +1052,9 @@ __global__ void DG_TILE_BOUNDS tile_kernel(const StageArgs<Pol> a) {
             acc += (r < rm) ? rp * (T(0.5) + T(0.5) * fdiv(r, rm)) : rp * fexp(-fdiv(r - rm, re));
         }
         Re = acc * T(1.0 / 3.0);
-      } else if (rain_kind == 3) {  // gridded: nodal rates interpolated by the node kernel of this stage
+      } else if (rain_kind == 3 && rr.r0) {
+        Re = rain_blend<T>(re0, re1, rr.f);
+      } else if (rain_kind == 3) {  // nodal rates interpolated by the node kernel of this stage
         Re = (a.rain_node[nd.x] + a.rain_node[nd.y] + a.rain_node[nd.z]) * T(1.0 / 3.0);
       }
     }
