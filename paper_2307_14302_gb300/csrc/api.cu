@@ -125,7 +125,7 @@ struct dgswe_ctx {
   int np = 0, rv = 0, gv = 0;      // modes, record and geometry sizes (16-byte units)
   long long E = 0, N = 0;          // padded element count, node count
   std::vector<long long> eoff, noff;
-  DevBuf rec[3], nbr, geo, nodes, node_xy, xy64, hbn, rain_e, rain_node, node_scen, lim, rain_rec, scen, tile_scen, tile_meta, xy0,
+  DevBuf rec[3], nbr, geo, nodes, node_xy, xy64, hbn, rain_e, rain_node, node_scen, lim, rain_rec, scen, tile_scen, tile_meta, plan, plan_x, xy0,
       ledger, ctl,
       einv, grids, rivers, scratch,
       gather_buf, edges, slots;
@@ -155,7 +155,7 @@ struct dgswe_ctx {
     DevBuf* bufs[] = {&rec[0], &rec[1], &rec[2], &nbr, &geo, &nodes, &node_xy, &xy64, &hbn, &rain_e, &scen,
                       &tile_scen, &tile_meta, &xy0, &ledger, &ctl, &einv, &grids, &rivers, &scratch, &gather_buf,
                       &edges, &slots,
-                      &rain_node, &node_scen, &lim, &rain_rec};
+                      &rain_node, &node_scen, &lim, &rain_rec, &plan, &plan_x};
     for (DevBuf* b : bufs) b->alloc(0);
     if (g1) cudaGraphExecDestroy(g1);
     if (gK) cudaGraphExecDestroy(gK);
@@ -666,6 +666,14 @@ static int build_layout(dgswe_h h) {
   CU(cudaMemcpy(h->tile_scen.p, ts.data(), 4 * ts.size(), cudaMemcpyHostToDevice));
   CU(cudaMemcpy(h->tile_meta.p, tm.data(), 4 * tm.size(), cudaMemcpyHostToDevice));
   CU(cudaMemset(h->ledger.p, 0, 16 * (size_t)h->wslots * ns));
+  size_t pb = 0, pxb = 0;
+  if (mx) plan_bytes<Mixed>(h->ntiles, pb, pxb);
+  else plan_bytes<Fp64>(h->ntiles, pb, pxb);
+  if (h->plan.alloc(pb) || h->plan_x.alloc(pxb)) return fail(DGSWE_ENOMEM, "device allocation failed");
+  CU(cudaDeviceSynchronize());  // the uploads above ran on the default stream, this stream does not wait for it
+  CU(mx ? launch_plan<Mixed>(h->nbr.as<int4>(), h->tile_meta.as<int4>(), h->ntiles, h->plan.as<uint4>(), h->plan_x.as<int32_t>(), h->stream)
+        : launch_plan<Fp64>(h->nbr.as<int4>(), h->tile_meta.as<int4>(), h->ntiles, h->plan.as<uint4>(), h->plan_x.as<int32_t>(), h->stream));
+  h->launches++;
   h->wcur = 0;
   CU(cudaMemcpy(h->scen.p, sd.data(), sizeof(ScenDev) * ns, cudaMemcpyHostToDevice));
   for (size_t s = 0; s < ns; ++s) {
@@ -750,6 +758,8 @@ static StageArgs<Pol> make_args(dgswe_h h, int stage, int tune) {
   a.scen = h->scen.as<ScenDev>();
   a.tile_scen = h->tile_scen.as<int32_t>();
   a.tile_meta = h->tile_meta.as<int4>();
+  a.plan = h->plan.as<uint4>();
+  a.plan_x = h->plan_x.as<int32_t>();
   a.xy0 = h->xy0.as<uint4>();
   a.ledger = h->ledger.as<double>();
   a.ctl = h->ctl.as<Ctl>();

@@ -41,6 +41,8 @@ struct StageArgs {
   const ScenDev* scen;
   const int32_t* tile_scen;  // scenario of each 32-element tile
   const int4* tile_meta;   // tile form: per tile {scenario, elements present (0..32), 0, 0}
+  const uint4* plan;       // tile form: per tile the edge words, halo elements, Manning, meta (tile.cuh)
+  const int32_t* plan_x;   // tile form: overflow of the plan, PLAN_X words per tile
   const uint4* xy0;        // tile form: first vertex of each element, [E] float2 (mixed) / double2 (FP64)
   double* ledger;          // [scenario][wslots][2]: rain volume, boundary inflow volume per warp
   Ctl* ctl;
@@ -111,6 +113,15 @@ DG_HD constexpr int ft_pow2(int ft) {
   return (ft & (FT_POW2 | FT_GENSSP)) == FT_POW2 ? 1 : (ft & (FT_POW2 | FT_GENSSP)) == FT_GENSSP ? 0 : -1;
 }
 DG_HD constexpr bool ft_covers(int ft, int need) { return (need & ~ft) == 0; }
+// the sets with specialised mixed-precision instantiations (Roe flux):
+// walls only, constant nodal rain, Manning friction, SSP(2,2)
+constexpr int FT_WALL_NODAL = FT_RAIN1 | FT_MANNING | FT_POW2;
+// tidal boundary, parametric storm rain, Manning friction, SSP(2,2)
+constexpr int FT_TIDE_STORM = FT_OCEAN | FT_RAIN2 | FT_MANNING | FT_POW2;
+// tidal boundary, gridded rain, Manning friction, SSP(2,2)
+constexpr int FT_TIDE_GRID = FT_OCEAN | FT_RAIN3 | FT_MANNING | FT_POW2;
+// tidal boundary, parametric storm rain, pressure set-up, Manning friction, SSP(3,3) (p = 2)
+constexpr int FT_TIDE_STORM_SETUP = FT_OCEAN | FT_RAIN2 | FT_PRESS | FT_MANNING | FT_POW2 | FT_GENSSP;
 
 // tile form (split = 2): reference tables and shared-memory limits of its translation units,
 // the launch (the specialised instantiation that covers the run's features, else the generic
@@ -130,6 +141,11 @@ int tile_spec_blocks_per_sm(int p, int flux, int feat, int block);
 int tile_spec_features(int p, int flux, int feat);
 // reference tables and shared-memory limits of the specialised instantiations' translation unit
 cudaError_t upload_tile_spec_tables(int p, const RefTab<float>& tf, const RefTab<double>& td);
+// tile plans of the mesh (sizes: plan_bytes), from the neighbour codes and the tiles' metadata
+template <class Pol>
+cudaError_t launch_plan(const int4* nbr, const int4* tile_meta, int ntiles, uint4* plan, int32_t* plan_x, cudaStream_t s);
+template <class Pol>
+void plan_bytes(int ntiles, size_t& plan, size_t& plan_x);
 // edge kernel of the split path: one thread per interior edge, writes both sides' slots
 template <class Pol>
 cudaError_t launch_edges(int p, int flux, const StageArgs<Pol>& a, int grid, int block, cudaStream_t s);

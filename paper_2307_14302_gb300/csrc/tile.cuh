@@ -46,47 +46,32 @@ constexpr int HALO = 32;    // staged out-of-tile neighbour records per tile
 static_assert(HALO == TILE, "own and halo records share one vector stride in shared memory");
 constexpr int TE_MAX = 96;  // edges touching a 32-element tile (3 per element at most)
 
-// edge descriptor: left side, right side (or boundary code), and the left side's scaled outward
-// normal (written by the lane that owns the edge, from its own geometry)
+// The tile plan: what the neighbour codes say about a tile's edges, laid out once per mesh by
+// plan_kernel (the connectivity never changes) and copied with the tile's other data.  One 32-bit
+// word per edge:
+//   bits 0-8    left side: source << 2 | local edge
+//   bits 9-17   right side, or the boundary code (bit 18): 0 land, 1 + tidal segment,
+//               1 + MAXSEG + river segment
+//   bit 18      boundary edge;  bit 19  the right side is the tile's own element (whose geometry
+//               holds the edge's normal, negated)
+// sources: 0-31 own element, 32-63 staged halo record, 64-127 entry source - 64 of the tile's list
+// of further neighbours (none on Hilbert-ordered meshes; read from global memory).  In-tile edges
+// come first, then the edges to other tiles, then the boundary edges: the first round of the edge
+// phase does not wait for the halo.  Per tile: EDGE_ROUND2 = 64 words, the 32 halo elements, (mixed
+// path) the Manning coefficients, and {scenario, elements present, counts, 0}; edges 64-95 and
+// neighbours 32-95 are in the overflow array, which a lane reads directly.
+// Before, every stage rebuilt this per tile from the neighbour codes (nine ballots, the population
+// counts, a descriptor of two sides and a normal per edge): about 190 of 1,940 warp instructions,
+// with the halo loads waiting for it.
+constexpr int EDGE_INLINE = 64;
+constexpr int PLAN_X = 32 + 64;  // overflow words per tile: edges 64..95, neighbours 32..95
+constexpr unsigned ED_BND = 1u << 18, ED_OWN_R = 1u << 19;
 template <class T>
-struct EdgeDesc;
-template <>
-struct alignas(16) EdgeDesc<float> {
-  int sL, sR;
-  float lnx, lny;
-};
-template <>
-struct alignas(16) EdgeDesc<double> {
-  int sL, sR, pad0, pad1;
-  double lnx, lny;
-};
-__device__ __forceinline__ void put_desc(EdgeDesc<float>* d, int i, int sL, int sR, float lnx, float lny) {
-  reinterpret_cast<int4*>(d)[i] = make_int4(sL, sR, __float_as_int(lnx), __float_as_int(lny));
-}
-__device__ __forceinline__ void put_desc(EdgeDesc<double>* d, int i, int sL, int sR, double lnx, double lny) {
-  int4* p = reinterpret_cast<int4*>(d) + 2 * i;
-  p[0] = make_int4(sL, sR, 0, 0);
-  reinterpret_cast<double2*>(p)[1] = make_double2(lnx, lny);
-}
-__device__ __forceinline__ void get_desc(const EdgeDesc<float>* d, int i, int& sL, int& sR, float& lnx, float& lny) {
-  const int4 v = reinterpret_cast<const int4*>(d)[i];
-  sL = v.x;
-  sR = v.y;
-  lnx = __int_as_float(v.z);
-  lny = __int_as_float(v.w);
-}
-__device__ __forceinline__ void get_desc(const EdgeDesc<double>* d, int i, int& sL, int& sR, double& lnx,
-                                         double& lny) {
-  const int4* p = reinterpret_cast<const int4*>(d) + 2 * i;
-  const int4 v = p[0];
-  const double2 n = reinterpret_cast<const double2*>(p)[1];
-  sL = v.x;
-  sR = v.y;
-  lnx = n.x;
-  lny = n.y;
+__host__ __device__ constexpr int plan_vec() {  // 16-byte units per tile
+  return (EDGE_INLINE + HALO + (sizeof(T) == 4 ? TILE : 0)) / 4 + 1;
 }
 
-template <int P, class Pol>
+template <int P, class Pol, int FT = FT_ALL>
 struct TileLayout {
   using T = typename Pol::T;
   static constexpr int NG = P + 1;
@@ -98,32 +83,27 @@ struct TileLayout {
   static constexpr bool MASSV = (NG % 2) == 1;
   static constexpr int NV = 3 * NG + (MASSV ? 1 : 0);
   static constexpr int NPR = (NV + 1) / 2;
-  static constexpr int XV = sizeof(T) == 4 ? 16 : 32;          // first vertices of a tile, 16-byte units
+  // first vertices of a tile (storm rain and pressure set-up only), 16-byte units
+  static constexpr int XV = (FT & (FT_RAIN2 | FT_PRESS)) ? (sizeof(T) == 4 ? 16 : 32) : 0;
   // one buffer: records [RV][32] (the tile's block of the tile-blocked record array), geometry
-  // [32][GV], neighbour codes [32], first vertices, the tile's metadata {scenario, elements
-  // present}, all filled by the TMA batch
+  // [32][GV], plan, first vertices, all filled by the TMA batch
+  static constexpr int PV = plan_vec<T>();
   static constexpr int O_GEO = TILE * RV;
-  static constexpr int O_NBR = O_GEO + TILE * GV;
-  static constexpr int O_XY = O_NBR + TILE;
-  static constexpr int O_META = O_XY + XV;
-  static constexpr int COPIED = O_META + 1;
-  // the edge slots [3][NPR][32] (pairs of T) overlay the geometry, codes, vertices and metadata,
-  // which every lane has read into registers (or into the edge descriptors) before the edge phase
-  static constexpr int O_FLX = O_GEO;
-  static constexpr int FLXV = 3 * NPR * 32 * 2 * (int)sizeof(T) / 16;
-  static constexpr int BUF = (O_FLX + FLXV > COPIED) ? O_FLX + FLXV : COPIED;
-  static constexpr int BUF0 = 0;
-  static constexpr int BUF1 = BUF;
+  static constexpr int O_PLAN = O_GEO + TILE * GV;
+  static constexpr int O_HALO = O_PLAN + EDGE_INLINE / 4;      // halo element indices
+  static constexpr int O_MAN = O_HALO + HALO / 4;              // Manning coefficients (mixed)
+  static constexpr int O_META = O_PLAN + PV - 1;
+  static constexpr int O_XY = O_PLAN + PV;
+  static constexpr int BUF = O_XY + XV;
   static constexpr int HAL = 2 * BUF;                          // [RV][HALO]
-  static constexpr int DESC = HAL + HALO * RV;                 // [96] EdgeDesc<T>
-  static constexpr int DV = (int)sizeof(EdgeDesc<T>) / 16;
-  static constexpr int BAR = DESC + TE_MAX * DV;               // two 8-byte mbarriers
+  static constexpr int FLX = HAL + HALO * RV;                  // edge slots [3][NPR][32], pairs of T
+  static constexpr int BAR = FLX + 3 * NPR * 32 * 2 * (int)sizeof(T) / 16;  // two 8-byte mbarriers
   static constexpr int VEC = BAR + 1;                          // 16-byte units per warp
-  static constexpr unsigned TILE_BYTES = 16u * COPIED;         // bytes of one buffer's copies
+  static constexpr unsigned TILE_BYTES = 16u * BUF;            // bytes of one buffer's copies
 };
-template <int P, class Pol>
+template <int P, class Pol, int FT = FT_ALL>
 __host__ __device__ constexpr int tile_smem_bytes(int block) {
-  return 16 * TileLayout<P, Pol>::VEC * (block / 32);
+  return 16 * TileLayout<P, Pol, FT>::VEC * (block / 32);
 }
 
 // ------------------------------------------------------------------ TMA bulk copies -----
@@ -173,8 +153,9 @@ __device__ __noinline__ void tile_timeout(const StageArgs<Pol>& a, uint32_t bar,
   (void)mbar_wait(bar, parity);
 }
 
-// static geometry record from shared memory (layout of load_geo)
-__device__ __forceinline__ void geo_from(const uint4* g, const int4& nb, Geo<Mixed>& G) {
+// static geometry record from shared memory (layout of load_geo); the Manning coefficient of the
+// mixed path is in the tile plan
+__device__ __forceinline__ void geo_from(const uint4* g, const float* man, Geo<Mixed>& G) {
   const uint4 a = g[0], b = g[1], c = g[2];
   G.lnx[0] = __uint_as_float(a.x); G.lny[0] = __uint_as_float(a.y);
   G.lnx[1] = __uint_as_float(a.z); G.lny[1] = __uint_as_float(a.w);
@@ -182,9 +163,9 @@ __device__ __forceinline__ void geo_from(const uint4* g, const int4& nb, Geo<Mix
   G.hbm = {__uint_as_float(b.z), __uint_as_float(b.w)};
   G.A = {__uint_as_float(c.x), __uint_as_float(c.y)};
   G.invA = {__uint_as_float(c.z), __uint_as_float(c.w)};
-  G.man = __int_as_float(nb.w);
+  G.man = *man;
 }
-__device__ __forceinline__ void geo_from(const uint4* g, const int4&, Geo<Fp64>& G) {
+__device__ __forceinline__ void geo_from(const uint4* g, const float*, Geo<Fp64>& G) {
   uint4 v[5];
 #pragma unroll
   for (int i = 0; i < 5; ++i) v[i] = g[i];
@@ -509,20 +490,30 @@ __device__ __forceinline__ void tile_area(const Elem<P, Pol>& E, const Geo<Pol>&
 }
 
 // ---------------------------------------------------------------------- edge phase ------
-// record of a side: own (src < 32: [RV][32]) or staged halo (src < 64: [RV][HALO]) records in
-// shared memory, vector-major, else the global record of element src - 64
-template <int RV>
-__device__ __forceinline__ void fetch_side(const uint4* own, const uint4* halo, const uint4* __restrict__ gin, int src,
-                                           Raw<RV>& r) {
+// record of a side: own (src < 32) or staged halo (src < 64) records [RV][32] in shared memory,
+// else neighbour src - 32 of the tile's list, read by far(element, record)
+template <int RV, class Far>
+__device__ __forceinline__ void fetch_side(const uint4* own, const uint4* halo, const Far& far,
+                                           const int32_t* __restrict__ over, int src, Raw<RV>& r) {
   if (src < 64) {  // shared memory, read as such (not through a generic address)
     const uint32_t p = smem_u32(src < 32 ? own + src : halo + (src - 32));
     constexpr uint32_t stride = 16u * TILE;  // HALO == TILE: one stride for both
 #pragma unroll
     for (int v = 0; v < RV; ++v) r.v[v] = lds128(p + stride * v);
   } else {
-#pragma unroll
-    for (int v = 0; v < RV; ++v) r.v[v] = __ldg(gin + rec_at<RV>(src - 64, v));
+    far(__ldg(over + 32 + (src - 64)), r);
   }
+}
+// scaled normal of local edge j of own element e from the geometry block
+__device__ __forceinline__ void edge_normal(const uint4* geo, int e, int j, float& nx, float& ny) {
+  const float2 n = reinterpret_cast<const float2*>(geo + 3 * e)[j];
+  nx = n.x;
+  ny = n.y;
+}
+__device__ __forceinline__ void edge_normal(const uint4* geo, int e, int j, double& nx, double& ny) {
+  const double2 n = reinterpret_cast<const double2*>(geo + 5 * e)[j];
+  nx = n.x;
+  ny = n.y;
 }
 
 // one side's edge slot at flx[(j NPR + i) 32 + lane], pairs of T: Gz[NG], Gx[NG], Gy[NG] (, mass)
@@ -585,24 +576,29 @@ __device__ __forceinline__ T wall_coef(const Trace<T>& t, T nx, T ny, T g, T H0)
   return qn * (un + c) + pdev(t.d, t.H, g);
 }
 
-template <int P, int FLUX, class Pol, int FT>
+template <int P, int FLUX, class Pol, int FT, class Far>
 __device__ __forceinline__ void tile_edge(const StageArgs<Pol>& a, const ScenDev& S, const uint4* own,
-                                          const uint4* halo, const EdgeDesc<typename Pol::T>* desc, void* flx, int i,
-                                          const typename Pol::T (*ephi)[P + 1][np_of(P)], const float4* ephi4,
-                                          double t64,
-                                          typename Pol::Acc& bdry_acc) {
+                                          const uint4* halo, const uint4* geo, const Far& far, const int32_t* over,
+                                          void* flx, unsigned ed, const typename Pol::T (*ephi)[P + 1][np_of(P)],
+                                          const float4* ephi4, double t64, typename Pol::Acc& bdry_acc) {
   using T = typename Pol::T;
-  using L = TileLayout<P, Pol>;
+  using L = TileLayout<P, Pol, FT>;
   constexpr int NG = P + 1, RV = L::RV, NPR = L::NPR, NV = L::NV;
   constexpr bool MASSV = L::MASSV;
   const RefTab<T>& tab = ctab<T, P>();
   const T g = a.g, H0 = a.H0;
-  int sL, sR;
-  T lnx, lny;  // L's scaled outward normal
-  get_desc(desc, i, sL, sR, lnx, lny);
-  const int jL = sL & 3, srcL = sL >> 2;
+  const int jL = ed & 3, srcL = (ed >> 2) & 127;
+  const int sR = (ed >> 9) & 511;  // right side, or the boundary code
   Raw<RV> rl;
-  fetch_side<RV>(own, halo, a.in, srcL, rl);
+  fetch_side<RV>(own, halo, far, over, srcL, rl);
+  T lnx, lny;  // L's scaled outward normal, from the own element's geometry
+  if (ed & ED_OWN_R) {
+    edge_normal(geo, sR >> 2, sR & 3, lnx, lny);
+    lnx = -lnx;
+    lny = -lny;
+  } else {
+    edge_normal(geo, srcL, jL, lnx, lny);
+  }
   Elem<P, Pol> EL;
   unpack<P>(rl, EL);
   T len, il;  // edge length and its inverse
@@ -627,9 +623,9 @@ __device__ __forceinline__ void tile_edge(const StageArgs<Pol>& a, const ScenDev
   }
   // boundary kind (an instantiation without a kind treats such an edge as a wall; the host never
   // selects it for a run that has one)
-  const bool interior = sR >= 0;
-  const bool river_e = (FT & FT_RIVER) && sR <= -2 - MAXSEG;
-  const bool ocean_e = (FT & FT_OCEAN) && sR <= -2 && sR > -2 - MAXSEG;
+  const bool interior = !(ed & ED_BND);
+  const bool river_e = (FT & FT_RIVER) && !interior && sR > MAXSEG;
+  const bool ocean_e = (FT & FT_OCEAN) && !interior && sR >= 1 && sR <= MAXSEG;
   const bool land = !interior && !river_e && !ocean_e;
   const bool dryL = (EL.flags & FLAG_DRY) != 0;
   bool dryR = false, river = false;
@@ -639,7 +635,7 @@ __device__ __forceinline__ void tile_edge(const StageArgs<Pol>& a, const ScenDev
     jR = sR & 3;
     srcR = sR >> 2;
     Raw<RV> rr;
-    fetch_side<RV>(own, halo, a.in, srcR, rr);
+    fetch_side<RV>(own, halo, far, over, srcR, rr);
     Elem<P, Pol> ER;
     unpack<P>(rr, ER);
     dcRL = acc_sub_r(ER.zb, EL.zb);
@@ -653,7 +649,7 @@ __device__ __forceinline__ void tile_edge(const StageArgs<Pol>& a, const ScenDev
       for (int k = 0; k < NG; ++k) tr[k] = trace_at<P, Pol>(ER, ephi[jR][NG - 1 - k]);  // the same points
     }
   } else if (river_e) {  // river: interior elevation, prescribed normal discharge
-    const int rs = min(-2 - MAXSEG - sR, MAXRIV - 1);
+    const int rs = min(sR - 1 - MAXSEG, MAXRIV - 1);
     qr = river_at<T>(S, rs, t64);
     river = true;
 #pragma unroll
@@ -663,7 +659,7 @@ __device__ __forceinline__ void tile_edge(const StageArgs<Pol>& a, const ScenDev
       tr[k].qy = -qr * ny;
     }
   } else if (ocean_e) {  // ocean: tidal elevation, interior discharge
-    const int seg = min(-2 - sR, MAXSEG - 1);
+    const int seg = sR - 1;
     const T zbc = tide_at<T>(S, seg, t64);
     const T dgh = acc_r(acc_addr(acc_neg(EL.zb), zbc));  // ghost zeta - mean of L
 #pragma unroll
@@ -817,6 +813,265 @@ __device__ __forceinline__ void tile_edge(const StageArgs<Pol>& a, const ScenDev
   }
 }
 
+// ------------------------------------------------------------------------ tile plan ------
+// one warp per tile, once per mesh: ownership of the tile's edges (boundary edges, edges to
+// out-of-tile neighbours and in-tile edges to a higher index belong to a lane's element; the lower
+// element index is the left side) and the order described at EDGE_INLINE
+template <class T>
+__global__ void __launch_bounds__(256) plan_kernel(const int4* nbr, const int4* tile_meta, int ntiles, uint4* plan,
+                                                   int32_t* plan_x) {
+  const int tile = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+  if (tile >= ntiles) return;
+  const int4 meta = tile_meta[tile];
+  const bool valid = lane < meta.y;
+  const int e0 = tile * TILE, e = e0 + lane;
+  const int4 nb = valid ? nbr[e] : make_int4(-1, -1, -1, 0);
+  const int code[3] = {nb.x, nb.y, nb.z};
+  const unsigned lt = (1u << lane) - 1u;
+  uint4* P = plan + (size_t)tile * plan_vec<T>();
+  unsigned* desc = reinterpret_cast<unsigned*>(P);
+  int32_t* halo = reinterpret_cast<int32_t*>(P + EDGE_INLINE / 4);
+  int32_t* over = plan_x + (size_t)tile * PLAN_X;
+  for (int i = lane; i < EDGE_INLINE + HALO; i += 32) desc[i] = 0u;
+  for (int i = lane; i < PLAN_X; i += 32) over[i] = 0;
+  __syncwarp();
+  int base = 0, hbase = 0, ninner = 0;
+#pragma unroll
+  for (int kind = 0; kind < 3; ++kind) {  // in-tile, to another tile, boundary
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      const int c = code[j], n = c >> 2, jn = c & 3, me = (lane << 2) | j;
+      const bool inside = c >= 0 && n >= e0 && n < e0 + TILE;
+      const bool mine = valid && (kind == 0 ? (inside && e < n) : kind == 1 ? (c >= 0 && !inside) : c < 0);
+      const unsigned m = __ballot_sync(0xffffffffu, mine);
+      const int i = base + __popc(m & lt), h = hbase + __popc(m & lt);
+      if (mine) {
+        unsigned d;
+        if (kind == 0) {
+          d = (unsigned)me | (unsigned)(((n - e0) << 2) | jn) << 9;
+        } else if (kind == 1) {
+          const unsigned other = (unsigned)(((32 + h) << 2) | jn);  // sources 32.. : halo, then overflow
+          d = e < n ? ((unsigned)me | other << 9) : (other | (unsigned)me << 9 | ED_OWN_R);
+          if (h < HALO) halo[h] = n;
+          else over[32 + (h - HALO)] = n;
+        } else {
+          d = (unsigned)me | (unsigned)(-1 - c) << 9 | ED_BND;
+        }
+        if (i < EDGE_INLINE) desc[i] = d;
+        else over[i - EDGE_INLINE] = (int32_t)d;
+      }
+      base += __popc(m);
+      if (kind == 1) hbase += __popc(m);
+      if (kind == 0) ninner = base;
+    }
+  }
+  if (sizeof(T) == 4) reinterpret_cast<int32_t*>(P + (EDGE_INLINE + HALO) / 4)[lane] = valid ? nb.w : 0;
+  if (lane == 0)
+    reinterpret_cast<int4*>(P)[plan_vec<T>() - 1] =
+        make_int4(meta.x, meta.y, base | ninner << 8 | min(hbase, HALO) << 16, 0);
+}
+
+// --------------------------------------------------------------------- one tile, one stage ---
+// Phases 1-3 of one tile: the area integrals and rain of each lane's element, every edge of the tile
+// once, then the lift, stage combination and positive-depth operator; O is the element's new record.
+// halo_ready() makes the staged halo records readable; it is called once by the whole warp, before
+// the first round that has an edge to another tile; far(element, record) reads a neighbour beyond the
+// halo slots after that.  The step-initial record comes from shared
+// memory (WNS) or from a.wn.
+template <int P, int FLUX, class Pol, int FT, bool WNS, class HaloReady, class Far>
+__device__ __forceinline__ void tile_body(const StageArgs<Pol>& a, const ScenDev& S, double t64, int rain_kind, int press,
+                                          const RainRec<typename Pol::T>& rr, int tile, int lane, bool valid, int counts,
+                                          const uint4* own, const uint4* halo, const uint4* geoS, const unsigned* planS,
+                                          const float* man, const typename Pol::T* xyS, void* flx, const uint4* wnS,
+                                          const typename Pol::T (*s_ephi)[P + 1][np_of(P)], const float4* s_ephi4,
+                                          HaloReady halo_ready, Far far, Elem<P, Pol>& O, typename Pol::Acc& rain_acc,
+                                          typename Pol::Acc& bdry_acc) {
+  using T = typename Pol::T;
+  using Acc = typename Pol::Acc;
+  using L = TileLayout<P, Pol, FT>;
+  constexpr int NP = np_of(P), NS = NP - 1, NG = P + 1, RV = L::RV, GV = L::GV, NPR = L::NPR, NV = L::NV;
+  const RefTab<T>& tab = ctab<T, P>();
+  const int e = tile * TILE + lane;
+  const T t = (T)t64;
+  const int nedge = counts & 255, ninner = (counts >> 8) & 255;
+  const int32_t* over = a.plan_x + (size_t)tile * PLAN_X;
+
+  // ---- element phase A: area integrals and rain, while the halo copies are in flight
+  T Rz[NP], Rx[NP], Ry[NP];
+  T Re = 0;
+  if (valid) {
+    Geo<Pol> G;
+    geo_from(geoS + lane * GV, man + lane, G);
+    // gridded rain: the element's two records now, blended after the area integrals; without
+    // records the node indices now, their nodal rates then
+    T re0 = T(0), re1 = T(0);
+    int4 nd = make_int4(0, 0, 0, 0);
+    if (rain_kind == 3) {
+      if (rr.r0) {
+        re0 = __ldg(rr.r0 + e);
+        re1 = __ldg(rr.r1 + e);
+      } else {
+        nd = __ldg(a.nodes + e);
+      }
+    }
+    Elem<P, Pol> E;
+    {
+      Raw<RV> r;
+#pragma unroll
+      for (int v = 0; v < RV; ++v) r.v[v] = own[v * TILE + lane];
+      unpack<P>(r, E);
+    }
+    // vertex coordinates: the first vertex, then along the edge vectors t_j = (-ln_j.y, ln_j.x)
+    T vx[3] = {0, 0, 0}, vy[3] = {0, 0, 0};
+    if (press || rain_kind == 2) {
+      const T* x0 = xyS + 2 * lane;
+      vx[0] = x0[0];
+      vy[0] = x0[1];
+      vx[1] = vx[0] - G.lny[0];
+      vy[1] = vy[0] + G.lnx[0];
+      vx[2] = vx[0] + G.lny[2];
+      vy[2] = vy[0] - G.lnx[2];
+    }
+    tile_area<P, Pol, FT>(E, G, S, a, press, vx, vy, Rz, Rx, Ry);
+    // forcing: element rain = mean of the three nodal rates (Eq. rain)
+    if (rain_kind == 1) {
+      Re = a.rain_e[e];
+    } else if (rain_kind == 2) {  // radial storm profile at the three vertices
+      const ForcingT<T>& F = forcing<T>(S);
+      const T tt = t - F.storm[7];
+      const T cx = F.storm[0] + F.storm[2] * tt, cy = F.storm[1] + F.storm[3] * tt;
+      const T rp = F.storm[4], rm = F.storm[5], re = F.storm[6];
+      T acc = 0;
+#pragma unroll
+      for (int i = 0; i < 3; ++i) {
+        const T dx = vx[i] - cx, dy = vy[i] - cy;
+        const T r = fsqrt0(dx * dx + dy * dy);
+        if constexpr (sizeof(T) == 4)  // with 1 / rm and log2(e) / re formed once on the host
+          acc += (r < rm) ? rp * fmaf(0.5f * F.storm[8], r, 0.5f) : rp * mufu_ex2((rm - r) * F.storm[9]);
+        else
+          acc += (r < rm) ? rp * (T(0.5) + T(0.5) * fdiv(r, rm)) : rp * fexp(-fdiv(r - rm, re));
+      }
+      Re = acc * T(1.0 / 3.0);
+    } else if (rain_kind == 3 && rr.r0) {
+      Re = rain_blend<T>(re0, re1, rr.f);
+    } else if (rain_kind == 3) {  // nodal rates interpolated by the node kernel of this stage
+      Re = (a.rain_node[nd.x] + a.rain_node[nd.y] + a.rain_node[nd.z]) * T(1.0 / 3.0);
+    }
+  }
+
+  // ---- edge phase: each edge touching the tile once, one per lane and round; the halo records are
+  // waited for before the first round that has an edge to another tile
+  bool staged = false;
+  for (int r = 0; r * 32 < nedge; ++r) {
+    if (!staged && r * 32 + 32 > ninner) {
+      halo_ready();
+      staged = true;
+    }
+    const int i = r * 32 + lane;
+    if (i < nedge) {
+      const unsigned ed = i < EDGE_INLINE ? planS[i] : (unsigned)__ldg(over + (i - EDGE_INLINE));
+      tile_edge<P, FLUX, Pol, FT>(a, S, own, halo, geoS, far, over, flx, ed, s_ephi, s_ephi4, t64, bdry_acc);
+    }
+  }
+  if (!staged) halo_ready();
+  __syncwarp();
+
+  // ---- element phase B: lift, inverse mass, stage combination, positive-depth operator
+  if (valid) {
+    Geo<Pol> G;
+    geo_from(geoS + lane * GV, man + lane, G);
+    Elem<P, Pol> E;
+    {
+      Raw<RV> r;
+#pragma unroll
+      for (int v = 0; v < RV; ++v) r.v[v] = own[v * TILE + lane];
+      unpack<P>(r, E);
+    }
+    Acc massout;  // edge mass outflow (volume per second), summed exactly over the three sides
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      T vals[NV + 1];
+      load_side<T, NPR, NV>(flx, lane, j, vals);
+#pragma unroll
+      for (int k = 0; k < NG; ++k) {
+#pragma unroll
+        for (int m = 0; m < NP; ++m) {
+          const T ph_ = tab.ephi[j][k][m];
+          if (m > 0) Rz[m] = fma(-ph_, vals[k], Rz[m]);
+          Rx[m] = fma(-ph_, vals[NG + k], Rx[m]);
+          Ry[m] = fma(-ph_, vals[2 * NG + k], Ry[m]);
+        }
+      }
+      const T ms = side_mass<T, NG, L::MASSV>(vals);
+      massout = (j == 0) ? acc_make<Acc>(ms, T(0), ms) : acc_addr(massout, ms);
+    }
+    if (E.flags & FLAG_DRY) {  // the momentum equations are not advanced on dry elements
+#pragma unroll
+      for (int m = 0; m < NP; ++m) Rx[m] = Ry[m] = 0;
+    }
+    // Shu-Osher combination: out = a_n w^n + a_in w^in + beta dt M^{-1} R
+    const T idetJ = T(2) * acc_r(G.invA);
+    const Acc an = acc_make<Acc>(a.a_n_hi, a.a_n_lo, a.a_n);
+    const Acc ain = acc_make<Acc>(a.a_in_hi, a.a_in_lo, a.a_in);
+    const Acc bdt = acc_make<Acc>(S.bdt_hi[a.stage], S.bdt_lo[a.stage], S.bdt[a.stage]);
+    // mean rates: d(zeta_bar)/dt = R_e - massout / A;  d(q_bar)/dt = phi_0 R_0 / detJ
+    const Acc zrate = acc_addr(acc_neg(acc_mul(massout, G.invA)), Re);
+    const T xrate = tab.phi0 * Rx[0] * idetJ, yrate = tab.phi0 * Ry[0] * idetJ;
+    O = E;
+    Elem<P, Pol> Wn = E;
+    if (a.has_n) {
+      Raw<RV> rn;
+#pragma unroll
+      for (int v = 0; v < RV; ++v) rn.v[v] = WNS ? wnS[v * TILE + lane] : __ldg(a.wn + rec_at<RV>(e, v));
+      unpack<P>(rn, Wn);
+    }
+    const T an_r = (sizeof(T) == 4) ? (T)a.a_n_hi : (T)a.a_n, ain_r = (sizeof(T) == 4) ? (T)a.a_in_hi : (T)a.a_in;
+    {
+      Acc z, x, y;
+      constexpr int PW = ft_pow2(FT);
+      if (sizeof(T) == 4 && (PW == 1 || (PW == -1 && a.pow2))) {  // exact scaling of both words by a power of two
+        z = acc_scale2(E.zb, ain_r);
+        x = acc_scale2(E.xb, ain_r);
+        y = acc_scale2(E.yb, ain_r);
+        if (a.has_n) {
+          z = acc_addf(z, acc_scale2(Wn.zb, an_r));
+          x = acc_addf(x, acc_scale2(Wn.xb, an_r));
+          y = acc_addf(y, acc_scale2(Wn.yb, an_r));
+        }
+      } else {
+        z = acc_mul(ain, E.zb);
+        x = acc_mul(ain, E.xb);
+        y = acc_mul(ain, E.yb);
+        if (a.has_n) {
+          z = acc_add(z, acc_mul(an, Wn.zb));
+          x = acc_add(x, acc_mul(an, Wn.xb));
+          y = acc_add(y, acc_mul(an, Wn.yb));
+        }
+      }
+      O.zb = acc_addf(z, acc_mul(bdt, zrate));
+      O.xb = acc_addr(x, acc_r(bdt) * xrate);
+      O.yb = acc_addr(y, acc_r(bdt) * yrate);
+    }
+    const T bdt_r = acc_r(bdt);
+#pragma unroll
+    for (int m = 0; m < NS; ++m) {
+      T z = ain_r * E.zs[m] + bdt_r * (Rz[m + 1] * idetJ);
+      T x = ain_r * E.xs[m] + bdt_r * (Rx[m + 1] * idetJ);
+      T y = ain_r * E.ys[m] + bdt_r * (Ry[m + 1] * idetJ);
+      if (a.has_n) {
+        z = fma(an_r, Wn.zs[m], z);
+        x = fma(an_r, Wn.xs[m], x);
+        y = fma(an_r, Wn.ys[m], y);
+      }
+      O.zs[m] = z;
+      O.xs[m] = x;
+      O.ys[m] = y;
+    }
+    apply_positivity<P, Pol>(O, G, e, a, &a.ctl->err);
+    rain_acc = acc_addf(rain_acc, acc_mulr(G.A, Re));
+  }
+}
+
 // -------------------------------------------------------------------------- the kernel ---
 #ifndef DG_TILE_MAXNREG
 // register budget: mixed p = 1 at 128 (16 warps per SM, as its shared memory allows); elsewhere
@@ -830,8 +1085,8 @@ template <int P, int FLUX, class Pol, int FT = FT_ALL>
 __global__ void DG_TILE_BOUNDS tile_kernel(const StageArgs<Pol> a) {
   using T = typename Pol::T;
   using Acc = typename Pol::Acc;
-  using L = TileLayout<P, Pol>;
-  constexpr int NP = np_of(P), NS = NP - 1, NG = P + 1, RV = L::RV, GV = L::GV, NPR = L::NPR, NV = L::NV;
+  using L = TileLayout<P, Pol, FT>;
+  constexpr int NP = np_of(P), NG = P + 1, RV = L::RV, GV = L::GV;
   const RefTab<T>& tab = ctab<T, P>();
 
   // edge basis values, read at edge-dependent indices; at p = 1 in FP32 also one 16-byte row per
@@ -851,7 +1106,7 @@ __global__ void DG_TILE_BOUNDS tile_kernel(const StageArgs<Pol> a) {
   const int lane = tid & 31;
   uint4* Wm = tsm + (size_t)(tid >> 5) * L::VEC;
   uint4* halo = Wm + L::HAL;                                       // [HALO][RV]
-  EdgeDesc<T>* desc = reinterpret_cast<EdgeDesc<T>*>(Wm + L::DESC);  // [96]
+  void* flx = Wm + L::FLX;                                         // [3][NPR][32] pairs
   const uint32_t bar0 = smem_u32(Wm + L::BAR), bar1 = bar0 + 8;
   if (lane == 0) {
     mbar_init(bar0, 1);
@@ -859,21 +1114,19 @@ __global__ void DG_TILE_BOUNDS tile_kernel(const StageArgs<Pol> a) {
     mbar_fence_init();
   }
   __syncwarp();
-  const unsigned lt = (1u << lane) - 1u;
   const int gw = blockIdx.x * (blockDim.x >> 5) + (tid >> 5);
   const int W = gridDim.x * (blockDim.x >> 5);
-  // one TMA batch: the tile's records, geometry and neighbour codes into a buffer (lane 0)
+  // one TMA batch: the tile's records, geometry, plan and first vertices into a buffer (lane 0)
   auto issue = [&](int t, int b) {
     if (lane == 0) {
-      uint4* buf = Wm + (b ? L::BUF1 : L::BUF0);
+      uint4* buf = Wm + (b ? L::BUF : 0);
       const uint32_t bar = b ? bar1 : bar0;
       fence_proxy_async();
       mbar_expect_tx(bar, L::TILE_BYTES);
       bulk_g2s(smem_u32(buf), a.in + (size_t)t * TILE * RV, 16u * TILE * RV, bar);
       bulk_g2s(smem_u32(buf + L::O_GEO), a.geo + (size_t)t * TILE * GV, 16u * TILE * GV, bar);
-      bulk_g2s(smem_u32(buf + L::O_NBR), a.nbr + (size_t)t * TILE, 16u * TILE, bar);
-      bulk_g2s(smem_u32(buf + L::O_XY), a.xy0 + (size_t)t * L::XV, 16u * L::XV, bar);
-      bulk_g2s(smem_u32(buf + L::O_META), a.tile_meta + t, 16u, bar);
+      bulk_g2s(smem_u32(buf + L::O_PLAN), a.plan + (size_t)t * L::PV, 16u * L::PV, bar);
+      if constexpr (L::XV > 0) bulk_g2s(smem_u32(buf + L::O_XY), a.xy0 + (size_t)t * L::XV, 16u * L::XV, bar);
     }
   };
   const double stepd = (double)a.ctl->step + a.cst;
@@ -896,11 +1149,10 @@ __global__ void DG_TILE_BOUNDS tile_kernel(const StageArgs<Pol> a) {
       return;
     }
     ph ^= 1u << b;
-    uint4* const buf = Wm + (b ? L::BUF1 : L::BUF0);
+    uint4* const buf = Wm + (b ? L::BUF : 0);
     const uint4* own = buf;                           // [RV][32] records
     const uint4* geoS = own + L::O_GEO;               // [32][GV]
-    void* flx = buf + L::O_FLX;                       // [3][NPR][32] pairs, over geoS .. meta
-    const int4* nbrS = reinterpret_cast<const int4*>(own + L::O_NBR);
+    const unsigned* planS = reinterpret_cast<const unsigned*>(own + L::O_PLAN);
     const int4 meta = reinterpret_cast<const int4*>(own + L::O_META)[0];
     const int sc = meta.x, present = meta.y;
     if (present == 0) {  // padding tile: no element (uniform over the warp)
@@ -926,243 +1178,33 @@ __global__ void DG_TILE_BOUNDS tile_kernel(const StageArgs<Pol> a) {
     const ScenDev& S = *Sp;
     const int e0 = tile * TILE, e = e0 + lane;
     const bool valid = lane < present;
-    const T t = (T)t64;
     if (a.has_n && lane == 0) bulk_prefetch_l2(a.wn + (size_t)e0 * RV, 16u * TILE * RV);  // read in phase B
 
-    // ---- edge ownership: boundary edges, edges to out-of-tile neighbours, and in-tile edges to a
-    // higher index belong to this lane; out-of-tile neighbours get a halo slot.  Edge slots: the
-    // interior edges first, then the boundary edges (fewer divergent rounds).
-    const int4 nb = valid ? nbrS[lane] : make_int4(-1, -1, -1, -1);
-    const int code[3] = {nb.x, nb.y, nb.z};
-    bool own_e[3], out[3];
-    int eidx[3], hslot[3];
-    unsigned bi[3], bb[3];
-    int nint = 0, hbase = 0;
+    // ---- the out-of-tile neighbours' records, one halo slot per lane, by the tile's plan
+    if (lane < (meta.z >> 16)) {
+      const int n = reinterpret_cast<const int32_t*>(own + L::O_HALO)[lane];
 #pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      const int c = code[j];
-      const int n = c >> 2;
-      const bool inside = c >= 0 && n >= e0 && n < e0 + TILE;
-      own_e[j] = valid && (c < 0 || !inside || e < n);
-      out[j] = valid && c >= 0 && !inside;
-      bi[j] = __ballot_sync(0xffffffffu, own_e[j] && c >= 0);
-      bb[j] = __ballot_sync(0xffffffffu, own_e[j] && c < 0);
-      const unsigned bh = __ballot_sync(0xffffffffu, out[j]);
-      hslot[j] = hbase + __popc(bh & lt);
-      hbase += __popc(bh);
-      nint += __popc(bi[j]);
+      for (int v = 0; v < RV; ++v) cp_async16(halo + v * HALO + lane, a.in + rec_at<RV>(n, v));
     }
-    {
-      int ib = 0, bbase = nint;
-#pragma unroll
-      for (int j = 0; j < 3; ++j) {
-        eidx[j] = code[j] >= 0 ? ib + __popc(bi[j] & lt) : bbase + __popc(bb[j] & lt);
-        ib += __popc(bi[j]);
-        bbase += __popc(bb[j]);
-      }
-    }
-    const int nedge = nint + __popc(bb[0]) + __popc(bb[1]) + __popc(bb[2]);
-#pragma unroll
-    for (int j = 0; j < 3; ++j)
-      if (out[j] && hslot[j] < HALO) {
-#pragma unroll
-        for (int v = 0; v < RV; ++v) cp_async16(halo + v * HALO + hslot[j], a.in + rec_at<RV>(code[j] >> 2, v));
-      }
     cp_async_commit();
-    Geo<Pol> G;
-    if (valid) geo_from(geoS + lane * GV, nb, G);
-    // edge descriptors {left side, right side or boundary code}
-#pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      if (!own_e[j]) continue;
-      const int c = code[j];
-      const int me = (lane << 2) | j;
-      int sL = me, sR = c;
-      T lnx = G.lnx[j], lny = G.lny[j];
-      if (c >= 0) {
-        const int n = c >> 2, jn = c & 3;
-        if (!out[j]) {
-          sR = ((n - e0) << 2) | jn;
-        } else {
-          const int other = (((hslot[j] < HALO) ? (32 + hslot[j]) : (64 + n)) << 2) | jn;
-          if (e < n) {
-            sR = other;
-          } else {  // the neighbour has the lower index: it is the left side
-            sL = other;
-            sR = me;
-            lnx = -lnx;
-            lny = -lny;
-          }
-        }
-      }
-      put_desc(desc, eidx[j], sL, sR, lnx, lny);
-    }
 
-    // ---- element phase A: area integrals and rain, while the halo copies are in flight
-    T Rz[NP], Rx[NP], Ry[NP];
-    T Re = 0;
+    Elem<P, Pol> O;
+    tile_body<P, FLUX, Pol, FT, false>(a, S, t64, rain_kind, press, rr, tile, lane, valid, meta.z, own, halo, geoS, planS,
+                                       reinterpret_cast<const float*>(own + L::O_MAN),
+                                       reinterpret_cast<const T*>(own + L::O_XY), flx, nullptr, s_ephi, s_ephi4,
+                                       [] {
+                                         cp_async_wait_all();
+                                         __syncwarp();
+                                       },
+                                       [&](int n, Raw<RV>& r) {
+#pragma unroll
+                                         for (int v = 0; v < RV; ++v) r.v[v] = __ldg(a.in + rec_at<RV>(n, v));
+                                       },
+                                       O, rain_acc, bdry_acc);
     if (valid) {
-      // gridded rain: the element's two records now, blended after the area integrals; without
-      // records the node indices now, their nodal rates then
-      T re0 = T(0), re1 = T(0);
-      int4 nd = make_int4(0, 0, 0, 0);
-      if (rain_kind == 3) {
-        if (rr.r0) {
-          re0 = __ldg(rr.r0 + e);
-          re1 = __ldg(rr.r1 + e);
-        } else {
-          nd = __ldg(a.nodes + e);
-        }
-      }
-      Elem<P, Pol> E;
-      {
-        Raw<RV> r;
-#pragma unroll
-        for (int v = 0; v < RV; ++v) r.v[v] = own[v * TILE + lane];
-        unpack<P>(r, E);
-      }
-      // vertex coordinates: the first vertex, then along the edge vectors t_j = (-ln_j.y, ln_j.x)
-      T vx[3] = {0, 0, 0}, vy[3] = {0, 0, 0};
-      if (press || rain_kind == 2) {
-        const T* x0 = reinterpret_cast<const T*>(own + L::O_XY) + 2 * lane;
-        vx[0] = x0[0];
-        vy[0] = x0[1];
-        vx[1] = vx[0] - G.lny[0];
-        vy[1] = vy[0] + G.lnx[0];
-        vx[2] = vx[0] + G.lny[2];
-        vy[2] = vy[0] - G.lnx[2];
-      }
-      tile_area<P, Pol, FT>(E, G, S, a, press, vx, vy, Rz, Rx, Ry);
-      // forcing: element rain = mean of the three nodal rates (Eq. rain)
-      if (rain_kind == 1) {
-        Re = a.rain_e[e];
-      } else if (rain_kind == 2) {  // radial storm profile at the three vertices
-        const ForcingT<T>& F = forcing<T>(S);
-        const T tt = t - F.storm[7];
-        const T cx = F.storm[0] + F.storm[2] * tt, cy = F.storm[1] + F.storm[3] * tt;
-        const T rp = F.storm[4], rm = F.storm[5], re = F.storm[6];
-        T acc = 0;
-#pragma unroll
-        for (int i = 0; i < 3; ++i) {
-          const T dx = vx[i] - cx, dy = vy[i] - cy;
-          const T r = fsqrt0(dx * dx + dy * dy);
-          if constexpr (sizeof(T) == 4)  // with 1 / rm and log2(e) / re formed once on the host
-            acc += (r < rm) ? rp * fmaf(0.5f * F.storm[8], r, 0.5f) : rp * mufu_ex2((rm - r) * F.storm[9]);
-          else
-            acc += (r < rm) ? rp * (T(0.5) + T(0.5) * fdiv(r, rm)) : rp * fexp(-fdiv(r - rm, re));
-        }
-        Re = acc * T(1.0 / 3.0);
-      } else if (rain_kind == 3 && rr.r0) {
-        Re = rain_blend<T>(re0, re1, rr.f);
-      } else if (rain_kind == 3) {  // nodal rates interpolated by the node kernel of this stage
-        Re = (a.rain_node[nd.x] + a.rain_node[nd.y] + a.rain_node[nd.z]) * T(1.0 / 3.0);
-      }
-    }
-    cp_async_wait_all();
-    __syncwarp();
-
-    // ---- edge phase: each edge touching the tile once, one per lane and round
-    for (int r = 0; r * 32 < nedge; ++r) {
-      const int i = r * 32 + lane;
-      if (i < nedge) tile_edge<P, FLUX, Pol, FT>(a, S, own, halo, desc, flx, i, s_ephi, s_ephi4, t64, bdry_acc);
-    }
-    fence_proxy_async();  // the slots' generic writes before the TMA batch that later refills the buffer
-    __syncwarp();
-
-    // ---- element phase B: lift, inverse mass, stage combination, positive-depth operator
-    if (valid) {
-      Elem<P, Pol> E;
-      {
-        Raw<RV> r;
-#pragma unroll
-        for (int v = 0; v < RV; ++v) r.v[v] = own[v * TILE + lane];
-        unpack<P>(r, E);
-      }
-      Acc massout;  // edge mass outflow (volume per second), summed exactly over the three sides
-#pragma unroll
-      for (int j = 0; j < 3; ++j) {
-        T vals[NV + 1];
-        load_side<T, NPR, NV>(flx, lane, j, vals);
-#pragma unroll
-        for (int k = 0; k < NG; ++k) {
-#pragma unroll
-          for (int m = 0; m < NP; ++m) {
-            const T ph_ = tab.ephi[j][k][m];
-            if (m > 0) Rz[m] = fma(-ph_, vals[k], Rz[m]);
-            Rx[m] = fma(-ph_, vals[NG + k], Rx[m]);
-            Ry[m] = fma(-ph_, vals[2 * NG + k], Ry[m]);
-          }
-        }
-        const T ms = side_mass<T, NG, L::MASSV>(vals);
-        massout = (j == 0) ? acc_make<Acc>(ms, T(0), ms) : acc_addr(massout, ms);
-      }
-      if (E.flags & FLAG_DRY) {  // the momentum equations are not advanced on dry elements
-#pragma unroll
-        for (int m = 0; m < NP; ++m) Rx[m] = Ry[m] = 0;
-      }
-      // Shu-Osher combination: out = a_n w^n + a_in w^in + beta dt M^{-1} R
-      const T idetJ = T(2) * acc_r(G.invA);
-      const Acc an = acc_make<Acc>(a.a_n_hi, a.a_n_lo, a.a_n);
-      const Acc ain = acc_make<Acc>(a.a_in_hi, a.a_in_lo, a.a_in);
-      const Acc bdt = acc_make<Acc>(S.bdt_hi[a.stage], S.bdt_lo[a.stage], S.bdt[a.stage]);
-      // mean rates: d(zeta_bar)/dt = R_e - massout / A;  d(q_bar)/dt = phi_0 R_0 / detJ
-      const Acc zrate = acc_addr(acc_neg(acc_mul(massout, G.invA)), Re);
-      const T xrate = tab.phi0 * Rx[0] * idetJ, yrate = tab.phi0 * Ry[0] * idetJ;
-      Elem<P, Pol> O = E;
-      Elem<P, Pol> Wn = E;
-      if (a.has_n) {
-        Raw<RV> rn;
-#pragma unroll
-        for (int v = 0; v < RV; ++v) rn.v[v] = __ldg(a.wn + rec_at<RV>(e, v));
-        unpack<P>(rn, Wn);
-      }
-      const T an_r = (sizeof(T) == 4) ? (T)a.a_n_hi : (T)a.a_n, ain_r = (sizeof(T) == 4) ? (T)a.a_in_hi : (T)a.a_in;
-      {
-        Acc z, x, y;
-        constexpr int PW = ft_pow2(FT);
-        if (sizeof(T) == 4 && (PW == 1 || (PW == -1 && a.pow2))) {  // exact scaling of both words by a power of two
-          z = acc_scale2(E.zb, ain_r);
-          x = acc_scale2(E.xb, ain_r);
-          y = acc_scale2(E.yb, ain_r);
-          if (a.has_n) {
-            z = acc_addf(z, acc_scale2(Wn.zb, an_r));
-            x = acc_addf(x, acc_scale2(Wn.xb, an_r));
-            y = acc_addf(y, acc_scale2(Wn.yb, an_r));
-          }
-        } else {
-          z = acc_mul(ain, E.zb);
-          x = acc_mul(ain, E.xb);
-          y = acc_mul(ain, E.yb);
-          if (a.has_n) {
-            z = acc_add(z, acc_mul(an, Wn.zb));
-            x = acc_add(x, acc_mul(an, Wn.xb));
-            y = acc_add(y, acc_mul(an, Wn.yb));
-          }
-        }
-        O.zb = acc_addf(z, acc_mul(bdt, zrate));
-        O.xb = acc_addr(x, acc_r(bdt) * xrate);
-        O.yb = acc_addr(y, acc_r(bdt) * yrate);
-      }
-      const T bdt_r = acc_r(bdt);
-#pragma unroll
-      for (int m = 0; m < NS; ++m) {
-        T z = ain_r * E.zs[m] + bdt_r * (Rz[m + 1] * idetJ);
-        T x = ain_r * E.xs[m] + bdt_r * (Rx[m + 1] * idetJ);
-        T y = ain_r * E.ys[m] + bdt_r * (Ry[m + 1] * idetJ);
-        if (a.has_n) {
-          z = fma(an_r, Wn.zs[m], z);
-          x = fma(an_r, Wn.xs[m], x);
-          y = fma(an_r, Wn.ys[m], y);
-        }
-        O.zs[m] = z;
-        O.xs[m] = x;
-        O.ys[m] = y;
-      }
-      apply_positivity<P, Pol>(O, G, e, a, &a.ctl->err);
       Raw<RV> ro;
       pack<P>(O, ro);
       store_raw<RV>(a.out, e, ro);
-      rain_acc = acc_addf(rain_acc, acc_mulr(G.A, Re));
     }
     __syncwarp();  // this tile's shared data is consumed: its buffers may be refilled
   }

@@ -34,6 +34,16 @@ inline int tile_try_spec_occ<Mixed>(int p, int flux, int feat, int block) {
 
 #define DG_DEFINE_TILE_LAUNCHERS(POL)                                                                        \
   template <>                                                                                                \
+  cudaError_t launch_plan<POL>(const int4* nbr, const int4* meta, int ntiles, uint4* plan, int32_t* px, cudaStream_t s) { \
+    plan_kernel<POL::T><<<(ntiles + 7) / 8, 256, 0, s>>>(nbr, meta, ntiles, plan, px);                       \
+    return cudaGetLastError();                                                                               \
+  }                                                                                                          \
+  template <>                                                                                                \
+  void plan_bytes<POL>(int ntiles, size_t& plan, size_t& px) {                                               \
+    plan = 16 * (size_t)plan_vec<POL::T>() * ntiles;                                                         \
+    px = 4 * (size_t)PLAN_X * ntiles;                                                                        \
+  }                                                                                                          \
+  template <>                                                                                                \
   cudaError_t upload_tile_tables<POL>(int p, const RefTab<float>& tf, const RefTab<double>& td) {            \
     cudaError_t e = cudaMemcpyToSymbol(c_tab_f, &tf, sizeof(RefTab<float>), p * sizeof(RefTab<float>));     \
     if (e != cudaSuccess) return e;                                                                          \

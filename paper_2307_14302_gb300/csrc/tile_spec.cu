@@ -12,25 +12,21 @@
 namespace dg {
 namespace {
 
-// tidal boundary, parametric storm rain, Manning friction, SSP(2,2)
-constexpr int FT_TIDE_STORM = FT_OCEAN | FT_RAIN2 | FT_MANNING | FT_POW2;
-// tidal boundary, gridded rain, Manning friction, SSP(2,2)
-constexpr int FT_TIDE_GRID = FT_OCEAN | FT_RAIN3 | FT_MANNING | FT_POW2;
-// walls only, constant nodal rain, Manning friction, SSP(2,2)
-constexpr int FT_WALL_NODAL = FT_RAIN1 | FT_MANNING | FT_POW2;
-// tidal boundary, parametric storm rain, pressure set-up, Manning friction, SSP(3,3) (p = 2)
-constexpr int FT_TIDE_STORM_SETUP = FT_OCEAN | FT_RAIN2 | FT_PRESS | FT_MANNING | FT_POW2 | FT_GENSSP;
-
 using Kernel = void (*)(const StageArgs<Mixed>);
 struct Spec {
   int p, flux, ft;
   Kernel k;
+  int smem;  // dynamic shared memory per warp
 };
+template <int P, int FLUX, int FT>
+constexpr Spec spec() {
+  return {P, FLUX, FT, tile_kernel<P, FLUX, Mixed, FT>, tile_smem_bytes<P, Mixed, FT>(32)};
+}
 const Spec kSpecs[] = {
-    {1, 0, FT_WALL_NODAL, tile_kernel<1, 0, Mixed, FT_WALL_NODAL>},
-    {1, 0, FT_TIDE_STORM, tile_kernel<1, 0, Mixed, FT_TIDE_STORM>},
-    {1, 0, FT_TIDE_GRID, tile_kernel<1, 0, Mixed, FT_TIDE_GRID>},
-    {2, 0, FT_TIDE_STORM_SETUP, tile_kernel<2, 0, Mixed, FT_TIDE_STORM_SETUP>},
+    spec<1, 0, FT_WALL_NODAL>(),
+    spec<1, 0, FT_TIDE_STORM>(),
+    spec<1, 0, FT_TIDE_GRID>(),
+    spec<2, 0, FT_TIDE_STORM_SETUP>(),
 };
 
 int bits(int x) {
@@ -46,7 +42,7 @@ const Spec* find_spec(int p, int flux, int feat) {
       best = &sp;
   return best;
 }
-int smem_bytes(int p, int block) { return p == 1 ? tile_smem_bytes<1, Mixed>(block) : tile_smem_bytes<2, Mixed>(block); }
+int smem_bytes(const Spec& sp, int block) { return sp.smem * (block / 32); }
 
 }  // namespace
 
@@ -54,7 +50,7 @@ cudaError_t launch_tile_spec(int p, int flux, int feat, const StageArgs<Mixed>& 
                              cudaStream_t s) {
   const Spec* sp = find_spec(p, flux, feat);
   if (!sp) return cudaErrorNotSupported;
-  sp->k<<<grid, block, smem_bytes(p, block), s>>>(a);
+  sp->k<<<grid, block, smem_bytes(*sp, block), s>>>(a);
   return cudaGetLastError();
 }
 
@@ -67,7 +63,7 @@ int tile_spec_blocks_per_sm(int p, int flux, int feat, int block) {
   const Spec* sp = find_spec(p, flux, feat);
   if (!sp) return -1;
   int n = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, sp->k, block, smem_bytes(p, block)) != cudaSuccess) {
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, sp->k, block, smem_bytes(*sp, block)) != cudaSuccess) {
     cudaGetLastError();
     return 0;
   }
@@ -83,7 +79,7 @@ cudaError_t upload_tile_spec_tables(int p, const RefTab<float>& tf, const RefTab
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess) return e;
   for (const Spec& sp : kSpecs)
-    if ((e = tile_smem_limit(sp.k, optin, smem_bytes(sp.p, 256))) != cudaSuccess) return e;
+    if ((e = tile_smem_limit(sp.k, optin, smem_bytes(sp, 256))) != cudaSuccess) return e;
   return cudaSuccess;
 }
 
