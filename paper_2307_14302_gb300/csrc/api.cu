@@ -139,6 +139,8 @@ struct dgswe_ctx {
   // launch configuration
   int block = 128, waves = 1, split = 1;
   bool autotune = true;
+  bool small = false;        // small mesh: whole steps in one cluster launch (steps.cuh) ...
+  int s_ctas = 0, s_wpc = 0; // ... of s_ctas CTAs with one warp for each of s_wpc tiles
   bool graphs = true;  // replay steps from CUDA graphs (else direct launches)
   bool grid_rain = false;  // gridded rain without element records: a node kernel runs before each stage
   int feat = FT_ALL;       // features of the run (Feature bits): selects the tile-kernel instantiation
@@ -310,6 +312,8 @@ static int upload_all_tables(int p) {
   CU(upload_tile_tables<Mixed>(p, g_tabf[p], g_tabd[p]));
   CU(upload_tile_spec_tables(p, g_tabf[p], g_tabd[p]));
   CU(upload_tile_tables<Fp64>(p, g_tabf[p], g_tabd[p]));
+  CU(upload_steps_tables<Mixed>(p, g_tabf[p], g_tabd[p]));
+  CU(upload_steps_tables<Fp64>(p, g_tabf[p], g_tabd[p]));
   return 0;
 }
 
@@ -859,9 +863,67 @@ static int apply_launch(dgswe_h h, int block, int waves, int split) {
   return 0;
 }
 
+// Small meshes: whole steps in one launch of one cluster (steps.cuh), when every tile can have a warp
+// in it and no other kernel runs between the stages.
+// At least four warps per CTA (one per SM sub-partition; fewer CTAs make the barrier cheaper), more
+// when 16 CTAs would not hold the mesh.
+static bool plan_small(dgswe_h h) {
+  const int nrec = h->stages.size() > 2 ? 3 : 2;
+  if (h->prm.limiter || h->grid_rain) return false;
+  int live = h->ntiles;  // the last tiles of the last scenario may be padding
+  while (live > 1 && (long long)(live - 1) * TILE >= h->eoff.back() + h->sc.back().m.ne) --live;
+  for (int ctas = 16; ctas >= 8; ctas -= 8) {
+    const int wpc = std::max(4, (live + ctas - 1) / ctas), use = (live + wpc - 1) / wpc;
+    if (wpc > 16) continue;
+    const bool ok = mixed(h) ? steps_fit<Mixed>(h->prm.p, h->prm.flux, h->feat, use, wpc, nrec)
+                             : steps_fit<Fp64>(h->prm.p, h->prm.flux, h->feat, use, wpc, nrec);
+    if (ok) {
+      h->s_ctas = use;
+      h->s_wpc = wpc;
+      return true;
+    }
+  }
+  return false;
+}
+
+template <class Pol>
+static cudaError_t enqueue_small(dgswe_h h, int n) {
+  StepsArgs st;
+  std::memset(&st, 0, sizeof st);
+  const int S = (int)h->stages.size();
+  for (int s = 0; s < S; ++s) {
+    const StageArgs<Pol> a = make_args<Pol>(h, s, 0);
+    StepsArgs::Stage& c = st.st[s];
+    c.in = s == 0 ? 0 : 1 + (s - 1) % 2;
+    c.out = s == S - 1 ? 0 : 1 + s % 2;
+    c.has_n = a.has_n;
+    c.pow2 = a.pow2;
+    c.a_n_hi = a.a_n_hi;
+    c.a_n_lo = a.a_n_lo;
+    c.a_in_hi = a.a_in_hi;
+    c.a_in_lo = a.a_in_lo;
+    c.a_n = a.a_n;
+    c.a_in = a.a_in;
+    c.cst = a.cst;
+    c.bw = h->stages[s].bw;
+    split_ff(c.bw, c.bw_hi, c.bw_lo);
+  }
+  st.nstage = S;
+  st.nsteps = n;
+  st.nrec = S > 2 ? 3 : 2;
+  return launch_steps<Pol>(h->prm.p, h->prm.flux, h->feat, make_args<Pol>(h, S - 1, 0), st, h->s_ctas, h->s_wpc, h->stream);
+}
+
 // time whole steps (every stage; timing runs write only the two scratch records) for each form
 // (fused, edge kernel + element kernel, tile), block size and number of waves
 static int autotune(dgswe_h h) {
+  h->small = plan_small(h);
+  if (h->small) {  // no timing: the tile form, for what is launched stage by stage (dgswe_set_graphs 0)
+    h->autotune = false;
+    if (int rc = apply_launch(h, 64, 1, 2)) return rc;
+    h->wcur = std::max(h->wcur, h->s_ctas * h->s_wpc);
+    return 0;
+  }
   cudaEvent_t e0, e1;
   CU(cudaEventCreate(&e0));
   CU(cudaEventCreate(&e1));
@@ -977,6 +1039,10 @@ static int prepare(dgswe_h h) {
     if (int rc = reduce_volume(h, s, h->V0[s], h->VH0[s])) return rc;
   }
   if (int rc = upload_dt(h)) return rc;
+  if (h->small) {  // the mesh may have changed: decide again at the next step
+    h->small = false;
+    h->autotune = true;
+  }
   if (int rc = apply_launch(h, h->block, h->waves, h->split)) return rc;
   CU(cudaStreamSynchronize(h->stream));
   h->ready = true;
@@ -1231,6 +1297,15 @@ int dgswe_step(dgswe_h h, int64_t n) {
     for (int64_t i = 0; i < n; ++i)
       for (size_t s = 0; s < h->stages.size(); ++s)
         if (int rc = launch_stage_once(h, (int)s, 0, h->stream)) return rc;
+    return 0;
+  }
+  if (h->small) {  // at most 1024 steps (a few milliseconds) per launch
+    for (int64_t i = 0; i < n; i += 1024) {
+      const int k = (int)std::min<int64_t>(1024, n - i);
+      const cudaError_t e = mixed(h) ? enqueue_small<Mixed>(h, k) : enqueue_small<Fp64>(h, k);
+      if (e != cudaSuccess) return fail(DGSWE_ECUDA, "small-mesh launch: %s", cudaGetErrorString(e));
+      h->launches++;
+    }
     return 0;
   }
   if (!h->g1)
@@ -1584,6 +1659,7 @@ int dgswe_set_launch(dgswe_h h, int32_t block, int32_t waves, int32_t split) {
   if (waves < 1 || waves > 2) return fail(DGSWE_EINVAL, "waves must be 1 or 2");
   if (split < 0 || split > 2) return fail(DGSWE_EINVAL, "split must be 0, 1 or 2");
   h->autotune = false;
+  h->small = false;
   if (!h->ready) {
     h->block = block;
     h->waves = waves;

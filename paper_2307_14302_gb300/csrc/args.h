@@ -65,6 +65,17 @@ struct StageArgs {
   T g, H0, cf;
 };
 
+// the stages of a step and the steps of one launch of the small-mesh kernel (steps.cuh); buffers:
+// 0 holds w^n and receives the step's result, 1 and 2 alternate as stage outputs
+struct StepsArgs {
+  struct Stage {
+    int in, out, has_n, pow2;
+    float a_n_hi, a_n_lo, a_in_hi, a_in_lo, bw_hi, bw_lo;
+    double a_n, a_in, cst, bw;
+  } st[MAXSTAGE];
+  int nstage, nsteps, nrec;
+};
+
 }  // namespace dg
 
 namespace dg {
@@ -132,6 +143,16 @@ template <class Pol>
 cudaError_t launch_tile(int p, int flux, int feat, const StageArgs<Pol>& a, int grid, int block, cudaStream_t s);
 template <class Pol>
 int tile_blocks_per_sm(int p, int flux, int feat, int block);
+// small meshes (steps.cuh): whole steps in one launch of one cluster of ctas CTAs with wpc tiles each;
+// whether a launch of that shape fits the device, the launch, and the reference tables of its
+// translation units
+template <class Pol>
+bool steps_fit(int p, int flux, int feat, int ctas, int wpc, int nrec);
+template <class Pol>
+cudaError_t launch_steps(int p, int flux, int feat, const StageArgs<Pol>& a, const StepsArgs& st, int ctas, int wpc,
+                         cudaStream_t s);
+template <class Pol>
+cudaError_t upload_steps_tables(int p, const RefTab<float>& tf, const RefTab<double>& td);
 // specialised mixed-precision tile kernels (tile_spec.cu): launch or occupancy of the one that
 // covers feat; cudaErrorNotSupported (launch) or -1 (occupancy) when none does
 cudaError_t launch_tile_spec(int p, int flux, int feat, const StageArgs<Mixed>& a, int grid, int block,
