@@ -23,10 +23,8 @@ template <int P, class Pol, int FT = FT_ALL>
 struct StepsLayout {
   using L = TileLayout<P, Pol, FT>;
   static constexpr int RECS = TILE * L::RV;                       // one record buffer of a tile, 16-byte units
-  static constexpr int GEO = 0;
-  static constexpr int PLAN = GEO + TILE * L::GV;
-  static constexpr int XY = PLAN + L::PV;
-  static constexpr int HAL = XY + L::XV;
+  static constexpr int GEO = L::S_GEO, PLAN = L::S_PLAN, XY = L::S_XY;
+  static constexpr int HAL = L::SV;
   static constexpr int FLX = HAL + HALO * L::RV;
   static constexpr int REC = FLX + (L::BAR - L::FLX);             // 2 or 3 record buffers
   DG_HD static constexpr int vec(int nrec) { return REC + nrec * RECS; }
@@ -98,7 +96,7 @@ __global__ void __maxnreg__(sizeof(typename Pol::T) == 4 ? (P == 1 ? 128 : 200) 
     return cluster_map(smem_u32(tsm + (size_t)(nt % wpc) * vec + SL::REC) + 16u * (n & 31), (uint32_t)(nt / wpc));
   };
   const uint32_t hsrc =
-      lane < nhalo ? remote(reinterpret_cast<const int32_t*>(Wm + SL::PLAN + EDGE_INLINE / 4)[lane]) : 0u;
+      lane < nhalo ? remote(reinterpret_cast<const int32_t*>(Wm + L::S_HALO)[lane]) : 0u;
   const ScenDev& S = a.scen[sc];
   const unsigned long long step0 = a.ctl->step;
   const int rain_kind = ft_rain(FT) >= 0 ? ft_rain(FT) : S.rain_kind;
@@ -148,7 +146,7 @@ __global__ void __maxnreg__(sizeof(typename Pol::T) == 4 ? (P == 1 ? 128 : 200) 
       tile_body<P, FLUX, Pol, FT, true>(a, S, t64, rain_kind, press, rr, tile, lane, valid, meta.z,
                                         Wm + SL::REC + c.in * SL::RECS, halo, Wm + SL::GEO,
                                         reinterpret_cast<const unsigned*>(Wm + SL::PLAN),
-                                        reinterpret_cast<const float*>(Wm + SL::PLAN + (EDGE_INLINE + HALO) / 4),
+                                        reinterpret_cast<const float*>(Wm + L::S_MAN),
                                         reinterpret_cast<const T*>(Wm + SL::XY), Wm + SL::FLX, Wm + SL::REC, s_ephi,
                                         s_ephi4, halo_ready,
                                         [&](int n, Raw<RV>& r) {
@@ -156,6 +154,7 @@ __global__ void __maxnreg__(sizeof(typename Pol::T) == 4 ? (P == 1 ? 128 : 200) 
 #pragma unroll
                                           for (int v = 0; v < RV; ++v) r.v[v] = ld_cluster128(at + 16u * TILE * v);
                                         },
+                                        [] {},
                                         O, rain_acc, bdry_acc);
       if (valid) {
         Raw<RV> ro;

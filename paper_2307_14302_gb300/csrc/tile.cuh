@@ -85,21 +85,29 @@ struct TileLayout {
   static constexpr int NPR = (NV + 1) / 2;
   // first vertices of a tile (storm rain and pressure set-up only), 16-byte units
   static constexpr int XV = (FT & (FT_RAIN2 | FT_PRESS)) ? (sizeof(T) == 4 ? 16 : 32) : 0;
-  // one buffer: records [RV][32] (the tile's block of the tile-blocked record array), geometry
-  // [32][GV], plan, first vertices, all filled by the TMA batch
+  // static part of a tile: geometry [32][GV], plan, first vertices
   static constexpr int PV = plan_vec<T>();
-  static constexpr int O_GEO = TILE * RV;
-  static constexpr int O_PLAN = O_GEO + TILE * GV;
-  static constexpr int O_HALO = O_PLAN + EDGE_INLINE / 4;      // halo element indices
-  static constexpr int O_MAN = O_HALO + HALO / 4;              // Manning coefficients (mixed)
-  static constexpr int O_META = O_PLAN + PV - 1;
-  static constexpr int O_XY = O_PLAN + PV;
-  static constexpr int BUF = O_XY + XV;
-  static constexpr int HAL = 2 * BUF;                          // [RV][HALO]
-  static constexpr int FLX = HAL + HALO * RV;                  // edge slots [3][NPR][32], pairs of T
-  static constexpr int BAR = FLX + 3 * NPR * 32 * 2 * (int)sizeof(T) / 16;  // two 8-byte mbarriers
-  static constexpr int VEC = BAR + 1;                          // 16-byte units per warp
-  static constexpr unsigned TILE_BYTES = 16u * BUF;            // bytes of one buffer's copies
+  static constexpr int S_GEO = 0;
+  static constexpr int S_PLAN = S_GEO + TILE * GV;
+  static constexpr int S_HALO = S_PLAN + EDGE_INLINE / 4;      // halo element indices
+  static constexpr int S_MAN = S_HALO + HALO / 4;              // Manning coefficients (mixed)
+  static constexpr int S_META = S_PLAN + PV - 1;
+  static constexpr int S_XY = S_PLAN + PV;
+  static constexpr int SV = S_XY + XV;
+  // per warp: two record buffers [RV][32] (the tile's block of the tile-blocked record array), the
+  // static buffers, the halo records [RV][HALO], the edge slots [3][NPR][32] (pairs of T) and three
+  // 8-byte mbarriers (buffers 0 and 1, single static).  Mixed p = 2 has one static buffer: the static
+  // part is done with after the edge phase and the next tile's is copied in during the rest of this
+  // one, which takes 2.3 KB less per warp and lets 12 warps share an SM instead of 8 (graded 300k:
+  // 159 -> 143 us per step).  At p = 1 the second buffer is free (registers allow 16 warps either
+  // way) and 2 % faster (hurricane 2M: 260 us per step against 265).
+  static constexpr int NSTAT = (sizeof(T) == 4 && P == 2) ? 1 : 2;
+  static constexpr int REC = TILE * RV;
+  static constexpr int STAT = 2 * REC;
+  static constexpr int HAL = STAT + NSTAT * SV;
+  static constexpr int FLX = HAL + HALO * RV;
+  static constexpr int BAR = FLX + 3 * NPR * 32 * 2 * (int)sizeof(T) / 16;
+  static constexpr int VEC = BAR + 2;                          // 16-byte units per warp
 };
 template <int P, class Pol, int FT = FT_ALL>
 __host__ __device__ constexpr int tile_smem_bytes(int block) {
@@ -145,12 +153,15 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
   return ok != 0;
 }
 
-// a bulk copy that did not complete: record it in the device error word, give the copy one more
-// bounded wait so that it does not land in shared memory after the warp has left, and return
+// a bulk copy that did not complete: record it in the device error word, give the warp's copies (this
+// tile's and the next tile's records, the static part) one more bounded wait so that none lands in
+// shared memory after the warp has left, and return
 template <class Pol>
-__device__ __noinline__ void tile_timeout(const StageArgs<Pol>& a, uint32_t bar, uint32_t parity, int lane) {
+__device__ __noinline__ void tile_timeout(const StageArgs<Pol>& a, uint32_t bar, int it, bool next, bool sd, int lane) {
   if (lane == 0) atomicOr(&a.ctl->err, ERR_TIMEOUT);
-  (void)mbar_wait(bar, parity);
+  if (!sd) (void)mbar_wait(bar + 16, it & 1);
+  (void)mbar_wait(bar + 8 * (it & 1), (it >> 1) & 1);
+  if (next) (void)mbar_wait(bar + 8 * ((it + 1) & 1), ((it + 1) >> 1) & 1);
 }
 
 // static geometry record from shared memory (layout of load_geo); the Manning coefficient of the
@@ -876,15 +887,15 @@ __global__ void __launch_bounds__(256) plan_kernel(const int4* nbr, const int4* 
 // once, then the lift, stage combination and positive-depth operator; O is the element's new record.
 // halo_ready() makes the staged halo records readable; it is called once by the whole warp, before
 // the first round that has an edge to another tile; far(element, record) reads a neighbour beyond the
-// halo slots after that.  The step-initial record comes from shared
-// memory (WNS) or from a.wn.
-template <int P, int FLUX, class Pol, int FT, bool WNS, class HaloReady, class Far>
+// halo slots after that; release() is called once by the whole warp when the tile's static data is
+// done with.  The step-initial record comes from shared memory (WNS) or from a.wn.
+template <int P, int FLUX, class Pol, int FT, bool WNS, class HaloReady, class Far, class Release>
 __device__ __forceinline__ void tile_body(const StageArgs<Pol>& a, const ScenDev& S, double t64, int rain_kind, int press,
                                           const RainRec<typename Pol::T>& rr, int tile, int lane, bool valid, int counts,
                                           const uint4* own, const uint4* halo, const uint4* geoS, const unsigned* planS,
                                           const float* man, const typename Pol::T* xyS, void* flx, const uint4* wnS,
                                           const typename Pol::T (*s_ephi)[P + 1][np_of(P)], const float4* s_ephi4,
-                                          HaloReady halo_ready, Far far, Elem<P, Pol>& O, typename Pol::Acc& rain_acc,
+                                          HaloReady halo_ready, Far far, Release release, Elem<P, Pol>& O, typename Pol::Acc& rain_acc,
                                           typename Pol::Acc& bdry_acc) {
   using T = typename Pol::T;
   using Acc = typename Pol::Acc;
@@ -977,9 +988,10 @@ __device__ __forceinline__ void tile_body(const StageArgs<Pol>& a, const ScenDev
   __syncwarp();
 
   // ---- element phase B: lift, inverse mass, stage combination, positive-depth operator
+  Geo<Pol> G;
+  if (valid) geo_from(geoS + lane * GV, man + lane, G);
+  release();
   if (valid) {
-    Geo<Pol> G;
-    geo_from(geoS + lane * GV, man + lane, G);
     Elem<P, Pol> E;
     {
       Raw<RV> r;
@@ -1074,9 +1086,11 @@ __device__ __forceinline__ void tile_body(const StageArgs<Pol>& a, const ScenDev
 
 // -------------------------------------------------------------------------- the kernel ---
 #ifndef DG_TILE_MAXNREG
-// register budget: mixed p = 1 at 128 (16 warps per SM, as its shared memory allows); elsewhere
-// shared memory allows about 10 (mixed p = 2) or 9 (FP64 p = 1) warps, which leaves 200 or more
-#define DG_TILE_BOUNDS __maxnreg__(sizeof(typename Pol::T) == 4 ? (P == 1 ? 128 : 200) : 224)
+// register budget (registers are allocated per SM sub-partition, so a kernel gets 4 floor(512 / regs)
+// warps): mixed p = 1 at 128 for 16 warps per SM, mixed p = 2 at 168 for 12; FP64 at 224 for 8.
+// Mixed p = 1 at 96 registers (20 warps, one static buffer) was slower: hurricane 2M 279 us per step
+// against 260, 500k LLF 224 against 188; the kernel wants instruction-level parallelism, not warps.
+#define DG_TILE_BOUNDS __maxnreg__(sizeof(typename Pol::T) == 4 ? (P == 1 ? 128 : 168) : 224)
 #else
 #define DG_TILE_BOUNDS __maxnreg__(DG_TILE_MAXNREG)
 #endif
@@ -1107,26 +1121,37 @@ __global__ void DG_TILE_BOUNDS tile_kernel(const StageArgs<Pol> a) {
   uint4* Wm = tsm + (size_t)(tid >> 5) * L::VEC;
   uint4* halo = Wm + L::HAL;                                       // [HALO][RV]
   void* flx = Wm + L::FLX;                                         // [3][NPR][32] pairs
-  const uint32_t bar0 = smem_u32(Wm + L::BAR), bar1 = bar0 + 8;
+  const uint32_t bar = smem_u32(Wm + L::BAR);  // record buffers 0 and 1 at +0 and +8, static at +16
   if (lane == 0) {
-    mbar_init(bar0, 1);
-    mbar_init(bar1, 1);
+    mbar_init(bar, 1);
+    mbar_init(bar + 8, 1);
+    mbar_init(bar + 16, 1);
     mbar_fence_init();
   }
   __syncwarp();
   const int gw = blockIdx.x * (blockDim.x >> 5) + (tid >> 5);
   const int W = gridDim.x * (blockDim.x >> 5);
-  // one TMA batch: the tile's records, geometry, plan and first vertices into a buffer (lane 0)
+  // TMA copies by lane 0: a tile's records into a buffer; its geometry, plan and first vertices, with
+  // the records' barrier when they are double-buffered too
+  constexpr bool SD = L::NSTAT == 2;
+  auto copy_static = [&](int t, uint4* to, uint32_t br) {
+    bulk_g2s(smem_u32(to + L::S_GEO), a.geo + (size_t)t * TILE * GV, 16u * TILE * GV, br);
+    bulk_g2s(smem_u32(to + L::S_PLAN), a.plan + (size_t)t * L::PV, 16u * L::PV, br);
+    if constexpr (L::XV > 0) bulk_g2s(smem_u32(to + L::S_XY), a.xy0 + (size_t)t * L::XV, 16u * L::XV, br);
+  };
   auto issue = [&](int t, int b) {
     if (lane == 0) {
-      uint4* buf = Wm + (b ? L::BUF : 0);
-      const uint32_t bar = b ? bar1 : bar0;
       fence_proxy_async();
-      mbar_expect_tx(bar, L::TILE_BYTES);
-      bulk_g2s(smem_u32(buf), a.in + (size_t)t * TILE * RV, 16u * TILE * RV, bar);
-      bulk_g2s(smem_u32(buf + L::O_GEO), a.geo + (size_t)t * TILE * GV, 16u * TILE * GV, bar);
-      bulk_g2s(smem_u32(buf + L::O_PLAN), a.plan + (size_t)t * L::PV, 16u * L::PV, bar);
-      if constexpr (L::XV > 0) bulk_g2s(smem_u32(buf + L::O_XY), a.xy0 + (size_t)t * L::XV, 16u * L::XV, bar);
+      mbar_expect_tx(bar + 8 * b, 16u * (L::REC + (SD ? L::SV : 0)));
+      bulk_g2s(smem_u32(Wm + b * L::REC), a.in + (size_t)t * L::REC, 16u * L::REC, bar + 8 * b);
+      if constexpr (SD) copy_static(t, Wm + L::STAT + b * L::SV, bar + 8 * b);
+    }
+  };
+  auto issue_static = [&](int t) {  // the single static buffer
+    if (!SD && lane == 0) {
+      fence_proxy_async();
+      mbar_expect_tx(bar + 16, 16u * L::SV);
+      copy_static(t, Wm + L::STAT, bar + 16);
     }
   };
   const double stepd = (double)a.ctl->step + a.cst;
@@ -1137,26 +1162,29 @@ __global__ void DG_TILE_BOUNDS tile_kernel(const StageArgs<Pol> a) {
   double t64 = 0.0;
   int rain_kind = 0, press = 0;
   RainRec<T> rr = {nullptr, nullptr, T(0)};  // gridded rain: the two records around the stage time
-  uint32_t ph = 0;  // parity of the next completion: bit 0 buffer 0, bit 1 buffer 1
-  if (gw < a.ntiles) issue(gw, 0);
+  if (gw < a.ntiles) {
+    issue_static(gw);
+    issue(gw, 0);
+  }
 
   int it = 0;
   for (int tile = gw; tile < a.ntiles; tile += W, ++it) {
-    const int b = it & 1;
-    if (tile + W < a.ntiles) issue(tile + W, b ^ 1);  // the other buffer's tile was consumed last iteration
-    if (!__all_sync(0xffffffffu, mbar_wait(b ? bar1 : bar0, (ph >> b) & 1u))) {
-      tile_timeout(a, b ? bar1 : bar0, (ph >> b) & 1u, lane);
+    const int b = it & 1, next = tile + W;
+    if (next < a.ntiles) issue(next, b ^ 1);  // the other buffer's tile was consumed last iteration
+    const bool arrived = (SD || mbar_wait(bar + 16, it & 1)) && mbar_wait(bar + 8 * b, (it >> 1) & 1);
+    if (!__all_sync(0xffffffffu, arrived)) {
+      tile_timeout(a, bar, it, next < a.ntiles, SD, lane);
       return;
     }
-    ph ^= 1u << b;
-    uint4* const buf = Wm + (b ? L::BUF : 0);
-    const uint4* own = buf;                           // [RV][32] records
-    const uint4* geoS = own + L::O_GEO;               // [32][GV]
-    const unsigned* planS = reinterpret_cast<const unsigned*>(own + L::O_PLAN);
-    const int4 meta = reinterpret_cast<const int4*>(own + L::O_META)[0];
+    const uint4* own = Wm + b * L::REC;                           // [RV][32] records
+    const uint4* stat = Wm + L::STAT + (SD ? b * L::SV : 0);
+    const uint4* geoS = stat + L::S_GEO;                          // [32][GV]
+    const unsigned* planS = reinterpret_cast<const unsigned*>(stat + L::S_PLAN);
+    const int4 meta = reinterpret_cast<const int4*>(stat + L::S_META)[0];
     const int sc = meta.x, present = meta.y;
     if (present == 0) {  // padding tile: no element (uniform over the warp)
       __syncwarp();
+      if (next < a.ntiles) issue_static(next);
       continue;
     }
     if (sc != cur) {
@@ -1182,7 +1210,7 @@ __global__ void DG_TILE_BOUNDS tile_kernel(const StageArgs<Pol> a) {
 
     // ---- the out-of-tile neighbours' records, one halo slot per lane, by the tile's plan
     if (lane < (meta.z >> 16)) {
-      const int n = reinterpret_cast<const int32_t*>(own + L::O_HALO)[lane];
+      const int n = reinterpret_cast<const int32_t*>(stat + L::S_HALO)[lane];
 #pragma unroll
       for (int v = 0; v < RV; ++v) cp_async16(halo + v * HALO + lane, a.in + rec_at<RV>(n, v));
     }
@@ -1190,8 +1218,8 @@ __global__ void DG_TILE_BOUNDS tile_kernel(const StageArgs<Pol> a) {
 
     Elem<P, Pol> O;
     tile_body<P, FLUX, Pol, FT, false>(a, S, t64, rain_kind, press, rr, tile, lane, valid, meta.z, own, halo, geoS, planS,
-                                       reinterpret_cast<const float*>(own + L::O_MAN),
-                                       reinterpret_cast<const T*>(own + L::O_XY), flx, nullptr, s_ephi, s_ephi4,
+                                       reinterpret_cast<const float*>(stat + L::S_MAN),
+                                       reinterpret_cast<const T*>(stat + L::S_XY), flx, nullptr, s_ephi, s_ephi4,
                                        [] {
                                          cp_async_wait_all();
                                          __syncwarp();
@@ -1199,6 +1227,11 @@ __global__ void DG_TILE_BOUNDS tile_kernel(const StageArgs<Pol> a) {
                                        [&](int n, Raw<RV>& r) {
 #pragma unroll
                                          for (int v = 0; v < RV; ++v) r.v[v] = __ldg(a.in + rec_at<RV>(n, v));
+                                       },
+                                       [&] {
+                                         if (SD) return;
+                                         __syncwarp();
+                                         if (next < a.ntiles) issue_static(next);
                                        },
                                        O, rain_acc, bdry_acc);
     if (valid) {
