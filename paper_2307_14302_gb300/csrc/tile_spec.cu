@@ -50,8 +50,7 @@ cudaError_t launch_tile_spec(int p, int flux, int feat, const StageArgs<Mixed>& 
                              cudaStream_t s) {
   const Spec* sp = find_spec(p, flux, feat);
   if (!sp) return cudaErrorNotSupported;
-  sp->k<<<grid, block, smem_bytes(*sp, block), s>>>(a);
-  return cudaGetLastError();
+  return tile_launch_pdl<Mixed>(sp->k, a, grid, block, smem_bytes(*sp, block), s);
 }
 
 int tile_spec_features(int p, int flux, int feat) {
