@@ -21,6 +21,7 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <cstring>
 
 #include "args.h"
 #include "layout.h"
@@ -1232,30 +1233,65 @@ __device__ __forceinline__ bool limit_var(typename Pol::T* s, const typename Pol
   return true;
 }
 
+// programmatic dependent launch: wait until the kernels before this one have finished and their
+// writes are visible; launch_pdl starts a kernel whose CTAs may come that early
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+template <class... P, class... A>
+static cudaError_t launch_pdl(void (*k)(P...), int grid, int block, int smem, cudaStream_t s, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k, args...);
+}
+
 template <class Pol>
 __global__ void __launch_bounds__(256) limit_kernel(const StageArgs<Pol> a, long long ne) {
   using T = typename Pol::T;
   constexpr int RV = Pol::template RV<1>;
   const RefTab<T>& tab = ctab<T, 1>();
-  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < ne; e += (long long)gridDim.x * blockDim.x) {
+  const long long e0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  bool waited = false;
+  for (long long e = e0; e < ne; e += (long long)gridDim.x * blockDim.x) {
     const int4 nb = __ldg(a.nbr + e);
-    if (nb.x < 0 || nb.y < 0 || nb.z < 0) continue;
-    const T* L = a.lim + 8 * e;
+    T L[8];
+    {
+      const uint4* lv = reinterpret_cast<const uint4*>(a.lim + 8 * e);
+      uint4 v[sizeof(T) / 2];
+#pragma unroll
+      for (int i = 0; i < (int)sizeof(T) / 2; ++i) v[i] = __ldg(lv + i);
+      memcpy(L, v, sizeof L);
+    }
+    if (!waited) pdl_wait();  // the stage's kernel before this one
+    waited = true;
     const int bits = (int)L[7];
-    if (bits < 0) continue;
-    Raw<RV> r;
+    if (bits < 0 || nb.x < 0 || nb.y < 0 || nb.z < 0) continue;
+    // the element's record and its neighbours' means (the first two vectors), all requested together:
+    // the kernel waits on one round of loads instead of three (flag, record, neighbours)
+    Raw<RV> r, rn[3];
     load_raw<RV>(a.out, e, r);
+#pragma unroll
+    for (int j = 0; j < 3; ++j) {
+      const int code = (j == 0) ? nb.x : (j == 1 ? nb.y : nb.z);
+      rn[j].v[0] = __ldg(a.out + rec_at<RV>(code >> 2, 0));
+      rn[j].v[1] = __ldg(a.out + rec_at<RV>(code >> 2, 1));
+#pragma unroll
+      for (int i = 2; i < RV; ++i) rn[j].v[i] = make_uint4(0, 0, 0, 0);
+    }
     Elem<1, Pol> E;
     unpack<1>(r, E);
     if (E.flags & FLAG_DRY) continue;
     T dz[3], dx[3], dy[3];
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
-      const int code = (j == 0) ? nb.x : (j == 1 ? nb.y : nb.z);
-      Raw<RV> rn;
-      load_raw<RV>(a.out, (long long)(code >> 2), rn);
       Elem<1, Pol> N;
-      unpack<1>(rn, N);
+      unpack<1>(rn[j], N);
       dz[j] = acc_diff(N.zb, E.zb);
       dx[j] = acc_diff(N.xb, E.xb);
       dy[j] = acc_diff(N.yb, E.yb);
@@ -2071,8 +2107,7 @@ static inline int grid_for(long long n, int block) {
   }                                                                                                          \
   template <>                                                                                                \
   cudaError_t launch_limiter<POL>(const StageArgs<POL>& a, long long ne, cudaStream_t s) {                   \
-    limit_kernel<POL><<<grid_for(ne, 256), 256, 0, s>>>(a, ne);                                              \
-    return cudaGetLastError();                                                                               \
+    return launch_pdl(limit_kernel<POL>, grid_for(ne, 256), 256, 0, s, a, ne);                               \
   }                                                                                                          \
   template <>                                                                                                \
   cudaError_t launch_node_rain<POL>(const StageArgs<POL>& a, long long nn, cudaStream_t s) {                 \

@@ -153,10 +153,6 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
   return ok != 0;
 }
 
-// programmatic dependent launch: wait until the kernels before this one have finished and their
-// writes are visible
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
 // a bulk copy that did not complete: record it in the device error word, give the warp's copies (this
 // tile's and the next tile's records, the static part) one more bounded wait so that none lands in
 // shared memory after the warp has left, and return

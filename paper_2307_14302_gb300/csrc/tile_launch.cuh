@@ -14,23 +14,6 @@ static cudaError_t tile_smem_limit(K kernel, int optin, int need) {
   const int room = optin - (int)fa.sharedSizeBytes;
   return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, need < room ? need : room);
 }
-// a launch that may start while the kernel before it in the stream drains (tile_kernel waits for it
-// before it touches what steps write)
-template <class Pol>
-static cudaError_t tile_launch_pdl(void (*k)(const StageArgs<Pol>), const StageArgs<Pol>& a, int grid, int block,
-                                   int smem, cudaStream_t s) {
-  cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  cfg.gridDim = dim3(grid);
-  cfg.blockDim = dim3(block);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, k, a);
-}
 // the specialised instantiations exist for the mixed path only
 template <class Pol>
 inline cudaError_t tile_try_spec(int, int, int, const StageArgs<Pol>&, int, int, cudaStream_t) {
@@ -85,10 +68,10 @@ inline int tile_try_spec_occ<Mixed>(int p, int flux, int feat, int block) {
     if (es != cudaErrorNotSupported) return es;                                                              \
     const int k = (p == 1 ? 0 : 2) + (flux ? 1 : 0);                                                         \
     switch (k) {                                                                                             \
-      case 0: return tile_launch_pdl<POL>(tile_kernel<1, 0, POL>, a, grid, block, tile_smem_bytes<1, POL>(block), s); \
-      case 1: return tile_launch_pdl<POL>(tile_kernel<1, 1, POL>, a, grid, block, tile_smem_bytes<1, POL>(block), s); \
-      case 2: return tile_launch_pdl<POL>(tile_kernel<2, 0, POL>, a, grid, block, tile_smem_bytes<2, POL>(block), s); \
-      default: return tile_launch_pdl<POL>(tile_kernel<2, 1, POL>, a, grid, block, tile_smem_bytes<2, POL>(block), s); \
+      case 0: return launch_pdl(tile_kernel<1, 0, POL>, grid, block, tile_smem_bytes<1, POL>(block), s, a); \
+      case 1: return launch_pdl(tile_kernel<1, 1, POL>, grid, block, tile_smem_bytes<1, POL>(block), s, a); \
+      case 2: return launch_pdl(tile_kernel<2, 0, POL>, grid, block, tile_smem_bytes<2, POL>(block), s, a); \
+      default: return launch_pdl(tile_kernel<2, 1, POL>, grid, block, tile_smem_bytes<2, POL>(block), s, a); \
     }                                                                                                        \
   }                                                                                                          \
   template <>                                                                                                \

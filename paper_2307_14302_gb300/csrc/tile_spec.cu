@@ -50,7 +50,7 @@ cudaError_t launch_tile_spec(int p, int flux, int feat, const StageArgs<Mixed>& 
                              cudaStream_t s) {
   const Spec* sp = find_spec(p, flux, feat);
   if (!sp) return cudaErrorNotSupported;
-  return tile_launch_pdl<Mixed>(sp->k, a, grid, block, smem_bytes(*sp, block), s);
+  return launch_pdl(sp->k, grid, block, smem_bytes(*sp, block), s, a);
 }
 
 int tile_spec_features(int p, int flux, int feat) {
