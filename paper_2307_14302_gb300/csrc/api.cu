@@ -149,6 +149,7 @@ struct dgswe_ctx {
   cudaGraphExec_t g1 = nullptr, gK = nullptr;
   int K = 8;
   long long launches = 0;
+  Summary* sum = nullptr;          // page-locked: sums written by the device (summarise)
   char* bound = nullptr;           // caller memory holding the three record buffers (dgswe_bind_device)
   size_t bound_bytes = 0;
 
@@ -159,6 +160,7 @@ struct dgswe_ctx {
                       &edges, &slots,
                       &rain_node, &node_scen, &lim, &rain_rec, &plan, &plan_x};
     for (DevBuf* b : bufs) b->alloc(0);
+    if (sum) cudaFreeHost(sum);
     if (g1) cudaGraphExecDestroy(g1);
     if (gK) cudaGraphExecDestroy(gK);
     if (cap) cudaStreamDestroy(cap);
@@ -167,43 +169,6 @@ struct dgswe_ctx {
 };
 
 // ------------------------------------------------------------------------------ helpers --
-// Neumaier-compensated sum of per-block (sum, compensation) pairs, one CTA, fixed order
-__global__ void __launch_bounds__(256) reduce_pairs_kernel(const double* part, int nblk, int npairs, double* out) {
-  __shared__ double sh[2][8];
-  for (int k = 0; k < npairs; ++k) {
-    double s = 0.0, c = 0.0;
-    for (int b = threadIdx.x; b < nblk; b += blockDim.x) {
-      const double v = part[4 * b + 2 * k], t = s + v;
-      c += (fabs(s) >= fabs(v)) ? (s - t) + v : (v - t) + s;
-      s = t;
-      c += part[4 * b + 2 * k + 1];
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-      const double v = __shfl_xor_sync(0xffffffffu, s, o), vc = __shfl_xor_sync(0xffffffffu, c, o);
-      const double t = s + v;
-      c += ((fabs(s) >= fabs(v)) ? (s - t) + v : (v - t) + s) + vc;
-      s = t;
-    }
-    if ((threadIdx.x & 31) == 0) { sh[0][threadIdx.x >> 5] = s; sh[1][threadIdx.x >> 5] = c; }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      for (int w = 1; w < (int)(blockDim.x >> 5); ++w) {
-        const double v = sh[0][w], t = s + v;
-        c += ((fabs(s) >= fabs(v)) ? (s - t) + v : (v - t) + s) + sh[1][w];
-        s = t;
-      }
-      out[2 * k] = s;
-      out[2 * k + 1] = c;
-    }
-    __syncthreads();
-  }
-}
-
-cudaError_t dg::launch_reduce_pairs(const double* partials, int nblk, int npairs, double* out, cudaStream_t s) {
-  reduce_pairs_kernel<<<1, 256, 0, s>>>(partials, nblk, npairs, out);
-  return cudaGetLastError();
-}
-
 static void split_ff(double v, float& hi, float& lo) {
   hi = (float)v;
   lo = (float)(v - (double)hi);
@@ -323,11 +288,6 @@ static size_t record_stride(size_t rbytes) { return (rbytes + 255) / 256 * 256; 
 // Element records on the device are tile-blocked (the layout the kernels read): the 16-byte
 // vector v of element e is vector ((e / 32) rv + v) 32 + e % 32 of the array.
 static size_t rec_vec(size_t e, size_t v, size_t rv) { return ((e >> 5) * rv + v) * 32 + (e & 31); }
-// 32-bit word w of element e's record in a tile-blocked array (e counted from the array's start,
-// which is tile-aligned)
-static uint32_t rec_word(const std::vector<uint32_t>& blk, size_t e, size_t w, size_t rv) {
-  return blk[4 * rec_vec(e, w / 4, rv) + w % 4];
-}
 // element-major records (rw = 4 rv words each) -> tile-blocked, E a multiple of 32
 static std::vector<uint32_t> to_blocked(const std::vector<uint32_t>& rec, size_t E, size_t rv) {
   std::vector<uint32_t> blk(rec.size());
@@ -604,6 +564,7 @@ static int build_layout(dgswe_h h) {
   if (h->rain_rec.alloc(records ? rr_bytes : 0)) return fail(DGSWE_ENOMEM, "device allocation of %zu bytes failed", rr_bytes);
   h->grid_rain = rr_elems > 0 && !records;
   CU(cudaMemset(h->ctl.p, 0, sizeof(Ctl)));
+  CU(cudaMemset(h->scratch.p, 0, h->scratch.n));
   // per-scenario parameter blocks (dt filled in later)
   std::vector<ScenDev> sd(ns);
   for (size_t s = 0; s < ns; ++s) {
@@ -978,22 +939,20 @@ static int build_graphs(dgswe_h h) {
   return 0;
 }
 
-static int reduce_volume(dgswe_h h, size_t s, double& V, double& VH) {
+// sums over scenario s (h->sum, valid after this returns): synchronises the stream
+static int summarise(dgswe_h h, size_t s, bool depth) {
   const long long b = h->eoff[s], e = b + h->sc[s].m.ne;
-  const int nblk = (int)std::min<long long>(1024, std::max<long long>(1, (e - b + 255) / 256));
+  // four elements per thread of 128-thread blocks, at most two blocks per SM
+  const int nblk = (int)std::min<long long>(304, std::max<long long>(1, (e - b + 511) / 512));
   double* part = h->scratch.as<double>();
-  cudaError_t ce = mixed(h) ? launch_volume<Mixed>(h->prm.p, h->rec[0].as<uint4>(), h->geo.as<uint4>(), b, e, part, nblk, h->stream)
-                            : launch_volume<Fp64>(h->prm.p, h->rec[0].as<uint4>(), h->geo.as<uint4>(), b, e, part, nblk, h->stream);
-  if (ce != cudaSuccess) return fail(DGSWE_ECUDA, "volume launch: %s", cudaGetErrorString(ce));
+  unsigned* ticket = reinterpret_cast<unsigned*>(part + 9 * 304);
+  const double* led = h->ledger.as<double>() + 2 * s * (size_t)h->wslots;
+  auto go = mixed(h) ? launch_summary<Mixed> : launch_summary<Fp64>;
+  const cudaError_t ce = go(h->prm.p, depth, h->rec[0].as<uint4>(), h->geo.as<uint4>(), b, e, led, h->wcur,
+                            h->ctl.as<Ctl>(), part, ticket, h->sum, nblk, h->stream);
+  if (ce != cudaSuccess) return fail(DGSWE_ECUDA, "summary launch: %s", cudaGetErrorString(ce));
   h->launches++;
-  ce = launch_reduce_pairs(part, nblk, 2, part + 4 * 1024, h->stream);
-  if (ce != cudaSuccess) return fail(DGSWE_ECUDA, "reduce launch: %s", cudaGetErrorString(ce));
-  h->launches++;
-  double out[4];
-  CU(cudaMemcpyAsync(out, part + 4 * 1024, sizeof out, cudaMemcpyDeviceToHost, h->stream));
   CU(cudaStreamSynchronize(h->stream));
-  V = out[0] + out[1];
-  VH = out[2] + out[3];
   return 0;
 }
 
@@ -1036,7 +995,9 @@ static int prepare(dgswe_h h) {
         h->sc[s].dt = *std::min_element(mins.begin(), mins.end());
       }
     }
-    if (int rc = reduce_volume(h, s, h->V0[s], h->VH0[s])) return rc;
+    if (int rc = summarise(h, s, true)) return rc;
+    h->V0[s] = h->sum->sum[0];
+    h->VH0[s] = h->sum->sum[1];
   }
   if (int rc = upload_dt(h)) return rc;
   if (h->small) {  // the mesh may have changed: decide again at the next step
@@ -1076,6 +1037,7 @@ int dgswe_create(dgswe_h* out, int device, void* cuda_stream) {
     h->own_stream = true;
   }
   CU(cudaStreamCreateWithFlags(&h->cap, cudaStreamNonBlocking));
+  CU(cudaHostAlloc((void**)&h->sum, sizeof(Summary), cudaHostAllocMapped));
   *out = h.release();
   return 0;
 }
@@ -1530,56 +1492,38 @@ int dgswe_get_dry(dgswe_h h, uint8_t* dry) {
   if (!h->ready) return fail(DGSWE_ESTATE, "no state");
   if (!dry) return fail(DGSWE_EINVAL, "null output");
   DeviceGuard dg_(h->device);
-  const HostMesh& M = h->sc[0].m;
-  const size_t rw = 4 * (size_t)h->rv;
-  std::vector<uint32_t> rec(rw * ((size_t)(M.ne + TILE - 1) / TILE * TILE));  // whole tiles
+  // the flags in caller order, written by the kernel to page-locked memory or staged through a device
+  // buffer: n bytes cross the host link instead of every record
+  const long long n = h->sc[0].m.ne, b = h->eoff[0];
+  uint8_t* to = (uint8_t*)host_mapped(dry);
+  const bool staged = to == nullptr;
+  if (staged) {
+    if (h->gather_buf.n < (size_t)n)
+      if (h->gather_buf.alloc((size_t)n)) return fail(DGSWE_ENOMEM, "gather buffer");
+    to = h->gather_buf.as<uint8_t>();
+  }
+  auto go = mixed(h) ? launch_dry<Mixed> : launch_dry<Fp64>;
+  const cudaError_t ce = go(h->prm.p, h->rec[0].as<uint4>(), b, n, h->einv.as<int32_t>() + b, to, h->stream);
+  if (ce != cudaSuccess) return fail(DGSWE_ECUDA, "dry flag launch: %s", cudaGetErrorString(ce));
+  h->launches++;
+  if (staged) CU(cudaMemcpyAsync(dry, to, (size_t)n, cudaMemcpyDeviceToHost, h->stream));
   CU(cudaStreamSynchronize(h->stream));
-  CU(cudaMemcpy(rec.data(), h->rec[0].p, 4 * rec.size(), cudaMemcpyDeviceToHost));
-  const int NS = h->np - 1;
-  const size_t off = mixed(h) ? (size_t)(6 + 3 * NS + 1) : (size_t)2 * (3 + 3 * NS + 1);
-  for (int e = 0; e < M.ne; ++e) dry[M.eorig[e]] = (rec_word(rec, e, off, h->rv) & FLAG_DRY) ? 1 : 0;
   return 0;
 }
 
 static int ledger_of(dgswe_h h, size_t s, dgswe_ledger* out) {
   DeviceGuard dg_(h->device);
-  CU(cudaStreamSynchronize(h->stream));
-  double V, VH;
-  if (int rc = reduce_volume(h, s, V, VH)) return rc;
-  (void)VH;
-  Ctl c;
-  CU(cudaMemcpy(&c, h->ctl.p, sizeof c, cudaMemcpyDeviceToHost));
-  std::vector<double> part(2 * (size_t)h->wcur);
-  CU(cudaMemcpy(part.data(), h->ledger.as<double>() + 2 * (size_t)s * h->wslots, 16 * (size_t)h->wcur,
-                cudaMemcpyDeviceToHost));
-  double rs = h->led_rain[s], rc_ = 0.0, bs = h->led_bdry[s], bc = 0.0;
-  auto neu = [](double& sum, double& comp, double v) {
-    const double t = sum + v;
-    comp += (std::fabs(sum) >= std::fabs(v)) ? (sum - t) + v : (v - t) + sum;
-    sum = t;
-  };
-  for (int w = 0; w < h->wcur; ++w) {
-    neu(rs, rc_, part[2 * w]);
-    neu(bs, bc, part[2 * w + 1]);
-  }
-  out->steps = (int64_t)c.step;
-  out->t = h->sc[s].t0 + (double)c.step * h->sc[s].dt;
+  if (int rc = summarise(h, s, false)) return rc;
+  const Summary& S = *h->sum;
+  out->steps = (int64_t)S.step;
+  out->t = h->sc[s].t0 + (double)S.step * h->sc[s].dt;
   out->V0 = h->V0[s];
-  out->V = V;
-  out->rain_in = rs + rc_;
-  out->bdry_in = bs + bc;
+  out->V = S.sum[0];
+  out->rain_in = h->led_rain[s] + S.sum[2];
+  out->bdry_in = h->led_bdry[s] + S.sum[3];
   out->VH0 = h->VH0[s];
-  out->rel_err = std::fabs(V - h->V0[s] - out->rain_in - out->bdry_in) / h->VH0[s];
-  // wet fraction from the dry flags
-  const HostMesh& M = h->sc[s].m;
-  const size_t rw = 4 * (size_t)h->rv;
-  std::vector<uint32_t> rec(rw * ((size_t)(M.ne + TILE - 1) / TILE * TILE));  // whole tiles
-  CU(cudaMemcpy(rec.data(), h->rec[0].as<uint32_t>() + rw * h->eoff[s], 4 * rec.size(), cudaMemcpyDeviceToHost));
-  const int NS = h->np - 1;
-  const size_t off = mixed(h) ? (size_t)(6 + 3 * NS + 1) : (size_t)2 * (3 + 3 * NS + 1);
-  long long wet = 0;
-  for (int e = 0; e < M.ne; ++e) wet += (rec_word(rec, e, off, h->rv) & FLAG_DRY) ? 0 : 1;
-  out->wet_frac = (double)wet / M.ne;
+  out->rel_err = std::fabs(out->V - h->V0[s] - out->rain_in - out->bdry_in) / h->VH0[s];
+  out->wet_frac = (double)S.wet / h->sc[s].m.ne;
   return 0;
 }
 
@@ -1595,8 +1539,9 @@ int dgswe_volume(dgswe_h h, double* out) {
   if (!h->ready) return fail(DGSWE_ESTATE, "no state");
   if (!out) return fail(DGSWE_EINVAL, "null output");
   DeviceGuard dg_(h->device);
-  double VH;
-  return reduce_volume(h, 0, *out, VH);
+  if (int rc = summarise(h, 0, false)) return rc;
+  *out = h->sum->sum[0];
+  return 0;
 }
 
 int dgswe_ensemble_create(dgswe_h* out, int32_t n, const dgswe_h* members, int device, void* stream) {

@@ -183,10 +183,21 @@ cudaError_t launch_node_rain(const StageArgs<Pol>& a, long long nn, cudaStream_t
 template <class Pol>
 cudaError_t launch_rain_records(const ScenDev* scen, int sc, const int4* nodes, const double* xy64, long long ne,
                                 long long stride, typename PolT<Pol>::T* rrec, cudaStream_t s);
-// partial FP64 sums of A*mean(zeta) and A*mean(H) over [begin, end): partials[4*block]
+// sums over a scenario, written by the device to page-locked host memory: compensated FP64 sums of
+// A mean(zeta), A mean(H) (0 unless asked for), ledger rain and boundary volumes; wet elements; steps
+struct Summary {
+  double sum[4];
+  long long wet;
+  unsigned long long step;
+};
 template <class Pol>
-cudaError_t launch_volume(int p, const uint4* rec, const uint4* geo, long long begin, long long end,
-                          double* partials, int nblk, cudaStream_t s);
+cudaError_t launch_summary(int p, bool depth, const uint4* rec, const uint4* geo, long long begin, long long end,
+                           const double* led, int nled, const Ctl* ctl, double* partials, unsigned* ticket, Summary* out,
+                           int nblk, cudaStream_t s);
+// wet/dry flags of [begin, begin + n) in caller order as 0/1 bytes
+template <class Pol>
+cudaError_t launch_dry(int p, const uint4* rec, long long begin, long long n, const int32_t* inv, uint8_t* out,
+                       cudaStream_t s);
 // per-block minimum of the CFL time step over [begin, end): partials[block]
 template <class Pol>
 cudaError_t launch_dt(int p, const uint4* rec, const int4* nodes, const double* xy64, const double* hb_nodal,
@@ -203,8 +214,5 @@ cudaError_t launch_gather(int p, const uint4* rec, long long begin, long long n,
 template <class Pol>
 cudaError_t launch_scatter(int p, uint4* rec, long long begin, long long n, const int32_t* inv, const double* z,
                            const double* x, const double* y, cudaStream_t s);
-
-// Neumaier-compensated reduction of per-block partial pairs (shared by all precisions)
-cudaError_t launch_reduce_pairs(const double* partials, int nblk, int npairs, double* out, cudaStream_t s);
 
 }  // namespace dg
