@@ -122,24 +122,10 @@ __device__ __forceinline__ ff acc_make<ff>(float hi, float lo, double) { return 
 __device__ __forceinline__ bool acc_finite(double a) { return isfinite(a); }
 __device__ __forceinline__ bool acc_finite(ff a) { return isfinite(a.hi) && isfinite(a.lo); }
 
-__device__ __forceinline__ float sqrt_r(float x) { return sqrtf(x); }
-__device__ __forceinline__ double sqrt_r(double x) { return sqrt(x); }
-__device__ __forceinline__ float rcp_r(float x) { return __frcp_rn(x); }
-__device__ __forceinline__ double rcp_r(double x) { return 1.0 / x; }
 __device__ __forceinline__ float abs_r(float x) { return fabsf(x); }
 __device__ __forceinline__ double abs_r(double x) { return fabs(x); }
 __device__ __forceinline__ float max_r(float a, float b) { return fmaxf(a, b); }
 __device__ __forceinline__ double max_r(double a, double b) { return fmax(a, b); }
-__device__ __forceinline__ float exp_r(float x) { return __expf(x); }
-__device__ __forceinline__ double exp_r(double x) { return exp(x); }
-__device__ __forceinline__ float sin_r(float x) { return sinf(x); }
-__device__ __forceinline__ double sin_r(double x) { return sin(x); }
-__device__ __forceinline__ float cos_r(float x) { return cosf(x); }
-__device__ __forceinline__ double cos_r(double x) { return cos(x); }
-// H^{4/3} as H * cbrt(H)
-__device__ __forceinline__ float pow43_r(float h) { return h * cbrtf(h); }
-__device__ __forceinline__ double pow43_r(double h) { return h * cbrt(h); }
-
 // FP32 path: single hardware (MUFU) instructions of the PTX ISA -- approximate to a few ulp,
 // deterministic, flushing subnormals to zero.  Every argument they get is a depth >= H0 > 0, a
 // wave speed, an edge length, a squared speed above 1e-30 or a bounded exponent, far from the
@@ -164,23 +150,70 @@ __device__ __forceinline__ float mufu_ex2(float x) {
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
+// FP64 path: its kernels are bound by the FP64 pipe (a warp instruction takes 16 cycles of an SM), so
+// what counts is the number of FP64 operations.  Reciprocal, inverse square root and inverse cube
+// root are one Householder step of second order (A. S. Householder, The Numerical Treatment of a
+// Single Nonlinear Equation, 1970) from a seed of about 20 bits: with e = 1 - x y^k the result is
+// y (1 - e)^(-1/k) expanded to e^2, whose remainder e^3 lies below 2^-57.  The seeds come from the PTX
+// ISA's approximate FP64 instructions (special-function unit) and, for the cube root, from FP32
+// special functions and integer operations on the exponent.  3, 5 and 6 FP64 operations; within 1, 2
+// and 2 ulp of the exact value for positive normal arguments (tests/test_gpu_fp64_functions.py).
+// FP64 coastal 61k: 845 -> 708 us per two steps (with the state read out) for these functions and the
+// fluxes and friction written on them.
+__device__ __forceinline__ double hh_rcp(double x) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-x, y, 1.0);
+  return fma(y, fma(e, e, e), y);
+}
+__device__ __forceinline__ double hh_rsqrt(double x) {
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  const double e = fma(-(x * y), y, 1.0);
+  return fma(y, e * fma(e, 0.375, 0.5), y);
+}
+__device__ __forceinline__ double hh_rcbrt(double x) {
+  const int hi = __double2hiint(x);
+  const unsigned lo = (unsigned)__double2loint(x);
+  const int ex = (hi >> 20) - 1023, q = (ex + 1023) / 3 - 341;  // x = 2^(3 q) m, m in [1, 8)
+  const float m = __int_as_float(((127 + ex - 3 * q) << 23) | ((hi & 0xfffff) << 3) | (int)(lo >> 29));
+  const int s = __float_as_int(mufu_ex2(mufu_lg2(m) * -0.33333334f));  // m^(-1/3) in [1/2, 1]
+  const double y = __hiloint2double((((s >> 23) + 896 - q) << 20) | ((s >> 3) & 0xfffff), s << 29);
+  const double y2 = y * y;
+  const double e = fma(-(x * y), y2, 1.0);
+  return fma(y, e * fma(e, 2.0 / 9.0, 1.0 / 3.0), y);
+}
 __device__ __forceinline__ float frcp(float x) { return mufu_rcp(x); }
-__device__ __forceinline__ double frcp(double x) { return 1.0 / x; }
-__device__ __forceinline__ float fdiv(float a, float b) { return a * mufu_rcp(b); }
-__device__ __forceinline__ double fdiv(double a, double b) { return a / b; }
+__device__ __forceinline__ double frcp(double x) { return hh_rcp(x); }
+__device__ __forceinline__ float frsqrt(float x) { return mufu_rsqrt(x); }  // x > 0
+__device__ __forceinline__ double frsqrt(double x) { return hh_rsqrt(x); }
 __device__ __forceinline__ float fsqrt_pos(float x) { return x * mufu_rsqrt(x); }  // x > 0
-__device__ __forceinline__ double fsqrt_pos(double x) { return sqrt(x); }
+__device__ __forceinline__ double fsqrt_pos(double x) { return x * hh_rsqrt(x); }
 // sqrt(x) for x >= 0 (a squared speed): zero below 1e-30, where the friction is negligible
 __device__ __forceinline__ float fsqrt0(float x) { return x > 1e-30f ? x * mufu_rsqrt(x) : 0.f; }
-__device__ __forceinline__ double fsqrt0(double x) { return sqrt(x); }
+__device__ __forceinline__ double fsqrt0(double x) { return x > 1e-290 ? x * hh_rsqrt(x) : 0.0; }
 // H^{-4/3} = 2^(-4/3 log2 H)
 __device__ __forceinline__ float fpowm43(float h) { return mufu_ex2(-1.3333333f * mufu_lg2(h)); }
-__device__ __forceinline__ double fpowm43(double h) { return 1.0 / (h * cbrt(h)); }
+// 1/H, and the depth factor of the friction law: H^{-4/3} (friction 0) or 1/H.  FP64 takes both from
+// one inverse cube root r (1/H = r^3 with a correction step, H^{-4/3} = r/H)
+__device__ __forceinline__ void depth_inverse(float h, int friction, float& i, float& f) {
+  i = frcp(h);
+  f = friction == 0 ? fpowm43(h) : i;
+}
+__device__ __forceinline__ void depth_inverse(double h, int friction, double& i, double& f) {
+  if (friction == 0) {
+    const double r = hh_rcbrt(h), c = r * r * r;
+    i = fma(fma(-h, c, 1.0), c, c);
+    f = i * r;
+  } else {
+    f = i = hh_rcp(h);
+  }
+}
 // e^x = 2^(x log2 e)
 __device__ __forceinline__ float fexp(float x) { return mufu_ex2(x * 1.4426950408889634f); }
 __device__ __forceinline__ double fexp(double x) { return exp(x); }
-__device__ __forceinline__ float fsin(float x) { return __sinf(x); }
-__device__ __forceinline__ double fsin(double x) { return sin(x); }
+__device__ __forceinline__ float fexp2(float x) { return mufu_ex2(x); }
+__device__ __forceinline__ double fexp2(double x) { return exp2(x); }
 
 // tidal elevation A sin(2 pi t / T + phi) of segment k at time t.  Mixed path: the phase is
 // formed and reduced to [-1/2, 1/2] turns in FP64 (ocean edges are few), the sine is the
@@ -472,73 +505,38 @@ __device__ __forceinline__ Trace<typename Pol::T> trace_p1(const Elem<1, Pol>& E
 template <int FLUX, class T>
 __device__ __forceinline__ void edge_flux(const Trace<T>& L, const Trace<T>& R, T dcRL, T nx, T ny, T g, T H0, T& fz,
                                           T& fx, T& fy) {
-  if constexpr (sizeof(T) == 4) {  // FP32: one reciprocal square root per side (as edge_flux_pair)
-    const float HsL = fmaxf(L.H, H0), HsR = fmaxf(R.H, H0);
-    const float rL = mufu_rsqrt(HsL), rR = mufu_rsqrt(HsR);
-    const float mL = L.qx * nx + L.qy * ny, mR = R.qx * nx + R.qy * ny;
-    const float unL = mL * (rL * rL), unR = mR * (rR * rR);
-    const float dz = (R.d - L.d) + dcRL;
-    const float dqx = R.qx - L.qx, dqy = R.qy - L.qy;
-    const float cx = 0.5f * (L.qx * unL + R.qx * unR);
-    const float cy = 0.5f * (L.qy * unL + R.qy * unR);
-    const float cz = 0.5f * (mL + mR);
-    const float sL = HsL * rL, sR = HsR * rR;
-    if (FLUX == 1) {
-      const float sg = fsqrt_pos(g);
-      const float lam = fmaxf(fabsf(unL) + sg * sL, fabsf(unR) + sg * sR);
-      fz = cz - 0.5f * lam * dz;
-      fx = cx - 0.5f * lam * dqx;
-      fy = cy - 0.5f * lam * dqy;
-      return;
-    }
-    const float is = frcp(sL + sR);
-    const float ut = (L.qx * rL + R.qx * rR) * is, vt = (L.qy * rL + R.qy * rR) * is;
-    const float c2 = 0.5f * g * (HsL + HsR);
-    const float ic = mufu_rsqrt(c2), c = c2 * ic;
-    const float utn = ut * nx + vt * ny, utt = vt * nx - ut * ny;
-    const float dqn = mR - mL, dqt = dqy * nx - dqx * ny;
-    const float w = (dqn - utn * dz) * ic;
-    const float a1 = 0.5f * (dz - w), a3 = 0.5f * (dz + w), a2 = dqt - utt * dz;
-    const float l1 = fabsf(utn - c) * a1, l2 = fabsf(utn) * a2, l3 = fabsf(utn + c) * a3;
-    fz = cz - 0.5f * (l1 + l3);
-    fx = cx - 0.5f * (l1 * (ut - c * nx) - l2 * ny + l3 * (ut + c * nx));
-    fy = cy - 0.5f * (l1 * (vt - c * ny) + l2 * nx + l3 * (vt + c * ny));
-    return;
-  }
-  T HsL = max_r(L.H, H0), HsR = max_r(R.H, H0);
-  T iL = frcp(HsL), iR = frcp(HsR);
-  T uL = L.qx * iL, vL = L.qy * iL, uR = R.qx * iR, vR = R.qy * iR;
-  T unL = uL * nx + vL * ny, unR = uR * nx + vR * ny;
-  T mL = L.qx * nx + L.qy * ny, mR = R.qx * nx + R.qy * ny;
-  T dz = (R.d - L.d) + dcRL;
-  T dqx = R.qx - L.qx, dqy = R.qy - L.qy;
-  T cx = T(0.5) * (L.qx * unL + R.qx * unR);
-  T cy = T(0.5) * (L.qy * unL + R.qy * unR);
-  T cz = T(0.5) * (mL + mR);
+  // one inverse square root per side (as edge_flux_pair)
+  const T HsL = max_r(L.H, H0), HsR = max_r(R.H, H0);
+  const T rL = frsqrt(HsL), rR = frsqrt(HsR);
+  const T mL = L.qx * nx + L.qy * ny, mR = R.qx * nx + R.qy * ny;
+  const T unL = mL * (rL * rL), unR = mR * (rR * rR);
+  const T dz = (R.d - L.d) + dcRL;
+  const T dqx = R.qx - L.qx, dqy = R.qy - L.qy;
+  const T cx = T(0.5) * (L.qx * unL + R.qx * unR);
+  const T cy = T(0.5) * (L.qy * unL + R.qy * unR);
+  const T cz = T(0.5) * (mL + mR);
+  const T sL = HsL * rL, sR = HsR * rR;
   if (FLUX == 1) {  // local Lax-Friedrichs
-    T lam = max_r(abs_r(unL) + fsqrt_pos(g * HsL), abs_r(unR) + fsqrt_pos(g * HsR));
+    const T sg = fsqrt_pos(g);
+    const T lam = max_r(abs_r(unL) + sg * sL, abs_r(unR) + sg * sR);
     fz = cz - T(0.5) * lam * dz;
     fx = cx - T(0.5) * lam * dqx;
     fy = cy - T(0.5) * lam * dqy;
     return;
   }
   // Roe: averages (arithmetic depth, sqrt-depth-weighted velocity), eigen-decomposition
-  T sL = fsqrt_pos(HsL), sR = fsqrt_pos(HsR);
-  T is = frcp(sL + sR);
-  T ut = (sL * uL + sR * uR) * is, vt = (sL * vL + sR * vR) * is;
-  T c = fsqrt_pos(g * T(0.5) * (HsL + HsR));
-  T ic = frcp(c);
-  T utn = ut * nx + vt * ny, utt = vt * nx - ut * ny;
-  T dqn = dqx * nx + dqy * ny, dqt = dqy * nx - dqx * ny;
-  T w = (dqn - utn * dz) * ic;
-  T a1 = T(0.5) * (dz - w), a3 = T(0.5) * (dz + w), a2 = dqt - utt * dz;
-  T l1 = abs_r(utn - c) * a1, l2 = abs_r(utn) * a2, l3 = abs_r(utn + c) * a3;
-  T D0 = l1 + l3;
-  T D1 = l1 * (ut - c * nx) - l2 * ny + l3 * (ut + c * nx);
-  T D2 = l1 * (vt - c * ny) + l2 * nx + l3 * (vt + c * ny);
-  fz = cz - T(0.5) * D0;
-  fx = cx - T(0.5) * D1;
-  fy = cy - T(0.5) * D2;
+  const T is = frcp(sL + sR);
+  const T ut = (L.qx * rL + R.qx * rR) * is, vt = (L.qy * rL + R.qy * rR) * is;
+  const T c2 = T(0.5) * g * (HsL + HsR);
+  const T ic = frsqrt(c2), c = c2 * ic;
+  const T utn = ut * nx + vt * ny, utt = vt * nx - ut * ny;
+  const T dqn = mR - mL, dqt = dqy * nx - dqx * ny;
+  const T w = (dqn - utn * dz) * ic;
+  const T a1 = T(0.5) * (dz - w), a3 = T(0.5) * (dz + w), a2 = dqt - utt * dz;
+  const T l1 = abs_r(utn - c) * a1, l2 = abs_r(utn) * a2, l3 = abs_r(utn + c) * a3;
+  fz = cz - T(0.5) * (l1 + l3);
+  fx = cx - T(0.5) * (l1 * (ut - c * nx) - l2 * ny + l3 * (ut + c * nx));
+  fy = cy - T(0.5) * (l1 * (vt - c * ny) + l2 * nx + l3 * (vt + c * ny));
 }
 
 #ifndef DG_PACKED_FLUX
@@ -1033,8 +1031,7 @@ __global__ void __launch_bounds__(256) edge_kernel(const StageArgs<Pol> a) {
     Elem<P, Pol> L, R;
     unpack<P>(rl, L);
     unpack<P>(rr, R);
-    const T len = fsqrt_pos(lnx * lnx + lny * lny);
-    const T il = frcp(len);
+    const T l2 = lnx * lnx + lny * lny, il = frsqrt(l2), len = l2 * il;
     const T nx = lnx * il, ny = lny * il;
     const T dcRL = acc_diff(R.zb, L.zb);
     Trace<T> tl[NG], tr[NG];
@@ -1535,12 +1532,12 @@ __global__ void DG_STAGE_BOUNDS stage_kernel(const StageArgs<Pol> a) {
     for (int q = q0; q < NQ; ++q) {
       const Trace<T> tq = trace_at<P, Pol>(E, tab.qphi[q]);
       const T Hs = max_r(tq.H, H0);
-      const T iH = frcp(Hs);
+      T iH, hf;
+      depth_inverse(Hs, a.friction, iH, hf);
       const T u = tq.qx * iH, v = tq.qy * iH;
       const T pp = pdev(tq.d, tq.H, g);
       T tau = 0;
-      if (a.friction == 0) tau = cfm * fsqrt0(u * u + v * v) * fpowm43(Hs);
-      else if (a.friction == 1) tau = cfm * fsqrt0(u * u + v * v) * iH;
+      if (a.friction <= 1) tau = cfm * fsqrt0(u * u + v * v) * hf;
       T Fxs = 0, Fys = 0;
       if (S.press) {
         const T px = tab.ql[q][0] * vx[0] + tab.ql[q][1] * vx[1] + tab.ql[q][2] * vx[2];
@@ -1605,8 +1602,8 @@ __global__ void DG_STAGE_BOUNDS stage_kernel(const StageArgs<Pol> a) {
           const T tt = t - F.storm[7];
           const T dx = px - (F.storm[0] + F.storm[2] * tt), dy = py - (F.storm[1] + F.storm[3] * tt);
           const T r = fsqrt0(dx * dx + dy * dy);
-          const T rp = F.storm[4], rm = F.storm[5], re = F.storm[6];
-          acc += (r < rm) ? rp * (T(0.5) + T(0.5) * fdiv(r, rm)) : rp * fexp(-fdiv(r - rm, re));
+          const T rp = F.storm[4], rm = F.storm[5];
+          acc += (r < rm) ? rp * (T(0.5) + T(0.5) * (r * F.storm[8])) : rp * fexp2((rm - r) * F.storm[9]);
         }
       } else if (S.rrec) {  // gridded: the element's records, blended in time
         const RainRec<T> rr = rain_records<T>(S, S.d.t0 + stepd * S.d.dt);
@@ -1644,8 +1641,7 @@ __global__ void DG_STAGE_BOUNDS stage_kernel(const StageArgs<Pol> a) {
         }
         wall = true;  // closed by the wet/dry rule: my own wall flux below
       }
-      const T len = fsqrt_pos(lnx * lnx + lny * lny);
-      const T il = frcp(len);
+      const T l2 = lnx * lnx + lny * lny, il = frsqrt(l2), len = l2 * il;
       const T nx = lnx * il, ny = lny * il;
       Trace<T> tm[NG], to[NG];  // my trace and the other side's, at my edge points
 #pragma unroll

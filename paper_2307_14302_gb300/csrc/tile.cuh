@@ -213,23 +213,28 @@ __device__ __forceinline__ f2 vrcp(f2 a) { return rcp2(a); }
 __device__ __forceinline__ float vsqrt0(float a) { return fsqrt0(a); }
 __device__ __forceinline__ double vsqrt0(double a) { return fsqrt0(a); }
 __device__ __forceinline__ f2 vsqrt0(f2 a) { return make_float2(fsqrt0(a.x), fsqrt0(a.y)); }
-__device__ __forceinline__ float vpowm43(float a) { return fpowm43(a); }
-__device__ __forceinline__ double vpowm43(double a) { return fpowm43(a); }
-__device__ __forceinline__ f2 vpowm43(f2 a) { return make_float2(fpowm43(a.x), fpowm43(a.y)); }
 // friction coefficient tau (source -tau q): Manning g n^2 |u| / Hs^(4/3) (friction 0) or
 // cf |u| / Hs (friction 1).  In FP32 as cfm 2^(lg2|q|^2 / 2 - c lg2 Hs) with c = 7/3 or 2, three
-// special-function operations and no square root (|q| = 0 gives 2^-inf = 0).
+// special-function operations and no square root (|q| = 0 gives 2^-inf = 0); in FP64 from the depth
+// factor hf of vdepth.
 __device__ __forceinline__ float vtau(float qx, float qy, float, float, float Hs, float, float cfm, int friction) {
   const float c = friction == 0 ? 2.3333333f : 2.0f;
   return cfm * mufu_ex2(fmaf(0.5f, mufu_lg2(fmaf(qx, qx, qy * qy)), -c * mufu_lg2(Hs)));
 }
-__device__ __forceinline__ f2 vtau(f2 qx, f2 qy, f2 u, f2 v, f2 Hs, f2 iH, f2 cfm, int friction) {
-  return make_float2(vtau(qx.x, qy.x, u.x, v.x, Hs.x, iH.x, cfm.x, friction),
-                     vtau(qx.y, qy.y, u.y, v.y, Hs.y, iH.y, cfm.y, friction));
+__device__ __forceinline__ f2 vtau(f2 qx, f2 qy, f2 u, f2 v, f2 Hs, f2 hf, f2 cfm, int friction) {
+  return make_float2(vtau(qx.x, qy.x, u.x, v.x, Hs.x, hf.x, cfm.x, friction),
+                     vtau(qx.y, qy.y, u.y, v.y, Hs.y, hf.y, cfm.y, friction));
 }
-__device__ __forceinline__ double vtau(double, double, double u, double v, double Hs, double iH, double cfm,
-                                       int friction) {
-  return cfm * (fsqrt0(fma(u, u, v * v)) * (friction == 0 ? fpowm43(Hs) : iH));
+__device__ __forceinline__ double vtau(double, double, double u, double v, double, double hf, double cfm, int) {
+  return cfm * (fsqrt0(fma(u, u, v * v)) * hf);
+}
+// 1/Hs and, in FP64, the friction law's depth factor
+__device__ __forceinline__ float vdepth(float Hs, int, float&) { return vrcp(Hs); }
+__device__ __forceinline__ f2 vdepth(f2 Hs, int, f2&) { return vrcp(Hs); }
+__device__ __forceinline__ double vdepth(double Hs, int friction, double& hf) {
+  double i;
+  depth_inverse(Hs, friction, i, hf);
+  return i;
 }
 template <class V>
 __device__ __forceinline__ V vbc(float x);
@@ -271,11 +276,12 @@ __device__ __forceinline__ void area_points_p1(AreaP1<V>& A, const RefTab<T>& ta
   const V hdev = vfma(hb1, ph1, vmul(hb2, ph2));
   const V H = vadd(Hb, vadd(d, hdev));
   const V Hs = vmax(H, H0v);
-  const V iH = vrcp(Hs);
+  V hf = vbc<V>(0.f);
+  const V iH = vdepth(Hs, friction, hf);
   const V u = vmul(qx, iH), v = vmul(qy, iH);
   const V pp = vmul(vmul(hg, d), vfma(vbc<V>(2.f), H, vneg(d)));  // g/2 d (2H - d)
   V tau = vbc<V>(0.f);
-  if (friction <= 1) tau = vtau(qx, qy, u, v, Hs, iH, cfm, friction);
+  if (friction <= 1) tau = vtau(qx, qy, u, v, Hs, hf, cfm, friction);
   const V sx = vfma(ghbx, d, vfma(vneg(tau), qx, Fxs));
   const V sy = vfma(ghby, d, vfma(vneg(tau), qy, Fys));
   const V w = vtab<V, T>(tab.qwT, q);
@@ -425,7 +431,7 @@ __device__ __forceinline__ void tile_area(const Elem<P, Pol>& E, const Geo<Pol>&
       const f2 u = mul2(qx, iH), v = mul2(qy, iH);
       const f2 pp = mul2(mul2(hg, d), fma2(p2(2.f), H, neg2(d)));  // g/2 d (2H - d)
       f2 tau = p2(0.f);
-      if (friction <= 1) tau = vtau(qx, qy, u, v, Hs, iH, cfm2, friction);
+      if (friction <= 1) tau = vtau(qx, qy, u, v, Hs, p2(0.f), cfm2, friction);
       float Fx0 = 0.f, Fy0 = 0.f, Fx1 = 0.f, Fy1 = 0.f;
       if (press) {
 #pragma unroll
@@ -467,11 +473,12 @@ __device__ __forceinline__ void tile_area(const Elem<P, Pol>& E, const Geo<Pol>&
     for (int q = 0; q < NQ; ++q) {
       const Trace<T> tq = trace_at<P, Pol>(E, tab.qphi[q]);
       const T Hs = max_r(tq.H, H0);
-      const T iH = frcp(Hs);
+      T hf = T(0);
+      const T iH = vdepth(Hs, friction, hf);
       const T u = tq.qx * iH, v = tq.qy * iH;
       const T pp = pdev(tq.d, tq.H, g);
       T tau = 0;
-      if (friction <= 1) tau = vtau(tq.qx, tq.qy, u, v, Hs, iH, cfm, friction);
+      if (friction <= 1) tau = vtau(tq.qx, tq.qy, u, v, Hs, hf, cfm, friction);
       T Fxs = 0, Fys = 0;
       if (press) {
         const T px = tab.ql[q][0] * vx[0] + tab.ql[q][1] * vx[1] + tab.ql[q][2] * vx[2];
@@ -581,8 +588,8 @@ template <int FLUX, class T>
 __device__ __forceinline__ T wall_coef(const Trace<T>& t, T nx, T ny, T g, T H0) {
   const T qn = t.qx * nx + t.qy * ny;
   const T Hs = max_r(t.H, H0);
-  const T iH = frcp(Hs);
-  const T c = fsqrt_pos(g * Hs);
+  const T r = frsqrt(Hs), iH = r * r;
+  const T c = fsqrt_pos(g) * (Hs * r);
   const T un = (FLUX == 1) ? (qn + abs_r(qn)) * iH : qn * iH;
   return qn * (un + c) + pdev(t.d, t.H, g);
 }
@@ -612,15 +619,7 @@ __device__ __forceinline__ void tile_edge(const StageArgs<Pol>& a, const ScenDev
   }
   Elem<P, Pol> EL;
   unpack<P>(rl, EL);
-  T len, il;  // edge length and its inverse
-  if constexpr (sizeof(T) == 4) {
-    const T l2 = lnx * lnx + lny * lny;
-    il = mufu_rsqrt(l2);
-    len = l2 * il;
-  } else {
-    len = fsqrt_pos(lnx * lnx + lny * lny);
-    il = frcp(len);
-  }
+  const T l2 = lnx * lnx + lny * lny, il = frsqrt(l2), len = l2 * il;  // edge length and its inverse
   const T nx = lnx * il, ny = lny * il;
   constexpr bool P1F = P == 1 && sizeof(T) == 4;  // basis values of both points in one 16-byte read
   Trace<T> tl[NG], tr[NG];
@@ -951,16 +950,14 @@ __device__ __forceinline__ void tile_body(const StageArgs<Pol>& a, const ScenDev
       const ForcingT<T>& F = forcing<T>(S);
       const T tt = t - F.storm[7];
       const T cx = F.storm[0] + F.storm[2] * tt, cy = F.storm[1] + F.storm[3] * tt;
-      const T rp = F.storm[4], rm = F.storm[5], re = F.storm[6];
+      const T rp = F.storm[4], rm = F.storm[5];
       T acc = 0;
 #pragma unroll
       for (int i = 0; i < 3; ++i) {
         const T dx = vx[i] - cx, dy = vy[i] - cy;
         const T r = fsqrt0(dx * dx + dy * dy);
-        if constexpr (sizeof(T) == 4)  // with 1 / rm and log2(e) / re formed once on the host
-          acc += (r < rm) ? rp * fmaf(0.5f * F.storm[8], r, 0.5f) : rp * mufu_ex2((rm - r) * F.storm[9]);
-        else
-          acc += (r < rm) ? rp * (T(0.5) + T(0.5) * fdiv(r, rm)) : rp * fexp(-fdiv(r - rm, re));
+        // with 1 / rm and log2(e) / re formed once on the host
+        acc += (r < rm) ? rp * fma(T(0.5) * F.storm[8], r, T(0.5)) : rp * fexp2((rm - r) * F.storm[9]);
       }
       Re = acc * T(1.0 / 3.0);
     } else if (rain_kind == 3 && rr.r0) {
