@@ -73,6 +73,7 @@ struct RefTab {
   T qwphiT[MAXNP][MAXNQP];         // qw[q] * qphi[q][m], same order
   T qdrT[MAXNP][MAXNQP];           // qdr transposed
   T qdsT[MAXNP][MAXNQP];           // qds transposed
+  T vmw[3][4][2];                  // p = 1: vertex k and the midpoint opposite it: weight, weight * phi_m
 };
 
 // per-scenario forcing constants in the arithmetic type of a path

@@ -189,8 +189,8 @@ __device__ __forceinline__ float frsqrt(float x) { return mufu_rsqrt(x); }  // x
 __device__ __forceinline__ double frsqrt(double x) { return hh_rsqrt(x); }
 __device__ __forceinline__ float fsqrt_pos(float x) { return x * mufu_rsqrt(x); }  // x > 0
 __device__ __forceinline__ double fsqrt_pos(double x) { return x * hh_rsqrt(x); }
-// sqrt(x) for x >= 0 (a squared speed): zero below 1e-30, where the friction is negligible
-__device__ __forceinline__ float fsqrt0(float x) { return x > 1e-30f ? x * mufu_rsqrt(x) : 0.f; }
+// sqrt(x) for x >= 0 (a squared speed or distance): below 1e-30, where it is negligible, at most 1e-15
+__device__ __forceinline__ float fsqrt0(float x) { return x * mufu_rsqrt(fmaxf(x, 1e-30f)); }
 __device__ __forceinline__ double fsqrt0(double x) { return x > 1e-290 ? x * hh_rsqrt(x) : 0.0; }
 // H^{-4/3} = 2^(-4/3 log2 H)
 __device__ __forceinline__ float fpowm43(float h) { return mufu_ex2(-1.3333333f * mufu_lg2(h)); }
@@ -739,7 +739,16 @@ __device__ __forceinline__ void apply_positivity(Elem<P, Pol>& E, const Geo<Pol>
   const T Hb = acc_sum_r(E.zb, G.hbm);  // mean depth
   constexpr int NL = NS < 2 ? NS : 2;  // linear modes among zs
   bool need64 = true, dry = false;
+  // bound on the magnitudes summed at any vertex: |Hb| + sum_m (|zs_m| + |hb_m|) max_i |phi_m(x_i)|
+  T bound = T(0), tol = T(0);
   if (sizeof(T) == 4) {
+    bound = (abs_r(E.hb1) + abs_r(E.zs[0])) * tab.vabs[1];
+    if (NL > 1) bound = fma(abs_r(E.hb2) + abs_r(E.zs[NL > 1 ? 1 : 0]), tab.vabs[2], bound);
+    tol = T(4.0e-6) * (abs_r(Hb) + bound);
+    // deep water: the bound alone keeps every vertex clear of the threshold (and of the blend of p = 2)
+    need64 = !((Hb - bound) - tol > (P >= 2 ? T(2) * H0 : H0));
+  }
+  if (sizeof(T) == 4 && need64) {
     T hv[3];
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
@@ -749,11 +758,7 @@ __device__ __forceinline__ void apply_positivity(Elem<P, Pol>& E, const Geo<Pol>
       v = fma(E.hb1, tab.vphi[i][1], v);
       hv[i] = fma(E.hb2, tab.vphi[i][2], v);
     }
-    // bound on the magnitudes summed at any vertex: |Hb| + sum_m (|zs_m| + |hb_m|) max_i |phi_m(x_i)|
-    T bound = (abs_r(E.hb1) + abs_r(E.zs[0])) * tab.vabs[1];
-    if (NL > 1) bound = fma(abs_r(E.hb2) + abs_r(E.zs[NL > 1 ? 1 : 0]), tab.vabs[2], bound);
     const T hmin = fminf(hv[0], fminf(hv[1], hv[2]));
-    const T tol = T(4.0e-6) * (abs_r(Hb) + bound);
     // mean depth clearly above H0: the element is wet whatever its vertices; a vertex depth within
     // tol of H0 then decides only whether a redistribution smaller than tol (below the FP32
     // resolution of the vertex depths) is made, and FP32 decides it

@@ -141,9 +141,11 @@ __global__ void __maxnreg__(sizeof(typename Pol::T) == 4 ? (P == 1 ? 128 : 200) 
         rr.r0 -= S.elem_begin;
         rr.r1 -= S.elem_begin;
       }
+      Storm<T> storm = {};
+      if constexpr (storm_regs<P, FT>()) storm = storm_at<T>(S, t64);
       Acc rain_acc = acc_make<Acc>(0.f, 0.f, 0.0), bdry_acc = acc_make<Acc>(0.f, 0.f, 0.0);
       Elem<P, Pol> O;
-      tile_body<P, FLUX, Pol, FT, true>(a, S, t64, rain_kind, press, rr, tile, lane, valid, meta.z,
+      tile_body<P, FLUX, Pol, FT, true>(a, S, t64, rain_kind, press, rr, storm, tile, lane, valid, meta.z,
                                         Wm + SL::REC + c.in * SL::RECS, halo, Wm + SL::GEO,
                                         reinterpret_cast<const unsigned*>(Wm + SL::PLAN),
                                         reinterpret_cast<const float*>(Wm + L::S_MAN),

@@ -173,6 +173,13 @@ void build_tables(int p, RefTab<double>& t) {
   for (int q = 0; q < t.nq; ++q) t.qwT[q] = t.qw[q];
   for (int m = 0; m < t.np; ++m)
     for (int i = 0; i < 3; ++i) t.vabs[m] = std::max(t.vabs[m], std::fabs(t.vphi[i][m]));
+  if (p == 1)
+    for (int k = 0; k < 3; ++k)
+      for (int i = 0; i < 2; ++i) {
+        const int q = (i == 0 ? 4 : 1) + k;
+        t.vmw[k][0][i] = t.qw[q];
+        for (int m = 0; m < 3; ++m) t.vmw[k][m + 1][i] = t.qw[q] * t.qphi[q][m];
+      }
   for (int m = 0; m < t.np; ++m)
     for (int q = 0; q < t.nq; ++q) {
       t.qphiT[m][q] = t.qphi[q][m];

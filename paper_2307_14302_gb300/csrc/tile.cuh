@@ -222,8 +222,10 @@ __device__ __forceinline__ float vtau(float qx, float qy, float, float, float Hs
   return cfm * mufu_ex2(fmaf(0.5f, mufu_lg2(fmaf(qx, qx, qy * qy)), -c * mufu_lg2(Hs)));
 }
 __device__ __forceinline__ f2 vtau(f2 qx, f2 qy, f2 u, f2 v, f2 Hs, f2 hf, f2 cfm, int friction) {
-  return make_float2(vtau(qx.x, qy.x, u.x, v.x, Hs.x, hf.x, cfm.x, friction),
-                     vtau(qx.y, qy.y, u.y, v.y, Hs.y, hf.y, cfm.y, friction));
+  const f2 q2 = fma2(qx, qx, mul2(qy, qy));
+  const f2 lq = make_float2(mufu_lg2(q2.x), mufu_lg2(q2.y)), lh = make_float2(mufu_lg2(Hs.x), mufu_lg2(Hs.y));
+  const f2 x = fma2(p2(0.5f), lq, mul2(p2(friction == 0 ? -2.3333333f : -2.0f), lh));
+  return mul2(cfm, make_float2(mufu_ex2(x.x), mufu_ex2(x.y)));
 }
 __device__ __forceinline__ double vtau(double, double, double u, double v, double, double hf, double cfm, int) {
   return cfm * (fsqrt0(fma(u, u, v * v)) * hf);
@@ -257,45 +259,67 @@ __device__ __forceinline__ f2 vtab<f2, float>(const float* row, int q) { return 
 
 // ------------------------------------------------------------------------ area (p = 1) ---
 // Degree-1 elements have constant basis gradients: the flux terms need only the weighted sums of
-// F over the points (SF), the sources their moments against each basis function (SS).
+// F over the points (SF), the sources their moments against each basis function (SS).  q_x v = q_y u, so
+// the two cross terms are one sum.  The degree-3 rule's points are the centroid (0), the edge midpoints
+// opposite vertex k (1 + k) and the vertices (4 + k): a linear field takes its mean at the centroid,
+// three sums at the vertices and one operation per midpoint (3/2 mean - 1/2 vertex k), instead of two
+// products per field and point with table values.  The pairs (vertex k, midpoint k) are evaluated
+// together in packed FP32x2, the centroid alone with what vanishes there left out.
 template <class V>
 struct AreaP1 {
-  V SF[6];     // sum_q w_q (Fx_z, Fx_x, Fx_y, Fy_z, Fy_x, Fy_y)
+  V SF[5];     // sum_q w_q (q_x, q_x u + p, q_y u, q_y, q_y v + p)
   V SS[3][2];  // sum_q w_q phi_m (s_x, s_y)
 };
 
-template <class V, class T>
-__device__ __forceinline__ void area_points_p1(AreaP1<V>& A, const RefTab<T>& tab, int q, V zs0, V zs1, V xs0,
-                                               V xs1, V ys0, V ys1, V xb, V yb, V Hb, V hb1, V hb2, V H0v, V hg,
-                                               V ghbx, V ghby, V cfm, int friction, V Fxs, V Fys) {
-  const V ph1 = vtab<V, T>(tab.qphiT[1], q), ph2 = vtab<V, T>(tab.qphiT[2], q);
-  // trace at the point(s): d = zeta - mean(zeta), H, qx, qy (same operation order as trace_at)
-  const V d = vfma(zs1, ph2, vmul(zs0, ph1));
-  const V qx = vfma(xs1, ph2, vfma(xs0, ph1, xb));
-  const V qy = vfma(ys1, ph2, vfma(ys0, ph1, yb));
-  const V hdev = vfma(hb1, ph1, vmul(hb2, ph2));
-  const V H = vadd(Hb, vadd(d, hdev));
+// values at the vertices v and at the midpoints m opposite them of the field with mean c and modes
+// a, b (phi_1 = sqrt(3) (-1, 1, 0), phi_2 = (-1, -1, 2) at the vertices)
+template <class T>
+__device__ __forceinline__ void tri_points(T c, T a, T b, T v[3], T m[3]) {
+  const T t = T(1.7320508075688772) * a, s = c - b, h = T(1.5) * c;
+  v[0] = s - t;
+  v[1] = s + t;
+  v[2] = fma(T(2), b, c);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) m[k] = fma(T(-0.5), v[k], h);
+}
+template <int K>
+struct IntC {
+  static constexpr int value = K;
+};
+
+// one point or pair: w and wp are its weight and weight times phi_m; CEN: the centroid (d = 0, phi_1 =
+// phi_2 = 0); K: the vertex of the pair, where phi_1 vanishes at K = 2
+template <bool CEN, int K, class V>
+__device__ __forceinline__ void area_point_p1(AreaP1<V>& A, V d, V H, V qx, V qy, V w, const V wp[3], V H0v, V hg, V ghbx,
+                                              V ghby, V cfm, int friction, V Fxs, V Fys) {
   const V Hs = vmax(H, H0v);
   V hf = vbc<V>(0.f);
   const V iH = vdepth(Hs, friction, hf);
   const V u = vmul(qx, iH), v = vmul(qy, iH);
-  const V pp = vmul(vmul(hg, d), vfma(vbc<V>(2.f), H, vneg(d)));  // g/2 d (2H - d)
   V tau = vbc<V>(0.f);
   if (friction <= 1) tau = vtau(qx, qy, u, v, Hs, hf, cfm, friction);
-  const V sx = vfma(ghbx, d, vfma(vneg(tau), qx, Fxs));
-  const V sy = vfma(ghby, d, vfma(vneg(tau), qy, Fys));
-  const V w = vtab<V, T>(tab.qwT, q);
+  V sx = vfma(vneg(tau), qx, Fxs), sy = vfma(vneg(tau), qy, Fys);
+  V fxx, fyy;
+  if (CEN) {
+    fxx = vmul(qx, u);
+    fyy = vmul(qy, v);
+  } else {
+    const V pp = vmul(vmul(hg, d), vfma(vbc<V>(2.f), H, vneg(d)));  // g/2 d (2H - d)
+    sx = vfma(ghbx, d, sx);
+    sy = vfma(ghby, d, sy);
+    fxx = vfma(qx, u, pp);
+    fyy = vfma(qy, v, pp);
+  }
   A.SF[0] = vfma(w, qx, A.SF[0]);
-  A.SF[1] = vfma(w, vfma(qx, u, pp), A.SF[1]);
+  A.SF[1] = vfma(w, fxx, A.SF[1]);
   A.SF[2] = vfma(w, vmul(qy, u), A.SF[2]);
   A.SF[3] = vfma(w, qy, A.SF[3]);
-  A.SF[4] = vfma(w, vmul(qx, v), A.SF[4]);
-  A.SF[5] = vfma(w, vfma(qy, v, pp), A.SF[5]);
+  A.SF[4] = vfma(w, fyy, A.SF[4]);
 #pragma unroll
   for (int m = 0; m < 3; ++m) {
-    const V wp = vtab<V, T>(tab.qwphiT[m], q);
-    A.SS[m][0] = vfma(wp, sx, A.SS[m][0]);
-    A.SS[m][1] = vfma(wp, sy, A.SS[m][1]);
+    if ((CEN && m > 0) || (K == 2 && m == 1)) continue;
+    A.SS[m][0] = vfma(wp[m], sx, A.SS[m][0]);
+    A.SS[m][1] = vfma(wp[m], sy, A.SS[m][1]);
   }
 }
 
@@ -347,49 +371,65 @@ __device__ __forceinline__ void tile_area(const Elem<P, Pol>& E, const Geo<Pol>&
         setup_force<T>(F, px, py, Hq, g, Fx[q], Fy[q]);
       }
     }
-    T SF[6], SS[3][2];
+    T dv[3], dm[3], Hv[3], Hm[3], xv[3], xm[3], yv[3], ym[3];
+    tri_points<T>(T(0), E.zs[0], E.zs[1], dv, dm);
+    tri_points<T>(E.Hb, E.zs[0] + E.hb1, E.zs[1] + E.hb2, Hv, Hm);
+    tri_points<T>(xb, E.xs[0], E.xs[1], xv, xm);
+    tri_points<T>(yb, E.ys[0], E.ys[1], yv, ym);
+    const T hg = T(0.5) * g, ghbx = g * hbx, ghby = g * hby;
+    T SF[5], SS[3][2];
+    AreaP1<T> A1;
+#pragma unroll
+    for (int i = 0; i < 5; ++i) A1.SF[i] = T(0);
+#pragma unroll
+    for (int m = 0; m < 3; ++m) A1.SS[m][0] = A1.SS[m][1] = T(0);
+    {
+      const T wp[3] = {tab.qwphiT[0][0], T(0), T(0)};
+      area_point_p1<true, 0, T>(A1, T(0), E.Hb, xb, yb, tab.qwT[0], wp, H0, hg, ghbx, ghby, cfm, friction, Fx[0], Fy[0]);
+    }
     if constexpr (sizeof(T) == 4 && DG_PACKED_FLUX) {
-      // points (0,1), (2,3), (4,5) in packed pairs, point 6 alone
       AreaP1<f2> A2;
 #pragma unroll
-      for (int i = 0; i < 6; ++i) A2.SF[i] = p2(0.f);
+      for (int i = 0; i < 5; ++i) A2.SF[i] = p2(0.f);
 #pragma unroll
       for (int m = 0; m < 3; ++m) A2.SS[m][0] = A2.SS[m][1] = p2(0.f);
-      const f2 zs0 = p2(E.zs[0]), zs1 = p2(E.zs[1]), xs0 = p2(E.xs[0]), xs1 = p2(E.xs[1]);
-      const f2 ys0 = p2(E.ys[0]), ys1 = p2(E.ys[1]), xb2 = p2(xb), yb2 = p2(yb), Hb2 = p2(E.Hb);
-      const f2 hb12 = p2(E.hb1), hb22 = p2(E.hb2), H02 = p2(H0), hg2 = p2(0.5f * g);
-      const f2 ghbx2 = p2(g * hbx), ghby2 = p2(g * hby), cfm2 = p2(cfm);
+      const f2 H02 = p2(H0), hg2 = p2(hg), gx2 = p2(ghbx), gy2 = p2(ghby), cfm2 = p2(cfm);
+      auto pair = [&](auto kc) {
+        constexpr int k = decltype(kc)::value;
+        const f2 wp[3] = {make_float2(tab.vmw[k][1][0], tab.vmw[k][1][1]), make_float2(tab.vmw[k][2][0], tab.vmw[k][2][1]),
+                          make_float2(tab.vmw[k][3][0], tab.vmw[k][3][1])};
+        area_point_p1<false, k, f2>(A2, make_float2(dv[k], dm[k]), make_float2(Hv[k], Hm[k]), make_float2(xv[k], xm[k]),
+                                    make_float2(yv[k], ym[k]), make_float2(tab.vmw[k][0][0], tab.vmw[k][0][1]), wp, H02, hg2,
+                                    gx2, gy2, cfm2, friction, make_float2(Fx[4 + k], Fx[1 + k]),
+                                    make_float2(Fy[4 + k], Fy[1 + k]));
+      };
+      pair(IntC<0>());
+      pair(IntC<1>());
+      pair(IntC<2>());
 #pragma unroll
-      for (int q = 0; q < 6; q += 2)
-        area_points_p1<f2, float>(A2, tab, q, zs0, zs1, xs0, xs1, ys0, ys1, xb2, yb2, Hb2, hb12, hb22, H02, hg2,
-                                  ghbx2, ghby2, cfm2, friction, make_float2(Fx[q], Fx[q + 1]),
-                                  make_float2(Fy[q], Fy[q + 1]));
-      AreaP1<float> A1;
+      for (int i = 0; i < 5; ++i) SF[i] = (A2.SF[i].x + A2.SF[i].y) + A1.SF[i];
+      SS[0][0] = (A2.SS[0][0].x + A2.SS[0][0].y) + A1.SS[0][0];
+      SS[0][1] = (A2.SS[0][1].x + A2.SS[0][1].y) + A1.SS[0][1];
 #pragma unroll
-      for (int i = 0; i < 6; ++i) A1.SF[i] = 0.f;
-#pragma unroll
-      for (int m = 0; m < 3; ++m) A1.SS[m][0] = A1.SS[m][1] = 0.f;
-      area_points_p1<float, float>(A1, tab, 6, E.zs[0], E.zs[1], E.xs[0], E.xs[1], E.ys[0], E.ys[1], xb, yb, E.Hb,
-                                   E.hb1, E.hb2, H0, 0.5f * g, g * hbx, g * hby, cfm, friction, Fx[6], Fy[6]);
-#pragma unroll
-      for (int i = 0; i < 6; ++i) SF[i] = (A2.SF[i].x + A2.SF[i].y) + A1.SF[i];
-#pragma unroll
-      for (int m = 0; m < 3; ++m) {
-        SS[m][0] = (A2.SS[m][0].x + A2.SS[m][0].y) + A1.SS[m][0];
-        SS[m][1] = (A2.SS[m][1].x + A2.SS[m][1].y) + A1.SS[m][1];
+      for (int m = 1; m < 3; ++m) {
+        SS[m][0] = A2.SS[m][0].x + A2.SS[m][0].y;
+        SS[m][1] = A2.SS[m][1].x + A2.SS[m][1].y;
       }
     } else {
-      AreaP1<T> A1;
+      auto both = [&](auto kc) {
+        constexpr int k = decltype(kc)::value;
+        const T wv[3] = {tab.vmw[k][1][0], tab.vmw[k][2][0], tab.vmw[k][3][0]};
+        const T wm[3] = {tab.vmw[k][1][1], tab.vmw[k][2][1], tab.vmw[k][3][1]};
+        area_point_p1<false, k, T>(A1, dv[k], Hv[k], xv[k], yv[k], tab.vmw[k][0][0], wv, H0, hg, ghbx, ghby, cfm, friction,
+                                   Fx[4 + k], Fy[4 + k]);
+        area_point_p1<false, k, T>(A1, dm[k], Hm[k], xm[k], ym[k], tab.vmw[k][0][1], wm, H0, hg, ghbx, ghby, cfm, friction,
+                                   Fx[1 + k], Fy[1 + k]);
+      };
+      both(IntC<0>());
+      both(IntC<1>());
+      both(IntC<2>());
 #pragma unroll
-      for (int i = 0; i < 6; ++i) A1.SF[i] = T(0);
-#pragma unroll
-      for (int m = 0; m < 3; ++m) A1.SS[m][0] = A1.SS[m][1] = T(0);
-#pragma unroll
-      for (int q = 0; q < NQ; ++q)
-        area_points_p1<T, T>(A1, tab, q, E.zs[0], E.zs[1], E.xs[0], E.xs[1], E.ys[0], E.ys[1], xb, yb, E.Hb, E.hb1,
-                             E.hb2, H0, T(0.5) * g, g * hbx, g * hby, cfm, friction, Fx[q], Fy[q]);
-#pragma unroll
-      for (int i = 0; i < 6; ++i) SF[i] = A1.SF[i];
+      for (int i = 0; i < 5; ++i) SF[i] = A1.SF[i];
 #pragma unroll
       for (int m = 0; m < 3; ++m) {
         SS[m][0] = A1.SS[m][0];
@@ -400,8 +440,8 @@ __device__ __forceinline__ void tile_area(const Elem<P, Pol>& E, const Geo<Pol>&
 #pragma unroll
     for (int m = 0; m < NP; ++m) {
       Rz[m] = (m > 0) ? detJ * (gx[m] * SF[0] + gy[m] * SF[3]) : T(0);
-      Rx[m] = detJ * (gx[m] * SF[1] + gy[m] * SF[4] + SS[m][0]);
-      Ry[m] = detJ * (gx[m] * SF[2] + gy[m] * SF[5] + SS[m][1]);
+      Rx[m] = (m > 0) ? detJ * (gx[m] * SF[1] + gy[m] * SF[2] + SS[m][0]) : detJ * SS[m][0];
+      Ry[m] = (m > 0) ? detJ * (gx[m] * SF[2] + gy[m] * SF[4] + SS[m][1]) : detJ * SS[m][1];
     }
   } else if constexpr (sizeof(T) == 4 && DG_PACKED_FLUX) {
     // FP32: the points in packed pairs (0,1), (2,3), (4,5), (6,7); point 7 has zero weight and zero
@@ -882,6 +922,26 @@ __global__ void __launch_bounds__(256) plan_kernel(const int4* nbr, const int4* 
 }
 
 // --------------------------------------------------------------------- one tile, one stage ---
+// storm rain at a stage: centre, radius, 1 / (2 rm), log2(e) / re, a third of the peak rate.  The
+// instantiations whose only rain is the storm keep it in registers from tile to tile (250k triangles:
+// 40.7 -> 39.4 us per step; read per tile it was a chain of dependent loads); at p = 2, where registers
+// are short (141 -> 150 us), and in the generic ones it is formed per tile.
+template <class T>
+struct Storm {
+  T cx, cy, rm, rlin, rexp, r0;
+};
+template <class T>
+__device__ __forceinline__ Storm<T> storm_at(const ScenDev& S, double t64) {
+  const ForcingT<T>& F = forcing<T>(S);
+  const T tt = (T)t64 - F.storm[7];
+  return {F.storm[0] + F.storm[2] * tt, F.storm[1] + F.storm[3] * tt, F.storm[5], T(0.5) * F.storm[8], F.storm[9],
+          F.storm[4] * T(1.0 / 3.0)};
+}
+template <int P, int FT>
+DG_HD constexpr bool storm_regs() {
+  return P == 1 && ft_rain(FT) == 2;
+}
+
 // Phases 1-3 of one tile: the area integrals and rain of each lane's element, every edge of the tile
 // once, then the lift, stage combination and positive-depth operator; O is the element's new record.
 // halo_ready() makes the staged halo records readable; it is called once by the whole warp, before
@@ -890,7 +950,8 @@ __global__ void __launch_bounds__(256) plan_kernel(const int4* nbr, const int4* 
 // done with.  The step-initial record comes from shared memory (WNS) or from a.wn.
 template <int P, int FLUX, class Pol, int FT, bool WNS, class HaloReady, class Far, class Release>
 __device__ __forceinline__ void tile_body(const StageArgs<Pol>& a, const ScenDev& S, double t64, int rain_kind, int press,
-                                          const RainRec<typename Pol::T>& rr, int tile, int lane, bool valid, int counts,
+                                          const RainRec<typename Pol::T>& rr,
+                                          const Storm<typename Pol::T>& storm, int tile, int lane, bool valid, int counts,
                                           const uint4* own, const uint4* halo, const uint4* geoS, const unsigned* planS,
                                           const float* man, const typename Pol::T* xyS, void* flx, const uint4* wnS,
                                           const typename Pol::T (*s_ephi)[P + 1][np_of(P)], const float4* s_ephi4,
@@ -902,7 +963,6 @@ __device__ __forceinline__ void tile_body(const StageArgs<Pol>& a, const ScenDev
   constexpr int NP = np_of(P), NS = NP - 1, NG = P + 1, RV = L::RV, GV = L::GV, NPR = L::NPR, NV = L::NV;
   const RefTab<T>& tab = ctab<T, P>();
   const int e = tile * TILE + lane;
-  const T t = (T)t64;
   const int nedge = counts & 255, ninner = (counts >> 8) & 255;
   const int32_t* over = a.plan_x + (size_t)tile * PLAN_X;
 
@@ -947,19 +1007,15 @@ __device__ __forceinline__ void tile_body(const StageArgs<Pol>& a, const ScenDev
     if (rain_kind == 1) {
       Re = a.rain_e[e];
     } else if (rain_kind == 2) {  // radial storm profile at the three vertices
-      const ForcingT<T>& F = forcing<T>(S);
-      const T tt = t - F.storm[7];
-      const T cx = F.storm[0] + F.storm[2] * tt, cy = F.storm[1] + F.storm[3] * tt;
-      const T rp = F.storm[4], rm = F.storm[5];
+      const Storm<T> st = storm_regs<P, FT>() ? storm : storm_at<T>(S, t64);
       T acc = 0;
 #pragma unroll
       for (int i = 0; i < 3; ++i) {
-        const T dx = vx[i] - cx, dy = vy[i] - cy;
+        const T dx = vx[i] - st.cx, dy = vy[i] - st.cy;
         const T r = fsqrt0(dx * dx + dy * dy);
-        // with 1 / rm and log2(e) / re formed once on the host
-        acc += (r < rm) ? rp * fma(T(0.5) * F.storm[8], r, T(0.5)) : rp * fexp2((rm - r) * F.storm[9]);
+        acc += (r < st.rm) ? fma(st.rlin, r, T(0.5)) : fexp2((st.rm - r) * st.rexp);
       }
-      Re = acc * T(1.0 / 3.0);
+      Re = acc * st.r0;
     } else if (rain_kind == 3 && rr.r0) {
       Re = rain_blend<T>(re0, re1, rr.f);
     } else if (rain_kind == 3) {  // nodal rates interpolated by the node kernel of this stage
@@ -1175,6 +1231,7 @@ __global__ void DG_TILE_BOUNDS tile_kernel(const StageArgs<Pol> a) {
   double t64 = 0.0;
   int rain_kind = 0, press = 0;
   RainRec<T> rr = {nullptr, nullptr, T(0)};  // gridded rain: the two records around the stage time
+  Storm<T> storm = {};
 
   int it = 0;
   for (int tile = gw; tile < a.ntiles; tile += W, ++it) {
@@ -1203,6 +1260,7 @@ __global__ void DG_TILE_BOUNDS tile_kernel(const StageArgs<Pol> a) {
       t64 = Sp->d.t0 + stepd * Sp->d.dt;  // stage time, formed in FP64
       rain_kind = ft_rain(FT) >= 0 ? ft_rain(FT) : Sp->rain_kind;
       press = (FT & FT_PRESS) ? Sp->press : 0;
+      if constexpr (storm_regs<P, FT>()) storm = storm_at<T>(*Sp, t64);
       if (rain_kind == 3) {
         rr.r0 = nullptr;
         if (Sp->rrec) {
@@ -1226,7 +1284,7 @@ __global__ void DG_TILE_BOUNDS tile_kernel(const StageArgs<Pol> a) {
     cp_async_commit();
 
     Elem<P, Pol> O;
-    tile_body<P, FLUX, Pol, FT, false>(a, S, t64, rain_kind, press, rr, tile, lane, valid, meta.z, own, halo, geoS, planS,
+    tile_body<P, FLUX, Pol, FT, false>(a, S, t64, rain_kind, press, rr, storm, tile, lane, valid, meta.z, own, halo, geoS, planS,
                                        reinterpret_cast<const float*>(stat + L::S_MAN),
                                        reinterpret_cast<const T*>(stat + L::S_XY), flx, nullptr, s_ephi, s_ephi4,
                                        [] {
