@@ -62,16 +62,14 @@ __global__ void __maxnreg__(sizeof(typename Pol::T) == 4 ? (P == 1 ? 128 : 200) 
   constexpr int NP = np_of(P), NG = P + 1, RV = L::RV, GV = L::GV;
   const RefTab<T>& tab = ctab<T, P>();
   __shared__ T s_ephi[3][NG][NP];
-  __shared__ float4 s_ephi4[3];
+  __shared__ float4 s_ephi4[P == 1 ? 3 : 15];
   extern __shared__ uint4 tsm[];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   for (int i = tid; i < 3 * NG * NP; i += blockDim.x) {
     const int j = i / (NG * NP), k = (i / NP) % NG, m = i % NP;
     s_ephi[j][k][m] = tab.ephi[j][k][m];
   }
-  if (P == 1 && tid < 3)
-    s_ephi4[tid] = make_float4((float)tab.ephi[tid][0][1], (float)tab.ephi[tid][0][2],
-                               (float)tab.ephi[tid][NG - 1][1], (float)tab.ephi[tid][NG - 1][2]);
+  edge_rows<P>(tab, s_ephi4);
   const int wpc = blockDim.x >> 5;
   const int tile = blockIdx.x * wpc + warp;  // one tile per warp
   const int vec = SL::vec(st.nrec);
@@ -145,16 +143,20 @@ __global__ void __maxnreg__(sizeof(typename Pol::T) == 4 ? (P == 1 ? 128 : 200) 
       if constexpr (storm_regs<P, FT>()) storm = storm_at<T>(S, t64);
       Acc rain_acc = acc_make<Acc>(0.f, 0.f, 0.0), bdry_acc = acc_make<Acc>(0.f, 0.f, 0.0);
       Elem<P, Pol> O;
-      tile_body<P, FLUX, Pol, FT, true>(a, S, t64, rain_kind, press, rr, storm, tile, lane, valid, meta.z,
+      tile_body<P, FLUX, Pol, FT, true>(a, S, t64, rain_kind, press, rr, storm, tile, lane, valid, meta.z, meta.w,
                                         Wm + SL::REC + c.in * SL::RECS, halo, Wm + SL::GEO,
                                         reinterpret_cast<const unsigned*>(Wm + SL::PLAN),
                                         reinterpret_cast<const float*>(Wm + L::S_MAN),
                                         reinterpret_cast<const T*>(Wm + SL::XY), Wm + SL::FLX, Wm + SL::REC, s_ephi,
                                         s_ephi4, halo_ready,
-                                        [&](int n, Raw<RV>& r) {
-                                          const uint32_t at = remote(n) + rin;
+                                        [&](int n) {
+                                          if (n >= 0) {
+                                            const uint32_t at = remote(n) + rin;
 #pragma unroll
-                                          for (int v = 0; v < RV; ++v) r.v[v] = ld_cluster128(at + 16u * TILE * v);
+                                            for (int v = 0; v < RV; ++v)
+                                              halo[v * HALO + lane] = ld_cluster128(at + 16u * TILE * v);
+                                          }
+                                          __syncwarp();
                                         },
                                         [] {},
                                         O, rain_acc, bdry_acc);

@@ -49,23 +49,24 @@ constexpr int TE_MAX = 96;  // edges touching a 32-element tile (3 per element a
 // The tile plan: what the neighbour codes say about a tile's edges, laid out once per mesh by
 // plan_kernel (the connectivity never changes) and copied with the tile's other data.  One 32-bit
 // word per edge:
-//   bits 0-8    left side: source << 2 | local edge
-//   bits 9-17   right side, or the boundary code (bit 18): 0 land, 1 + tidal segment,
+//   bits 0-7    left side: source << 2 | local edge
+//   bits 8-15   right side, or the boundary code (bit 16): 0 land, 1 + tidal segment,
 //               1 + MAXSEG + river segment
-//   bit 18      boundary edge;  bit 19  the right side is the tile's own element (whose geometry
-//               holds the edge's normal, negated)
-// sources: 0-31 own element, 32-63 staged halo record, 64-127 entry source - 64 of the tile's list
-// of further neighbours (none on Hilbert-ordered meshes; read from global memory).  In-tile edges
-// come first, then the edges to other tiles, then the boundary edges: the first round of the edge
-// phase does not wait for the halo.  Per tile: EDGE_ROUND2 = 64 words, the 32 halo elements, (mixed
-// path) the Manning coefficients, and {scenario, elements present, counts, 0}; edges 64-95 and
-// neighbours 32-95 are in the overflow array, which a lane reads directly.
+//   bit 16      boundary edge;  bits 18-25  place of the edge's scaled normal in the geometry block;
+//   bit 31      the right side is the tile's own element: the normal is negated
+// sources: 0-31 own element, 32-63 staged halo record.  In-tile edges come first, then the edges to
+// the first 32 neighbours in other tiles, then the boundary edges: the first round of the edge phase
+// does not wait for the halo.  Tiles with more neighbours (about one in a thousand on Hilbert-ordered
+// meshes) have two further batches: 32 more halo records each, and their edges.  Per tile:
+// EDGE_INLINE words, the first 32 halo elements, (mixed path) the Manning coefficients, and {scenario,
+// elements present, counts, further batches}; the words 64-95 and the further neighbours are in the
+// overflow array.
 // Before, every stage rebuilt this per tile from the neighbour codes (nine ballots, the population
 // counts, a descriptor of two sides and a normal per edge): about 190 of 1,940 warp instructions,
 // with the halo loads waiting for it.
 constexpr int EDGE_INLINE = 64;
 constexpr int PLAN_X = 32 + 64;  // overflow words per tile: edges 64..95, neighbours 32..95
-constexpr unsigned ED_BND = 1u << 18, ED_OWN_R = 1u << 19;
+constexpr unsigned ED_BND = 1u << 16, ED_OWN_R = 1u << 31;
 template <class T>
 __host__ __device__ constexpr int plan_vec() {  // 16-byte units per tile
   return (EDGE_INLINE + HALO + (sizeof(T) == 4 ? TILE : 0)) / 4 + 1;
@@ -548,30 +549,64 @@ __device__ __forceinline__ void tile_area(const Elem<P, Pol>& E, const Geo<Pol>&
 }
 
 // ---------------------------------------------------------------------- edge phase ------
-// record of a side: own (src < 32) or staged halo (src < 64) records [RV][32] in shared memory,
-// else neighbour src - 32 of the tile's list, read by far(element, record)
-template <int RV, class Far>
-__device__ __forceinline__ void fetch_side(const uint4* own, const uint4* halo, const Far& far,
-                                           const int32_t* __restrict__ over, int src, Raw<RV>& r) {
-  if (src < 64) {  // shared memory, read as such (not through a generic address)
-    const uint32_t p = smem_u32(src < 32 ? own + src : halo + (src - 32));
-    constexpr uint32_t stride = 16u * TILE;  // HALO == TILE: one stride for both
+// record of a side in shared memory (read as such, not through a generic address): own (src < 32) or
+// staged halo; ownB and halB are the addresses of the blocks' first vectors, halB less 32 of them
+template <int RV>
+__device__ __forceinline__ void fetch_side(uint32_t ownB, uint32_t halB, unsigned src, Raw<RV>& r) {
+  const uint32_t p = (src < 32 ? ownB : halB) + 16u * src;
+  constexpr uint32_t stride = 16u * TILE;  // HALO == TILE: one stride for both
 #pragma unroll
-    for (int v = 0; v < RV; ++v) r.v[v] = lds128(p + stride * v);
+  for (int v = 0; v < RV; ++v) r.v[v] = lds128(p + stride * v);
+}
+// an edge's scaled normal along its left side's outward direction
+__device__ __forceinline__ void edge_normal(const uint4* geo, unsigned ed, float& nx, float& ny) {
+  const float2 n = reinterpret_cast<const float2*>(geo)[(ed >> 18) & 255];
+  const unsigned sg = ed & ED_OWN_R;
+  nx = __uint_as_float(__float_as_uint(n.x) ^ sg);
+  ny = __uint_as_float(__float_as_uint(n.y) ^ sg);
+}
+__device__ __forceinline__ void edge_normal(const uint4* geo, unsigned ed, double& nx, double& ny) {
+  const double2 n = reinterpret_cast<const double2*>(geo)[(ed >> 18) & 255];
+  nx = (ed & ED_OWN_R) ? -n.x : n.x;
+  ny = (ed & ED_OWN_R) ? -n.y : n.y;
+}
+// traces of a side at the points of its local edge j, in reverse order with REV (the points of the
+// other side).  ephi4 (FP32): p = 1 one row per edge {phi_1, phi_2 at point 0, at point 1}; p = 2 one row
+// per edge and mode m = 1..5 with phi_m at the three points
+template <int P, class Pol, bool REV>
+__device__ __forceinline__ void side_traces(const Elem<P, Pol>& E, int j, const typename Pol::T (*ephi)[P + 1][np_of(P)],
+                                            const float4* ephi4, Trace<typename Pol::T> (&t)[P + 1]) {
+  using T = typename Pol::T;
+  constexpr int NG = P + 1;
+  if constexpr (sizeof(T) == 4 && P == 1) {
+    const float4 b = ephi4[j];
+    t[REV ? 1 : 0] = trace_p1(E, b.x, b.y);
+    t[REV ? 0 : 1] = trace_p1(E, b.z, b.w);
+  } else if constexpr (sizeof(T) == 4) {
+    const T xb = acc_r(E.xb), yb = acc_r(E.yb);
+    T h[NG];
+#pragma unroll
+    for (int k = 0; k < NG; ++k) t[k] = {T(0), T(0), xb, yb};
+#pragma unroll
+    for (int m = 0; m < np_of(P) - 1; ++m) {
+      const float4 b = ephi4[5 * j + m];
+#pragma unroll
+      for (int k = 0; k < NG; ++k) {
+        const int q = REV ? NG - 1 - k : k;
+        const float ph = q == 0 ? b.x : (q == 1 ? b.y : b.z);
+        t[k].d = fma(E.zs[m], ph, t[k].d);
+        t[k].qx = fma(E.xs[m], ph, t[k].qx);
+        t[k].qy = fma(E.ys[m], ph, t[k].qy);
+        if (m == 0) h[k] = E.hb1 * ph;
+        if (m == 1) h[k] = fma(E.hb2, ph, h[k]);
+      }
+    }
+#pragma unroll
+    for (int k = 0; k < NG; ++k) t[k].H = E.Hb + (t[k].d + h[k]);
   } else {
-    far(__ldg(over + 32 + (src - 64)), r);
+#pragma unroll
+    for (int k = 0; k < NG; ++k) t[k] = trace_at<P, Pol>(E, ephi[j][REV ? NG - 1 - k : k]);
   }
-}
-// scaled normal of local edge j of own element e from the geometry block
-__device__ __forceinline__ void edge_normal(const uint4* geo, int e, int j, float& nx, float& ny) {
-  const float2 n = reinterpret_cast<const float2*>(geo + 3 * e)[j];
-  nx = n.x;
-  ny = n.y;
-}
-__device__ __forceinline__ void edge_normal(const uint4* geo, int e, int j, double& nx, double& ny) {
-  const double2 n = reinterpret_cast<const double2*>(geo + 5 * e)[j];
-  nx = n.x;
-  ny = n.y;
 }
 
 // one side's edge slot at flx[(j NPR + i) 32 + lane], pairs of T: Gz[NG], Gx[NG], Gy[NG] (, mass)
@@ -634,155 +669,168 @@ __device__ __forceinline__ T wall_coef(const Trace<T>& t, T nx, T ny, T g, T H0)
   return qn * (un + c) + pdev(t.d, t.H, g);
 }
 
-template <int P, int FLUX, class Pol, int FT, class Far>
-__device__ __forceinline__ void tile_edge(const StageArgs<Pol>& a, const ScenDev& S, const uint4* own,
-                                          const uint4* halo, const uint4* geo, const Far& far, const int32_t* over,
-                                          void* flx, unsigned ed, const typename Pol::T (*ephi)[P + 1][np_of(P)],
-                                          const float4* ephi4, double t64, typename Pol::Acc& bdry_acc) {
+// Edge slots at p = 1 in FP32 hold, per variable, the sum S and the difference D of the two point
+// values instead of the values: seen from the other side (negated, points in reverse order) they are
+// (-S, D), so the right side needs no reordering, S of the mass flux is the mass integral, and the lift
+// needs only the basis' means and differences over the points, several of which are zero.  With the
+// normals by one index, the boundary cases in a branch of their own and no run-time test for far
+// neighbours: 361 -> about 300 warp instructions per edge round, 250k triangles 39.2 -> 36.3 us per step,
+// hurricane 2M 253.6 -> 233.9, 500k LLF SSP(5,2) 185.3 -> 175.4, graded p = 2 300k 140.2 -> 136.2.
+template <int P, class Pol>
+DG_HD constexpr bool slots_sd() {
+  return DG_PACKED_FLUX && P == 1 && sizeof(typename Pol::T) == 4;
+}
+__device__ __forceinline__ f2 sum_diff(f2 v) { return make_float2(v.x + v.y, v.y - v.x); }
+// slot of side j of element e: {Gz, Gx} at [j][32] float4, then Gy at [j][32] float2
+__device__ __forceinline__ void store_sd(void* flx, int e, int j, f2 z, f2 x, f2 y) {
+  reinterpret_cast<float4*>(flx)[j * 32 + e] = make_float4(z.x, z.y, x.x, x.y);
+  reinterpret_cast<float2*>(reinterpret_cast<float4*>(flx) + 96)[j * 32 + e] = y;
+}
+
+template <int P, int FLUX, class Pol, int FT>
+__device__ __forceinline__ void tile_edge(const StageArgs<Pol>& a, const ScenDev& S, uint32_t ownB, uint32_t halB,
+                                          const uint4* geo, void* flx, unsigned ed,
+                                          const typename Pol::T (*ephi)[P + 1][np_of(P)], const float4* ephi4, double t64,
+                                          typename Pol::Acc& bdry_acc) {
   using T = typename Pol::T;
   using L = TileLayout<P, Pol, FT>;
   constexpr int NG = P + 1, RV = L::RV, NPR = L::NPR, NV = L::NV;
   constexpr bool MASSV = L::MASSV;
   const RefTab<T>& tab = ctab<T, P>();
   const T g = a.g, H0 = a.H0;
-  const int jL = ed & 3, srcL = (ed >> 2) & 127;
-  const int sR = (ed >> 9) & 511;  // right side, or the boundary code
+  const unsigned jL = ed & 3, srcL = (ed >> 2) & 63;
+  const unsigned jR = (ed >> 8) & 3, srcR = (ed >> 10) & 63;
   Raw<RV> rl;
-  fetch_side<RV>(own, halo, far, over, srcL, rl);
-  T lnx, lny;  // L's scaled outward normal, from the own element's geometry
-  if (ed & ED_OWN_R) {
-    edge_normal(geo, sR >> 2, sR & 3, lnx, lny);
-    lnx = -lnx;
-    lny = -lny;
-  } else {
-    edge_normal(geo, srcL, jL, lnx, lny);
-  }
+  fetch_side<RV>(ownB, halB, srcL, rl);
+  T lnx, lny;
+  edge_normal(geo, ed, lnx, lny);
   Elem<P, Pol> EL;
   unpack<P>(rl, EL);
   const T l2 = lnx * lnx + lny * lny, il = frsqrt(l2), len = l2 * il;  // edge length and its inverse
   const T nx = lnx * il, ny = lny * il;
-  constexpr bool P1F = P == 1 && sizeof(T) == 4;  // basis values of both points in one 16-byte read
   Trace<T> tl[NG], tr[NG];
-  if constexpr (P1F) {
-    const float4 b = ephi4[jL];
-    tl[0] = trace_p1(EL, b.x, b.y);
-    tl[NG - 1] = trace_p1(EL, b.z, b.w);
-  } else {
-#pragma unroll
-    for (int k = 0; k < NG; ++k) tl[k] = trace_at<P, Pol>(EL, ephi[jL][k]);
-  }
-  // boundary kind (an instantiation without a kind treats such an edge as a wall; the host never
-  // selects it for a run that has one)
+  side_traces<P, Pol, false>(EL, jL, ephi, ephi4, tl);
   const bool interior = !(ed & ED_BND);
-  const bool river_e = (FT & FT_RIVER) && !interior && sR > MAXSEG;
-  const bool ocean_e = (FT & FT_OCEAN) && !interior && sR >= 1 && sR <= MAXSEG;
-  const bool land = !interior && !river_e && !ocean_e;
   const bool dryL = (EL.flags & FLAG_DRY) != 0;
-  bool dryR = false, river = false;
-  int jR = 0, srcR = 64;
+  bool dryR = false, land = false, river = false;
   T dcRL = T(0), qr = T(0);
   if (interior) {
-    jR = sR & 3;
-    srcR = sR >> 2;
     Raw<RV> rr;
-    fetch_side<RV>(own, halo, far, over, srcR, rr);
+    fetch_side<RV>(ownB, halB, srcR, rr);
     Elem<P, Pol> ER;
     unpack<P>(rr, ER);
     dcRL = acc_sub_r(ER.zb, EL.zb);
     dryR = (ER.flags & FLAG_DRY) != 0;
-    if constexpr (P1F) {  // R's point 1 - k is L's point k
-      const float4 b = ephi4[jR];
-      tr[0] = trace_p1(ER, b.z, b.w);
-      tr[NG - 1] = trace_p1(ER, b.x, b.y);
+    side_traces<P, Pol, true>(ER, jR, ephi, ephi4, tr);  // the same points
+  } else {
+    // boundary kind (an instantiation without a kind treats such an edge as a wall; the host never
+    // selects it for a run that has one); a land edge takes the flux evaluation against its own trace
+    const int code = (ed >> 8) & 255;
+#pragma unroll
+    for (int k = 0; k < NG; ++k) tr[k] = tl[k];
+    if ((FT & FT_RIVER) && code > MAXSEG) {  // river: interior elevation, prescribed normal discharge
+      qr = river_at<T>(S, min(code - 1 - MAXSEG, MAXRIV - 1), t64);
+      river = true;
+#pragma unroll
+      for (int k = 0; k < NG; ++k) {
+        tr[k].qx = -qr * nx;
+        tr[k].qy = -qr * ny;
+      }
+    } else if ((FT & FT_OCEAN) && code >= 1 && code <= MAXSEG) {  // ocean: tidal elevation, interior discharge
+      const T zbc = tide_at<T>(S, code - 1, t64);
+      const T dgh = acc_r(acc_addr(acc_neg(EL.zb), zbc));  // ghost zeta - mean of L
+#pragma unroll
+      for (int k = 0; k < NG; ++k) {
+        tr[k].H = tl[k].H + (dgh - tl[k].d);
+        tr[k].d = dgh;
+      }
     } else {
-#pragma unroll
-      for (int k = 0; k < NG; ++k) tr[k] = trace_at<P, Pol>(ER, ephi[jR][NG - 1 - k]);  // the same points
-    }
-  } else if (river_e) {  // river: interior elevation, prescribed normal discharge
-    const int rs = min(sR - 1 - MAXSEG, MAXRIV - 1);
-    qr = river_at<T>(S, rs, t64);
-    river = true;
-#pragma unroll
-    for (int k = 0; k < NG; ++k) {
-      tr[k] = tl[k];
-      tr[k].qx = -qr * nx;
-      tr[k].qy = -qr * ny;
-    }
-  } else if (ocean_e) {  // ocean: tidal elevation, interior discharge
-    const int seg = sR - 1;
-    const T zbc = tide_at<T>(S, seg, t64);
-    const T dgh = acc_r(acc_addr(acc_neg(EL.zb), zbc));  // ghost zeta - mean of L
-#pragma unroll
-    for (int k = 0; k < NG; ++k) {
-      tr[k] = tl[k];
-      tr[k].H = tl[k].H + (dgh - tl[k].d);
-      tr[k].d = dgh;
+      land = true;
     }
   }
-  constexpr bool PK = DG_PACKED_FLUX && P == 1 && sizeof(T) == 4;  // both points in packed FP32x2
-  T fz[NG], fx[NG], fy[NG];
-  T ec = T(0);  // mass flux integral along n (L's outward normal)
-  bool closed = land;
-  FluxAux2 ax;  // packed path: per-side quantities for the wall flux
-  if constexpr (PK) {
-    // every edge takes the flux evaluation (a land edge against its own trace: the wall below needs
-    // only the left side's quantities), so that no lane takes a separate wall path
-    if (land) {
-#pragma unroll
-      for (int k = 0; k < NG; ++k) tr[k] = tl[k];
-    }
+  const T hl = T(0.5) * len;
+  if constexpr (slots_sd<P, Pol>()) {
+    // both points in packed FP32x2; every edge takes the flux evaluation, so that no lane takes a
+    // separate wall path.  Both Gauss weights are 1.
     const Trace2 L2{make_float2(tl[0].d, tl[1].d), make_float2(tl[0].H, tl[1].H), make_float2(tl[0].qx, tl[1].qx),
                     make_float2(tl[0].qy, tl[1].qy)};
     const Trace2 R2{make_float2(tr[0].d, tr[1].d), make_float2(tr[0].H, tr[1].H), make_float2(tr[0].qx, tr[1].qx),
                     make_float2(tr[0].qy, tr[1].qy)};
     f2 fz2, fx2, fy2;
+    FluxAux2 ax;  // per-side quantities for the wall flux
     edge_flux_pair<FLUX>(L2, R2, p2(dcRL), p2(nx), p2(ny), g, H0, fz2, fx2, fy2, ax);
-    fz[0] = fz2.x; fz[1] = fz2.y;
-    fx[0] = fx2.x; fx[1] = fx2.y;
-    fy[0] = fy2.x; fy[1] = fy2.y;
-  }
-  if (!land) {
-    if constexpr (!PK && P == 2 && sizeof(T) == 4 && DG_PACKED_FLUX) {  // points 0 and 1 packed, point 2 alone
-      const Trace2 L2{make_float2(tl[0].d, tl[1].d), make_float2(tl[0].H, tl[1].H), make_float2(tl[0].qx, tl[1].qx),
-                      make_float2(tl[0].qy, tl[1].qy)};
-      const Trace2 R2{make_float2(tr[0].d, tr[1].d), make_float2(tr[0].H, tr[1].H), make_float2(tr[0].qx, tr[1].qx),
-                      make_float2(tr[0].qy, tr[1].qy)};
-      f2 fz2, fx2, fy2;
-      FluxAux2 ax2;
-      edge_flux_pair<FLUX>(L2, R2, p2(dcRL), p2(nx), p2(ny), g, H0, fz2, fx2, fy2, ax2);
-      fz[0] = fz2.x; fz[1] = fz2.y;
-      fx[0] = fx2.x; fx[1] = fx2.y;
-      fy[0] = fy2.x; fy[1] = fy2.y;
-      edge_flux<FLUX, T>(tl[NG - 1], tr[NG - 1], dcRL, nx, ny, g, H0, fz[NG - 1], fx[NG - 1], fy[NG - 1]);
-    } else if constexpr (!PK) {
-#pragma unroll
-      for (int k = 0; k < NG; ++k) edge_flux<FLUX, T>(tl[k], tr[k], dcRL, nx, ny, g, H0, fz[k], fx[k], fy[k]);
-    }
-    if (river) {
-#pragma unroll
-      for (int k = 0; k < NG; ++k) fz[k] = -qr;  // the specified normal flow is the mass flux
-    }
-#pragma unroll
-    for (int k = 0; k < NG; ++k) ec = fma(tab.gw[k], fz[k], ec);
-    ec = ec * (T(0.5) * len);
+    if (river) fz2 = p2(-qr);  // the specified normal flow is the mass flux
+    const f2 hl2 = p2(hl);
+    const f2 Fz = mul2(sum_diff(fz2), hl2);  // Fz.x: the mass integral along n
     // wet/dry closure: no water leaves a dry element (interior: either side; ocean/river: L)
-    closed = interior ? ((dryL && ec > T(0)) || (dryR && ec < T(0))) : (dryL && ec > T(0));
-  }
-  const T hl = T(0.5) * len;
-  T vals[NV + 1];
-  if (srcL < TILE) {  // L's slot, in L's point order
+    const bool closed = land || (dryL && Fz.x > 0.f) || (dryR && Fz.x < 0.f);
     if (!closed) {
-      if constexpr (PK) {
-        const f2 hq = p2(0.25f * g), dc = p2(dcRL);  // the mean of the sides' g/2 d (2H - d)
-        const f2 Ld = make_float2(tl[0].d, tl[1].d), LH = make_float2(tl[0].H, tl[1].H);
-        const f2 Rd = add2(make_float2(tr[0].d, tr[1].d), dc), RH = make_float2(tr[0].H, tr[1].H);
-        const f2 pp = mul2(hq, fma2(Ld, fma2(p2(2.f), LH, neg2(Ld)), mul2(Rd, fma2(p2(2.f), RH, neg2(Rd)))));
-        const f2 wk = mul2(make_float2(tab.gw[0], tab.gw[1]), p2(hl));
-        const f2 vz = mul2(wk, make_float2(fz[0], fz[1]));
-        const f2 vx = mul2(wk, fma2(pp, p2(nx), make_float2(fx[0], fx[1])));
-        const f2 vy = mul2(wk, fma2(pp, p2(ny), make_float2(fy[0], fy[1])));
-        vals[0] = vz.x; vals[1] = vz.y; vals[2] = vx.x; vals[3] = vx.y; vals[4] = vy.x; vals[5] = vy.y;
+      const f2 Fx = mul2(sum_diff(fx2), hl2), Fy = mul2(sum_diff(fy2), hl2), dc = p2(dcRL), hq = p2(0.25f * g);
+      if (srcL < TILE) {  // pressure: the mean of the sides' g/2 d (2H - d) relative to L's mean
+        const f2 Rd = add2(R2.d, dc);
+        const f2 pp = fma2(L2.d, fma2(p2(2.f), L2.H, neg2(L2.d)), mul2(Rd, fma2(p2(2.f), R2.H, neg2(Rd))));
+        const f2 Pd = mul2(sum_diff(mul2(hq, pp)), hl2);
+        store_sd(flx, srcL, jL, Fz, fma2(Pd, p2(nx), Fx), fma2(Pd, p2(ny), Fy));
+        if (!interior) bdry_acc = acc_addr(bdry_acc, -Fz.x);  // inflow
+      }
+      if (interior && srcR < TILE) {  // relative to R's mean, along -n
+        const f2 Ld = sub2(L2.d, dc);
+        const f2 pp = fma2(R2.d, fma2(p2(2.f), R2.H, neg2(R2.d)), mul2(Ld, fma2(p2(2.f), L2.H, neg2(Ld))));
+        const f2 Pd = mul2(sum_diff(mul2(hq, pp)), hl2);
+        store_sd(flx, srcR, jR, make_float2(-Fz.x, Fz.y), fma2(Pd, make_float2(-nx, nx), make_float2(-Fx.x, Fx.y)),
+                 fma2(Pd, make_float2(-ny, ny), make_float2(-Fy.x, Fy.y)));
+      }
+    } else {
+      // wall: q.n (q.n / Hs + c) + pressure relative to the side's mean (LLF: (q.n + |q.n|) / Hs)
+      const f2 z = p2(0.f), sg = p2(fsqrt_pos(g)), hg = p2(0.5f * g);
+      if (srcL < TILE) {
+        const f2 un = (FLUX == 1) ? mul2(add2(ax.mL, abs2(ax.mL)), ax.iL) : mul2(ax.mL, ax.iL);
+        const f2 w = fma2(ax.mL, fma2(sg, ax.sL, un), mul2(hg, mul2(L2.d, fma2(p2(2.f), L2.H, neg2(L2.d)))));
+        const f2 Wd = mul2(sum_diff(w), hl2);
+        store_sd(flx, srcL, jL, z, mul2(Wd, p2(nx)), mul2(Wd, p2(ny)));
+      }
+      if (interior && srcR < TILE) {  // seen from R along -n: q.n_R = -mR
+        const f2 mR = neg2(ax.mR);
+        const f2 un = (FLUX == 1) ? mul2(add2(mR, abs2(mR)), ax.iR) : mul2(mR, ax.iR);
+        const f2 w = fma2(mR, fma2(sg, ax.sR, un), mul2(hg, mul2(R2.d, fma2(p2(2.f), R2.H, neg2(R2.d)))));
+        const f2 Wd = mul2(sum_diff(w), hl2);
+        store_sd(flx, srcR, jR, z, mul2(Wd, make_float2(-nx, nx)), mul2(Wd, make_float2(-ny, ny)));
+      }
+    }
+  } else {
+    T fz[NG], fx[NG], fy[NG];
+    T ec = T(0);  // mass flux integral along n (L's outward normal)
+    bool closed = land;
+    if (!land) {
+      if constexpr (P == 2 && sizeof(T) == 4 && DG_PACKED_FLUX) {  // points 0 and 1 packed, point 2 alone
+        const Trace2 L2{make_float2(tl[0].d, tl[1].d), make_float2(tl[0].H, tl[1].H), make_float2(tl[0].qx, tl[1].qx),
+                        make_float2(tl[0].qy, tl[1].qy)};
+        const Trace2 R2{make_float2(tr[0].d, tr[1].d), make_float2(tr[0].H, tr[1].H), make_float2(tr[0].qx, tr[1].qx),
+                        make_float2(tr[0].qy, tr[1].qy)};
+        f2 fz2, fx2, fy2;
+        FluxAux2 ax2;
+        edge_flux_pair<FLUX>(L2, R2, p2(dcRL), p2(nx), p2(ny), g, H0, fz2, fx2, fy2, ax2);
+        fz[0] = fz2.x; fz[1] = fz2.y;
+        fx[0] = fx2.x; fx[1] = fx2.y;
+        fy[0] = fy2.x; fy[1] = fy2.y;
+        edge_flux<FLUX, T>(tl[NG - 1], tr[NG - 1], dcRL, nx, ny, g, H0, fz[NG - 1], fx[NG - 1], fy[NG - 1]);
       } else {
+#pragma unroll
+        for (int k = 0; k < NG; ++k) edge_flux<FLUX, T>(tl[k], tr[k], dcRL, nx, ny, g, H0, fz[k], fx[k], fy[k]);
+      }
+      if (river) {
+#pragma unroll
+        for (int k = 0; k < NG; ++k) fz[k] = -qr;  // the specified normal flow is the mass flux
+      }
+#pragma unroll
+      for (int k = 0; k < NG; ++k) ec = fma(tab.gw[k], fz[k], ec);
+      ec = ec * hl;
+      // wet/dry closure: no water leaves a dry element (interior: either side; ocean/river: L)
+      closed = (dryL && ec > T(0)) || (dryR && ec < T(0));
+    }
+    T vals[NV + 1];
+    if (srcL < TILE) {  // L's slot, in L's point order
+      if (!closed) {
 #pragma unroll
         for (int k = 0; k < NG; ++k) {
           const T p = T(0.5) * (pdev(tl[k].d, tl[k].H, g) + pdev(tr[k].d + dcRL, tr[k].H, g));
@@ -791,42 +839,22 @@ __device__ __forceinline__ void tile_edge(const StageArgs<Pol>& a, const ScenDev
           vals[NG + k] = wk * (fx[k] + p * nx);
           vals[2 * NG + k] = wk * (fy[k] + p * ny);
         }
-      }
-      if (MASSV) vals[3 * NG] = ec;
-    } else if constexpr (PK) {  // wall: q.n (q.n / Hs + c) + pressure relative to L's mean (LLF: (q.n + |q.n|) / Hs)
-      const f2 Ld = make_float2(tl[0].d, tl[1].d), LH = make_float2(tl[0].H, tl[1].H);
-      const f2 un = (FLUX == 1) ? mul2(add2(ax.mL, abs2(ax.mL)), ax.iL) : mul2(ax.mL, ax.iL);
-      const f2 wl = fma2(ax.mL, fma2(p2(fsqrt_pos(g)), ax.sL, un), mul2(p2(0.5f * g), mul2(Ld, fma2(p2(2.f), LH, neg2(Ld)))));
-      const f2 cw = mul2(mul2(make_float2(tab.gw[0], tab.gw[1]), p2(hl)), wl);
-      const f2 vx = mul2(cw, p2(nx)), vy = mul2(cw, p2(ny));
-      vals[0] = vals[1] = T(0);
-      vals[2] = vx.x; vals[3] = vx.y; vals[4] = vy.x; vals[5] = vy.y;
-    } else {
-#pragma unroll
-      for (int k = 0; k < NG; ++k) {
-        const T cw = tab.gw[k] * hl * wall_coef<FLUX, T>(tl[k], nx, ny, g, H0);
-        vals[k] = T(0);
-        vals[NG + k] = cw * nx;
-        vals[2 * NG + k] = cw * ny;
-      }
-      if (MASSV) vals[3 * NG] = T(0);
-    }
-    store_side<T, NPR, NV>(flx, srcL, jL, vals);
-    if (!interior && !land && !closed) bdry_acc = acc_addr(bdry_acc, -side_mass<T, NG, MASSV>(vals));  // inflow
-  }
-  if (interior && srcR < TILE) {  // R's slot, in R's point order (its point k is L's NG-1-k)
-    if (!closed) {
-      if constexpr (PK) {  // R's point kr is L's point 1 - kr
-        const f2 hq = p2(0.25f * g), dc = p2(dcRL);  // the mean of the sides' g/2 d (2H - d)
-        const f2 Rd = make_float2(tr[1].d, tr[0].d), RH = make_float2(tr[1].H, tr[0].H);
-        const f2 Ld = sub2(make_float2(tl[1].d, tl[0].d), dc), LH = make_float2(tl[1].H, tl[0].H);
-        const f2 pp = mul2(hq, fma2(Rd, fma2(p2(2.f), RH, neg2(Rd)), mul2(Ld, fma2(p2(2.f), LH, neg2(Ld)))));
-        const f2 wk = mul2(make_float2(tab.gw[0], tab.gw[1]), p2(-hl));
-        const f2 vz = mul2(wk, make_float2(fz[1], fz[0]));
-        const f2 vx = mul2(wk, fma2(pp, p2(nx), make_float2(fx[1], fx[0])));
-        const f2 vy = mul2(wk, fma2(pp, p2(ny), make_float2(fy[1], fy[0])));
-        vals[0] = vz.x; vals[1] = vz.y; vals[2] = vx.x; vals[3] = vx.y; vals[4] = vy.x; vals[5] = vy.y;
+        if (MASSV) vals[3 * NG] = ec;
       } else {
+#pragma unroll
+        for (int k = 0; k < NG; ++k) {
+          const T cw = tab.gw[k] * hl * wall_coef<FLUX, T>(tl[k], nx, ny, g, H0);
+          vals[k] = T(0);
+          vals[NG + k] = cw * nx;
+          vals[2 * NG + k] = cw * ny;
+        }
+        if (MASSV) vals[3 * NG] = T(0);
+      }
+      store_side<T, NPR, NV>(flx, srcL, jL, vals);
+      if (!interior && !closed) bdry_acc = acc_addr(bdry_acc, -side_mass<T, NG, MASSV>(vals));  // inflow
+    }
+    if (interior && srcR < TILE) {  // R's slot, in R's point order (its point k is L's NG-1-k)
+      if (!closed) {
 #pragma unroll
         for (int kr = 0; kr < NG; ++kr) {
           const int k = NG - 1 - kr;
@@ -836,30 +864,20 @@ __device__ __forceinline__ void tile_edge(const StageArgs<Pol>& a, const ScenDev
           vals[NG + kr] = -(wk * (fx[k] + p * nx));
           vals[2 * NG + kr] = -(wk * (fy[k] + p * ny));
         }
-      }
-      if (MASSV) vals[3 * NG] = -ec;
-    } else if constexpr (PK) {  // wall seen from R along -n: q.n_R = -mR
-      const f2 mR = neg2(ax.mR);
-      const f2 Rd = make_float2(tr[0].d, tr[1].d), RH = make_float2(tr[0].H, tr[1].H);
-      const f2 un = (FLUX == 1) ? mul2(add2(mR, abs2(mR)), ax.iR) : mul2(mR, ax.iR);
-      const f2 wr = fma2(mR, fma2(p2(fsqrt_pos(g)), ax.sR, un), mul2(p2(0.5f * g), mul2(Rd, fma2(p2(2.f), RH, neg2(Rd)))));
-      // R's point kr is L's point 1 - kr
-      const f2 cw = mul2(mul2(make_float2(tab.gw[0], tab.gw[1]), p2(-hl)), make_float2(wr.y, wr.x));
-      const f2 vx = mul2(cw, p2(nx)), vy = mul2(cw, p2(ny));
-      vals[0] = vals[1] = T(0);
-      vals[2] = vx.x; vals[3] = vx.y; vals[4] = vy.x; vals[5] = vy.y;
-    } else {
+        if (MASSV) vals[3 * NG] = -ec;
+      } else {
 #pragma unroll
-      for (int kr = 0; kr < NG; ++kr) {
-        const int k = NG - 1 - kr;
-        const T cw = tab.gw[kr] * hl * wall_coef<FLUX, T>(tr[k], -nx, -ny, g, H0);
-        vals[kr] = T(0);
-        vals[NG + kr] = -(cw * nx);
-        vals[2 * NG + kr] = -(cw * ny);
+        for (int kr = 0; kr < NG; ++kr) {
+          const int k = NG - 1 - kr;
+          const T cw = tab.gw[kr] * hl * wall_coef<FLUX, T>(tr[k], -nx, -ny, g, H0);
+          vals[kr] = T(0);
+          vals[NG + kr] = -(cw * nx);
+          vals[2 * NG + kr] = -(cw * ny);
+        }
+        if (MASSV) vals[3 * NG] = T(0);
       }
-      if (MASSV) vals[3 * NG] = T(0);
+      store_side<T, NPR, NV>(flx, srcR, jR, vals);
     }
-    store_side<T, NPR, NV>(flx, srcR, jR, vals);
   }
 }
 
@@ -885,40 +903,55 @@ __global__ void __launch_bounds__(256) plan_kernel(const int4* nbr, const int4* 
   for (int i = lane; i < EDGE_INLINE + HALO; i += 32) desc[i] = 0u;
   for (int i = lane; i < PLAN_X; i += 32) over[i] = 0;
   __syncwarp();
-  int base = 0, hbase = 0, ninner = 0;
+  // halo slot of each edge to another tile
+  int hs[3], nhalo = 0;
 #pragma unroll
-  for (int kind = 0; kind < 3; ++kind) {  // in-tile, to another tile, boundary
+  for (int j = 0; j < 3; ++j) {
+    const int c = code[j], n = c >> 2;
+    const bool out = valid && c >= 0 && (n < e0 || n >= e0 + TILE);
+    const unsigned m = __ballot_sync(0xffffffffu, out);
+    hs[j] = out ? nhalo + __popc(m & lt) : -1;
+    if (out) {
+      if (hs[j] < HALO) halo[hs[j]] = n;
+      else over[hs[j]] = n;  // neighbour 32 and on, after the 32 edge words
+    }
+    nhalo += __popc(m);
+  }
+  int base = 0, count[5];
+#pragma unroll
+  for (int kind = 0; kind < 5; ++kind) {  // in-tile; to the first 32 neighbours; boundary; batches 1 and 2
+    const int before = base;
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
-      const int c = code[j], n = c >> 2, jn = c & 3, me = (lane << 2) | j;
-      const bool inside = c >= 0 && n >= e0 && n < e0 + TILE;
-      const bool mine = valid && (kind == 0 ? (inside && e < n) : kind == 1 ? (c >= 0 && !inside) : c < 0);
+      const int c = code[j], n = c >> 2, jn = c & 3;
+      const unsigned me = (unsigned)((lane << 2) | j);
+      const bool inside = valid && c >= 0 && hs[j] < 0;
+      const bool mine = kind == 0 ? (inside && e < n) : kind == 2 ? (valid && c < 0) : (hs[j] >= 0 && hs[j] / HALO == (kind == 1 ? 0 : kind - 2));
       const unsigned m = __ballot_sync(0xffffffffu, mine);
-      const int i = base + __popc(m & lt), h = hbase + __popc(m & lt);
       if (mine) {
         unsigned d;
         if (kind == 0) {
-          d = (unsigned)me | (unsigned)(((n - e0) << 2) | jn) << 9;
-        } else if (kind == 1) {
-          const unsigned other = (unsigned)(((32 + h) << 2) | jn);  // sources 32.. : halo, then overflow
-          d = e < n ? ((unsigned)me | other << 9) : (other | (unsigned)me << 9 | ED_OWN_R);
-          if (h < HALO) halo[h] = n;
-          else over[32 + (h - HALO)] = n;
+          d = me | (unsigned)(((n - e0) << 2) | jn) << 8;
+        } else if (kind == 2) {
+          d = me | (unsigned)(-1 - c) << 8 | ED_BND;
         } else {
-          d = (unsigned)me | (unsigned)(-1 - c) << 9 | ED_BND;
+          const unsigned other = (unsigned)(((32 + hs[j] % HALO) << 2) | jn);
+          d = e < n ? (me | other << 8) : (other | me << 8 | ED_OWN_R);
         }
+        d |= (unsigned)(lane * (sizeof(T) == 4 ? 6 : 5) + j) << 18;  // float2 / double2 of the own element's normal j
+        const int i = base + __popc(m & lt);
         if (i < EDGE_INLINE) desc[i] = d;
         else over[i - EDGE_INLINE] = (int32_t)d;
       }
       base += __popc(m);
-      if (kind == 1) hbase += __popc(m);
-      if (kind == 0) ninner = base;
     }
+    count[kind] = base - before;
   }
   if (sizeof(T) == 4) reinterpret_cast<int32_t*>(P + (EDGE_INLINE + HALO) / 4)[lane] = valid ? nb.w : 0;
   if (lane == 0)
     reinterpret_cast<int4*>(P)[plan_vec<T>() - 1] =
-        make_int4(meta.x, meta.y, base | ninner << 8 | min(hbase, HALO) << 16, 0);
+        make_int4(meta.x, meta.y, (count[0] + count[1] + count[2]) | count[0] << 8 | min(nhalo, HALO) << 16,
+                  count[3] | count[4] << 8);
 }
 
 // --------------------------------------------------------------------- one tile, one stage ---
@@ -945,17 +978,17 @@ DG_HD constexpr bool storm_regs() {
 // Phases 1-3 of one tile: the area integrals and rain of each lane's element, every edge of the tile
 // once, then the lift, stage combination and positive-depth operator; O is the element's new record.
 // halo_ready() makes the staged halo records readable; it is called once by the whole warp, before
-// the first round that has an edge to another tile; far(element, record) reads a neighbour beyond the
-// halo slots after that; release() is called once by the whole warp when the tile's static data is
+// the first round that has an edge to another tile; halo_more(n) replaces them by the records of the
+// element that each lane names (n < 0: none); release() is called once by the whole warp when the tile's static data is
 // done with.  The step-initial record comes from shared memory (WNS) or from a.wn.
-template <int P, int FLUX, class Pol, int FT, bool WNS, class HaloReady, class Far, class Release>
+template <int P, int FLUX, class Pol, int FT, bool WNS, class HaloReady, class HaloMore, class Release>
 __device__ __forceinline__ void tile_body(const StageArgs<Pol>& a, const ScenDev& S, double t64, int rain_kind, int press,
                                           const RainRec<typename Pol::T>& rr,
-                                          const Storm<typename Pol::T>& storm, int tile, int lane, bool valid, int counts,
+                                          const Storm<typename Pol::T>& storm, int tile, int lane, bool valid, int counts, int more,
                                           const uint4* own, const uint4* halo, const uint4* geoS, const unsigned* planS,
                                           const float* man, const typename Pol::T* xyS, void* flx, const uint4* wnS,
                                           const typename Pol::T (*s_ephi)[P + 1][np_of(P)], const float4* s_ephi4,
-                                          HaloReady halo_ready, Far far, Release release, Elem<P, Pol>& O, typename Pol::Acc& rain_acc,
+                                          HaloReady halo_ready, HaloMore halo_more, Release release, Elem<P, Pol>& O, typename Pol::Acc& rain_acc,
                                           typename Pol::Acc& bdry_acc) {
   using T = typename Pol::T;
   using Acc = typename Pol::Acc;
@@ -1025,16 +1058,26 @@ __device__ __forceinline__ void tile_body(const StageArgs<Pol>& a, const ScenDev
 
   // ---- edge phase: each edge touching the tile once, one per lane and round; the halo records are
   // waited for before the first round that has an edge to another tile
+  const uint32_t ownB = smem_u32(own), halB = smem_u32(halo) - 16u * TILE;
+  const int nr0 = (nedge + 31) >> 5, nr = nr0 + (more ? (more >> 8 ? 2 : 1) : 0);
   bool staged = false;
-  for (int r = 0; r * 32 < nedge; ++r) {
+  int base = 0, lim = nedge;
+  for (int r = 0; r < nr; ++r, base += 32) {
     if (!staged && r * 32 + 32 > ninner) {
       halo_ready();
       staged = true;
     }
-    const int i = r * 32 + lane;
-    if (i < nedge) {
+    if (r >= nr0) {  // further neighbours (rare): their records in place of the ones before, and their edges
+      const int b = r - nr0, n = (more >> (8 * b)) & 255;
+      __syncwarp();
+      halo_more(lane < n ? __ldg(over + 32 + HALO * b + lane) : -1);
+      base = lim;
+      lim += n;
+    }
+    const int i = base + lane;
+    if (i < lim) {
       const unsigned ed = i < EDGE_INLINE ? planS[i] : (unsigned)__ldg(over + (i - EDGE_INLINE));
-      tile_edge<P, FLUX, Pol, FT>(a, S, own, halo, geoS, far, over, flx, ed, s_ephi, s_ephi4, t64, bdry_acc);
+      tile_edge<P, FLUX, Pol, FT>(a, S, ownB, halB, geoS, flx, ed, s_ephi, s_ephi4, t64, bdry_acc);
     }
   }
   if (!staged) halo_ready();
@@ -1053,22 +1096,49 @@ __device__ __forceinline__ void tile_body(const StageArgs<Pol>& a, const ScenDev
       unpack<P>(r, E);
     }
     Acc massout;  // edge mass outflow (volume per second), summed exactly over the three sides
+    if constexpr (slots_sd<P, Pol>()) {
+      // basis over an edge's two points: mean * S + difference / 2 * D, for phi_1 and phi_2 on edges 0, 1, 2
+      constexpr float MID[3][2] = {{0.f, -1.f}, {0.8660254f, 0.5f}, {-0.8660254f, 0.5f}};
+      constexpr float DIF[3][2] = {{1.f, 0.f}, {-0.5f, 0.8660254f}, {-0.5f, -0.8660254f}};
 #pragma unroll
-    for (int j = 0; j < 3; ++j) {
-      T vals[NV + 1];
-      load_side<T, NPR, NV>(flx, lane, j, vals);
+      for (int j = 0; j < 3; ++j) {
+        const float4 zx = reinterpret_cast<const float4*>(flx)[j * 32 + lane];
+        const float2 y = reinterpret_cast<const float2*>(reinterpret_cast<const float4*>(flx) + 96)[j * 32 + lane];
+        Rx[0] = fma(-tab.phi0, zx.z, Rx[0]);
+        Ry[0] = fma(-tab.phi0, y.x, Ry[0]);
 #pragma unroll
-      for (int k = 0; k < NG; ++k) {
-#pragma unroll
-        for (int m = 0; m < NP; ++m) {
-          const T ph_ = tab.ephi[j][k][m];
-          if (m > 0) Rz[m] = fma(-ph_, vals[k], Rz[m]);
-          Rx[m] = fma(-ph_, vals[NG + k], Rx[m]);
-          Ry[m] = fma(-ph_, vals[2 * NG + k], Ry[m]);
+        for (int m = 1; m < 3; ++m) {
+          if (MID[j][m - 1] != 0.f) {
+            Rz[m] = fma(-MID[j][m - 1], zx.x, Rz[m]);
+            Rx[m] = fma(-MID[j][m - 1], zx.z, Rx[m]);
+            Ry[m] = fma(-MID[j][m - 1], y.x, Ry[m]);
+          }
+          if (DIF[j][m - 1] != 0.f) {
+            Rz[m] = fma(-DIF[j][m - 1], zx.y, Rz[m]);
+            Rx[m] = fma(-DIF[j][m - 1], zx.w, Rx[m]);
+            Ry[m] = fma(-DIF[j][m - 1], y.y, Ry[m]);
+          }
         }
+        massout = (j == 0) ? acc_make<Acc>(zx.x, T(0), zx.x) : acc_addr(massout, zx.x);
       }
-      const T ms = side_mass<T, NG, L::MASSV>(vals);
-      massout = (j == 0) ? acc_make<Acc>(ms, T(0), ms) : acc_addr(massout, ms);
+    } else {
+#pragma unroll
+      for (int j = 0; j < 3; ++j) {
+        T vals[NV + 1];
+        load_side<T, NPR, NV>(flx, lane, j, vals);
+#pragma unroll
+        for (int k = 0; k < NG; ++k) {
+#pragma unroll
+          for (int m = 0; m < NP; ++m) {
+            const T ph_ = tab.ephi[j][k][m];
+            if (m > 0) Rz[m] = fma(-ph_, vals[k], Rz[m]);
+            Rx[m] = fma(-ph_, vals[NG + k], Rx[m]);
+            Ry[m] = fma(-ph_, vals[2 * NG + k], Ry[m]);
+          }
+        }
+        const T ms = side_mass<T, NG, L::MASSV>(vals);
+        massout = (j == 0) ? acc_make<Acc>(ms, T(0), ms) : acc_addr(massout, ms);
+      }
     }
     if (E.flags & FLAG_DRY) {  // the momentum equations are not advanced on dry elements
 #pragma unroll
@@ -1148,6 +1218,17 @@ __device__ __forceinline__ void tile_body(const StageArgs<Pol>& a, const ScenDev
 #define DG_TILE_BOUNDS __maxnreg__(DG_TILE_MAXNREG)
 #endif
 
+// the 16-byte rows of edge basis values that side_traces reads
+template <int P, class T>
+__device__ __forceinline__ void edge_rows(const RefTab<T>& tab, float4* rows) {
+  const int t = threadIdx.x;
+  if (P == 1 && t < 3)
+    rows[t] = make_float4((float)tab.ephi[t][0][1], (float)tab.ephi[t][0][2], (float)tab.ephi[t][1][1], (float)tab.ephi[t][1][2]);
+  if (P == 2 && t < 15)
+    rows[t] = make_float4((float)tab.ephi[t / 5][0][t % 5 + 1], (float)tab.ephi[t / 5][1][t % 5 + 1],
+                          (float)tab.ephi[t / 5][2][t % 5 + 1], 0.f);
+}
+
 template <int P, int FLUX, class Pol, int FT = FT_ALL>
 __global__ void DG_TILE_BOUNDS tile_kernel(const StageArgs<Pol> a) {
   using T = typename Pol::T;
@@ -1156,19 +1237,16 @@ __global__ void DG_TILE_BOUNDS tile_kernel(const StageArgs<Pol> a) {
   constexpr int NP = np_of(P), NG = P + 1, RV = L::RV, GV = L::GV;
   const RefTab<T>& tab = ctab<T, P>();
 
-  // edge basis values, read at edge-dependent indices; at p = 1 in FP32 also one 16-byte row per
-  // edge {phi_1, phi_2 at point 0, phi_1, phi_2 at point 1} (phi_0 is constant and not read)
+  // edge basis values, read at edge-dependent indices; in FP32 as rows of 16 bytes (side_traces)
   __shared__ T s_ephi[3][NG][NP];
-  __shared__ float4 s_ephi4[3];
+  __shared__ float4 s_ephi4[P == 1 ? 3 : 15];
   extern __shared__ uint4 tsm[];
   const int tid = threadIdx.x;
   for (int i = tid; i < 3 * NG * NP; i += blockDim.x) {
     const int j = i / (NG * NP), k = (i / NP) % NG, m = i % NP;
     s_ephi[j][k][m] = tab.ephi[j][k][m];
   }
-  if (P == 1 && tid < 3)
-    s_ephi4[tid] = make_float4((float)tab.ephi[tid][0][1], (float)tab.ephi[tid][0][2],
-                               (float)tab.ephi[tid][NG - 1][1], (float)tab.ephi[tid][NG - 1][2]);
+  edge_rows<P>(tab, s_ephi4);
   __syncthreads();
   const int lane = tid & 31;
   uint4* Wm = tsm + (size_t)(tid >> 5) * L::VEC;
@@ -1284,16 +1362,22 @@ __global__ void DG_TILE_BOUNDS tile_kernel(const StageArgs<Pol> a) {
     cp_async_commit();
 
     Elem<P, Pol> O;
-    tile_body<P, FLUX, Pol, FT, false>(a, S, t64, rain_kind, press, rr, storm, tile, lane, valid, meta.z, own, halo, geoS, planS,
+    tile_body<P, FLUX, Pol, FT, false>(a, S, t64, rain_kind, press, rr, storm, tile, lane, valid, meta.z, meta.w, own, halo, geoS, planS,
                                        reinterpret_cast<const float*>(stat + L::S_MAN),
                                        reinterpret_cast<const T*>(stat + L::S_XY), flx, nullptr, s_ephi, s_ephi4,
                                        [] {
                                          cp_async_wait_all();
                                          __syncwarp();
                                        },
-                                       [&](int n, Raw<RV>& r) {
+                                       [&](int n) {
+                                         if (n >= 0) {
 #pragma unroll
-                                         for (int v = 0; v < RV; ++v) r.v[v] = __ldg(a.in + rec_at<RV>(n, v));
+                                           for (int v = 0; v < RV; ++v)
+                                             cp_async16(halo + v * HALO + lane, a.in + rec_at<RV>(n, v));
+                                         }
+                                         cp_async_commit();
+                                         cp_async_wait_all();
+                                         __syncwarp();
                                        },
                                        [&] {
                                          if (SD) return;
