@@ -125,7 +125,7 @@ struct dgswe_ctx {
   int np = 0, rv = 0, gv = 0;      // modes, record and geometry sizes (16-byte units)
   long long E = 0, N = 0;          // padded element count, node count
   std::vector<long long> eoff, noff;
-  DevBuf rec[3], nbr, geo, nodes, node_xy, xy64, hbn, rain_e, rain_node, node_scen, lim, rain_rec, scen, tile_scen, tile_meta, plan, plan_x, xy0,
+  DevBuf rec[3], nbr, geo, nodes, node_xy, xy64, hbn, rain_e, rain_node, node_scen, lim, rain_rec, scen, tile_scen, tile_meta, stat, plan_x,
       ledger, ctl,
       einv, grids, rivers, scratch,
       gather_buf, edges, slots;
@@ -156,9 +156,9 @@ struct dgswe_ctx {
   ~dgswe_ctx() {
     DeviceGuard dg_(device);
     DevBuf* bufs[] = {&rec[0], &rec[1], &rec[2], &nbr, &geo, &nodes, &node_xy, &xy64, &hbn, &rain_e, &scen,
-                      &tile_scen, &tile_meta, &xy0, &ledger, &ctl, &einv, &grids, &rivers, &scratch, &gather_buf,
+                      &tile_scen, &tile_meta, &ledger, &ctl, &einv, &grids, &rivers, &scratch, &gather_buf,
                       &edges, &slots,
-                      &rain_node, &node_scen, &lim, &rain_rec, &plan, &plan_x};
+                      &rain_node, &node_scen, &lim, &rain_rec, &stat, &plan_x};
     for (DevBuf* b : bufs) b->alloc(0);
     if (sum) cudaFreeHost(sum);
     if (g1) cudaGraphExecDestroy(g1);
@@ -366,8 +366,6 @@ static int build_layout(dgswe_h h) {
   const size_t rw = 4 * (size_t)h->rv, gw = 4 * (size_t)h->gv;  // 32-bit words per element
   std::vector<uint32_t> rec(rw * E, 0u), geo(gw * E, 0u);
   std::vector<int32_t> nbr(4 * E, -1), nodes(4 * E, 0), einv(E, 0);
-  std::vector<float> xy0f(mx ? 2 * E : 0, 0.f);     // first vertex of each element (tile form)
-  std::vector<double> xy0d(mx ? 0 : 2 * E, 0.0);
   std::vector<double> xy64(2 * N), hbn(N);
   std::vector<int32_t> nscen(N, 0);
   std::vector<float> xyf(mx ? 2 * N : 0), rainf(mx ? E : 0);
@@ -393,13 +391,6 @@ static int build_layout(dgswe_h h) {
       const long long ge = eo + e;
       const int32_t* v = &M.tri[3 * (size_t)e];
       einv[eo + M.eorig[e]] = e;  // caller element -> position in the library's order
-      if (mx) {
-        xy0f[2 * ge] = (float)M.x[v[0]];
-        xy0f[2 * ge + 1] = (float)M.y[v[0]];
-      } else {
-        xy0d[2 * ge] = M.x[v[0]];
-        xy0d[2 * ge + 1] = M.y[v[0]];
-      }
       for (int j = 0; j < 3; ++j) {
         const int32_t c = M.code[3 * (size_t)e + j];
         nbr[4 * ge + j] = c >= 0 ? (int32_t)((((c >> 2) + eo) << 2) | (c & 3)) : c;
@@ -523,9 +514,6 @@ static int build_layout(dgswe_h h) {
   CU(cudaMemcpy(h->xy64.p, xy64.data(), 8 * xy64.size(), cudaMemcpyHostToDevice));
   CU(cudaMemcpy(h->hbn.p, hbn.data(), 8 * hbn.size(), cudaMemcpyHostToDevice));
   CU(cudaMemcpy(h->einv.p, einv.data(), 4 * einv.size(), cudaMemcpyHostToDevice));
-  if (h->xy0.alloc(mx ? 8 * (size_t)E : 16 * (size_t)E)) return fail(DGSWE_ENOMEM, "device allocation failed");
-  if (mx) CU(cudaMemcpy(h->xy0.p, xy0f.data(), 4 * xy0f.size(), cudaMemcpyHostToDevice));
-  else CU(cudaMemcpy(h->xy0.p, xy0d.data(), 8 * xy0d.size(), cudaMemcpyHostToDevice));
   if (mx) {
     CU(cudaMemcpy(h->node_xy.p, xyf.data(), 4 * xyf.size(), cudaMemcpyHostToDevice));
     CU(cudaMemcpy(h->rain_e.p, rainf.data(), 4 * rainf.size(), cudaMemcpyHostToDevice));
@@ -634,10 +622,11 @@ static int build_layout(dgswe_h h) {
   size_t pb = 0, pxb = 0;
   if (mx) plan_bytes<Mixed>(h->ntiles, pb, pxb);
   else plan_bytes<Fp64>(h->ntiles, pb, pxb);
-  if (h->plan.alloc(pb) || h->plan_x.alloc(pxb)) return fail(DGSWE_ENOMEM, "device allocation failed");
+  if (h->stat.alloc(pb) || h->plan_x.alloc(pxb)) return fail(DGSWE_ENOMEM, "device allocation failed");
   CU(cudaDeviceSynchronize());  // the uploads above ran on the default stream, this stream does not wait for it
-  CU(mx ? launch_plan<Mixed>(h->nbr.as<int4>(), h->tile_meta.as<int4>(), h->ntiles, h->plan.as<uint4>(), h->plan_x.as<int32_t>(), h->stream)
-        : launch_plan<Fp64>(h->nbr.as<int4>(), h->tile_meta.as<int4>(), h->ntiles, h->plan.as<uint4>(), h->plan_x.as<int32_t>(), h->stream));
+  CU((mx ? launch_plan<Mixed> : launch_plan<Fp64>)(h->nbr.as<int4>(), h->geo.as<uint4>(), h->nodes.as<int4>(),
+                                                   h->xy64.as<double>(), h->tile_meta.as<int4>(), h->ntiles, h->rv,
+                                                   h->stat.as<uint4>(), h->plan_x.as<int32_t>(), h->stream));
   h->launches++;
   h->wcur = 0;
   CU(cudaMemcpy(h->scen.p, sd.data(), sizeof(ScenDev) * ns, cudaMemcpyHostToDevice));
@@ -723,9 +712,8 @@ static StageArgs<Pol> make_args(dgswe_h h, int stage, int tune) {
   a.scen = h->scen.as<ScenDev>();
   a.tile_scen = h->tile_scen.as<int32_t>();
   a.tile_meta = h->tile_meta.as<int4>();
-  a.plan = h->plan.as<uint4>();
+  a.stat = h->stat.as<uint4>();
   a.plan_x = h->plan_x.as<int32_t>();
-  a.xy0 = h->xy0.as<uint4>();
   a.ledger = h->ledger.as<double>();
   a.ctl = h->ctl.as<Ctl>();
   a.edges = h->edges.as<uint4>();

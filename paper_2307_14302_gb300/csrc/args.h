@@ -41,9 +41,8 @@ struct StageArgs {
   const ScenDev* scen;
   const int32_t* tile_scen;  // scenario of each 32-element tile
   const int4* tile_meta;   // tile form: per tile {scenario, elements present (0..32), 0, 0}
-  const uint4* plan;       // tile form: per tile the edge words, halo elements, Manning, meta (tile.cuh)
+  const uint4* stat;       // tile form: static block per tile: geometry, plan, first vertices (tile.cuh)
   const int32_t* plan_x;   // tile form: overflow of the plan, PLAN_X words per tile
-  const uint4* xy0;        // tile form: first vertex of each element, [E] float2 (mixed) / double2 (FP64)
   double* ledger;          // [scenario][wslots][2]: rain volume, boundary inflow volume per warp
   Ctl* ctl;
   const uint4* edges;      // edge-split path: interior edge records
@@ -162,11 +161,12 @@ int tile_spec_blocks_per_sm(int p, int flux, int feat, int block);
 int tile_spec_features(int p, int flux, int feat);
 // reference tables and shared-memory limits of the specialised instantiations' translation unit
 cudaError_t upload_tile_spec_tables(int p, const RefTab<float>& tf, const RefTab<double>& td);
-// tile plans of the mesh (sizes: plan_bytes), from the neighbour codes and the tiles' metadata
+// static blocks of the mesh's tiles (sizes: plan_bytes; rv: 16-byte vectors per record)
 template <class Pol>
-cudaError_t launch_plan(const int4* nbr, const int4* tile_meta, int ntiles, uint4* plan, int32_t* plan_x, cudaStream_t s);
+cudaError_t launch_plan(const int4* nbr, const uint4* geo, const int4* nodes, const double* xy, const int4* tile_meta,
+                        int ntiles, int rv, uint4* stat, int32_t* plan_x, cudaStream_t s);
 template <class Pol>
-void plan_bytes(int ntiles, size_t& plan, size_t& plan_x);
+void plan_bytes(int ntiles, size_t& stat, size_t& plan_x);
 // edge kernel of the split path: one thread per interior edge, writes both sides' slots
 template <class Pol>
 cudaError_t launch_edges(int p, int flux, const StageArgs<Pol>& a, int grid, int block, cudaStream_t s);

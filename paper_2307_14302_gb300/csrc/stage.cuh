@@ -91,6 +91,30 @@ __device__ __forceinline__ ff acc_addf(ff a, ff b) {
   ff s = two_sum(a.hi, b.hi);
   return quick_two_sum(s.hi, __fadd_rn(s.lo, __fadd_rn(a.lo, b.lo)));
 }
+// sum of three values as a pair, and the stage's increment bdt (r - m inv): intermediate pairs are not
+// renormalised (their low words stay within a few ulps of the high ones, so the products and sums keep
+// the same 2^-47), which saves 3 operations each time
+__device__ __forceinline__ ff acc_sum3(float a, float b, float c, ff) {
+  const ff s = two_sum(a, b), t = two_sum(s.hi, c);
+  return {t.hi, __fadd_rn(t.lo, s.lo)};
+}
+__device__ __forceinline__ double acc_sum3(double a, double b, double c, double) { return a + b + c; }
+__device__ __forceinline__ ff mul_raw(ff a, ff b) {
+  const float p = __fmul_rn(a.hi, b.hi);
+  return {p, __fmaf_rn(a.lo, b.hi, __fmaf_rn(a.hi, b.lo, __fmaf_rn(a.hi, b.hi, -p)))};
+}
+__device__ __forceinline__ double acc_increment(double bdt, double r, double m, double inv) { return bdt * (r - m * inv); }
+__device__ __forceinline__ ff acc_increment(ff bdt, float r, ff m, ff inv) {
+  const ff t = mul_raw(m, inv), s = two_sum(r, -t.hi);
+  return mul_raw(bdt, {s.hi, __fsub_rn(s.lo, t.lo)});
+}
+// s + a b accumulated without renormalising s (a ledger sum over a warp's tiles)
+__device__ __forceinline__ double acc_addmul(double s, double a, double b) { return s + a * b; }
+__device__ __forceinline__ ff acc_addmul(ff s, ff a, float b) {
+  const float p = __fmul_rn(a.hi, b);
+  const ff t = two_sum(s.hi, p);
+  return {t.hi, __fadd_rn(s.lo, __fadd_rn(t.lo, __fmaf_rn(a.lo, b, __fmaf_rn(a.hi, b, -p))))};
+}
 // a - b rounded to the working precision (float: within an ulp, from the words' differences)
 __device__ __forceinline__ double acc_sub_r(double a, double b) { return a - b; }
 __device__ __forceinline__ float acc_sub_r(ff a, ff b) { return __fadd_rn(__fsub_rn(a.hi, b.hi), __fsub_rn(a.lo, b.lo)); }
@@ -496,7 +520,7 @@ __device__ __forceinline__ Trace<typename Pol::T> trace_p1(const Elem<1, Pol>& E
   t.d = fma(E.zs[1], p2, E.zs[0] * p1);
   t.qx = fma(E.xs[1], p2, fma(E.xs[0], p1, acc_r(E.xb)));
   t.qy = fma(E.ys[1], p2, fma(E.ys[0], p1, acc_r(E.yb)));
-  t.H = E.Hb + (t.d + fma(E.hb1, p1, E.hb2 * p2));
+  t.H = fma(E.zs[0] + E.hb1, p1, fma(E.zs[1] + E.hb2, p2, E.Hb));
   return t;
 }
 

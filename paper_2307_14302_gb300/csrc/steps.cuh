@@ -59,7 +59,7 @@ __global__ void __maxnreg__(sizeof(typename Pol::T) == 4 ? (P == 1 ? 128 : 200) 
   using Acc = typename Pol::Acc;
   using L = TileLayout<P, Pol, FT>;
   using SL = StepsLayout<P, Pol, FT>;
-  constexpr int NP = np_of(P), NG = P + 1, RV = L::RV, GV = L::GV;
+  constexpr int NP = np_of(P), NG = P + 1, RV = L::RV;
   const RefTab<T>& tab = ctab<T, P>();
   __shared__ T s_ephi[3][NG][NP];
   __shared__ float4 s_ephi4[P == 1 ? 3 : 15];
@@ -78,23 +78,23 @@ __global__ void __maxnreg__(sizeof(typename Pol::T) == 4 ? (P == 1 ? 128 : 200) 
   StageArgs<Pol> a = a0;
   int4 meta = make_int4(0, 0, 0, 0);
   if (tile < a.ntiles) {
-    meta = reinterpret_cast<const int4*>(a.plan + (size_t)tile * L::PV)[L::PV - 1];
-    for (int i = lane; i < TILE * GV; i += 32) Wm[SL::GEO + i] = __ldg(a.geo + (size_t)tile * TILE * GV + i);
-    for (int i = lane; i < L::PV; i += 32) Wm[SL::PLAN + i] = __ldg(a.plan + (size_t)tile * L::PV + i);
-    for (int i = lane; i < L::XV; i += 32) Wm[SL::XY + i] = __ldg(a.xy0 + (size_t)tile * L::XV + i);
+    const uint4* from = a.stat + (size_t)tile * L::SVM;
+    meta = reinterpret_cast<const int4*>(from)[L::S_META];
+    for (int i = lane; i < L::SV; i += 32) Wm[i] = __ldg(from + i);
     for (int i = lane; i < SL::RECS; i += 32) Wm[SL::REC + i] = a.wn[(size_t)tile * SL::RECS + i];
   }
   const int sc = meta.x, present = meta.y, nhalo = meta.z >> 16;
   const bool valid = lane < present;
   __syncthreads();  // edge basis table; the tile's data is read by its own warp and, after the cluster barrier, by others
   cluster_arrive();
-  // address of element n's record in buffer 0 of its CTA, and that of this lane's halo neighbour
-  auto remote = [&](int n) {
-    const int nt = n >> 5;
-    return cluster_map(smem_u32(tsm + (size_t)(nt % wpc) * vec + SL::REC) + 16u * (n & 31), (uint32_t)(nt / wpc));
+  // address, in buffer 0 of its CTA, of the record at a place of the record array, and that of this
+  // lane's halo neighbour
+  auto remote = [&](uint32_t at) {
+    const uint32_t nt = at / (uint32_t)(TILE * RV);
+    return cluster_map(smem_u32(tsm + (size_t)(nt % wpc) * vec + SL::REC) + 16u * (at & 31), nt / (uint32_t)wpc);
   };
   const uint32_t hsrc =
-      lane < nhalo ? remote(reinterpret_cast<const int32_t*>(Wm + L::S_HALO)[lane]) : 0u;
+      lane < nhalo ? remote(reinterpret_cast<const uint32_t*>(Wm + L::S_HALO)[lane]) : 0u;
   const ScenDev& S = a.scen[sc];
   const unsigned long long step0 = a.ctl->step;
   const int rain_kind = ft_rain(FT) >= 0 ? ft_rain(FT) : S.rain_kind;
@@ -149,12 +149,12 @@ __global__ void __maxnreg__(sizeof(typename Pol::T) == 4 ? (P == 1 ? 128 : 200) 
                                         reinterpret_cast<const float*>(Wm + L::S_MAN),
                                         reinterpret_cast<const T*>(Wm + SL::XY), Wm + SL::FLX, Wm + SL::REC, s_ephi,
                                         s_ephi4, halo_ready,
-                                        [&](int n) {
-                                          if (n >= 0) {
-                                            const uint32_t at = remote(n) + rin;
+                                        [&](bool mine, uint32_t at) {
+                                          if (mine) {
+                                            const uint32_t from = remote(at) + rin;
 #pragma unroll
                                             for (int v = 0; v < RV; ++v)
-                                              halo[v * HALO + lane] = ld_cluster128(at + 16u * TILE * v);
+                                              halo[v * HALO + lane] = ld_cluster128(from + 16u * TILE * v);
                                           }
                                           __syncwarp();
                                         },

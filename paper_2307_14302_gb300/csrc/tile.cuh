@@ -61,6 +61,9 @@ constexpr int TE_MAX = 96;  // edges touching a 32-element tile (3 per element a
 // EDGE_INLINE words, the first 32 halo elements, (mixed path) the Manning coefficients, and {scenario,
 // elements present, counts, further batches}; the words 64-95 and the further neighbours are in the
 // overflow array.
+// The plan lies between the tile's geometry and its first vertices in one block per tile (the static
+// block), so that one bulk copy brings everything that does not change; a halo entry is the place of
+// the neighbour's first record vector, (n / 32) RV 32 + n % 32.
 // Before, every stage rebuilt this per tile from the neighbour codes (nine ballots, the population
 // counts, a descriptor of two sides and a normal per edge): about 190 of 1,940 warp instructions,
 // with the halo loads waiting for it.
@@ -95,6 +98,7 @@ struct TileLayout {
   static constexpr int S_META = S_PLAN + PV - 1;
   static constexpr int S_XY = S_PLAN + PV;
   static constexpr int SV = S_XY + XV;
+  static constexpr int SVM = S_XY + (sizeof(T) == 4 ? 16 : 32);  // in memory (first vertices always there)
   // per warp: two record buffers [RV][32] (the tile's block of the tile-blocked record array), the
   // static buffers, the halo records [RV][HALO], the edge slots [3][NPR][32] (pairs of T) and three
   // 8-byte mbarriers (buffers 0 and 1, single static).  Mixed p = 2 has one static buffer: the static
@@ -347,14 +351,11 @@ __device__ __forceinline__ void tile_area(const Elem<P, Pol>& E, const Geo<Pol>&
   const T g = a.g, H0 = a.H0;
   const T detJ = T(0.5) * acc_r(G.A);
   const T idetJ = T(2) * acc_r(G.invA);
-  // inverse Jacobian from the edge vectors: t0 = x1 - x0 = 2 (xr, yr), t2 = x0 - x2 = -2 (xs, ys)
-  // and ln_j = (t_j.y, -t_j.x)
-  const T xr = T(-0.5) * G.lny[0], yr = T(0.5) * G.lnx[0];
-  const T xs = T(0.5) * G.lny[2], ys = T(-0.5) * G.lnx[2];
-  const T rx = ys * idetJ, ry = -xs * idetJ, sx = -yr * idetJ, sy = xr * idetJ;
-  const T g1x = tab.qdr[0][1] * rx + tab.qds[0][1] * sx, g1y = tab.qdr[0][1] * ry + tab.qds[0][1] * sy;
-  const T g2x = tab.qdr[0][2] * rx + tab.qds[0][2] * sx, g2y = tab.qdr[0][2] * ry + tab.qds[0][2] * sy;
-  const T hbx = E.hb1 * g1x + E.hb2 * g2x, hby = E.hb1 * g1y + E.hb2 * g2y;  // constant grad(hb)
+  // detJ grad(phi_1) and detJ grad(phi_2) of the linear modes phi_1 = sqrt(3) (lambda_1 - lambda_0),
+  // phi_2 = 3 lambda_2 - 1: the barycentric gradients are -1 / (2 A) times the opposite edges' scaled normals
+  const T G1x = T(0.4330127018922193) * (G.lnx[1] - G.lnx[2]), G1y = T(0.4330127018922193) * (G.lny[1] - G.lny[2]);
+  const T G2x = T(-0.75) * G.lnx[0], G2y = T(-0.75) * G.lny[0];
+  const T hbx = idetJ * (E.hb1 * G1x + E.hb2 * G2x), hby = idetJ * (E.hb1 * G1y + E.hb2 * G2y);  // constant grad(hb)
   const int friction = ft_friction(FT) >= 0 ? ft_friction(FT) : a.friction;
   const T cfm = (friction == 0) ? g * G.man * G.man : a.cf;
   if constexpr (P == 1) {
@@ -437,17 +438,22 @@ __device__ __forceinline__ void tile_area(const Elem<P, Pol>& E, const Geo<Pol>&
         SS[m][1] = A1.SS[m][1];
       }
     }
-    const T gx[3] = {T(0), g1x, g2x}, gy[3] = {T(0), g1y, g2y};
+    const T gx[3] = {T(0), G1x, G2x}, gy[3] = {T(0), G1y, G2y};
+    Rz[0] = T(0);
+    Rx[0] = detJ * SS[0][0];
+    Ry[0] = detJ * SS[0][1];
 #pragma unroll
-    for (int m = 0; m < NP; ++m) {
-      Rz[m] = (m > 0) ? detJ * (gx[m] * SF[0] + gy[m] * SF[3]) : T(0);
-      Rx[m] = (m > 0) ? detJ * (gx[m] * SF[1] + gy[m] * SF[2] + SS[m][0]) : detJ * SS[m][0];
-      Ry[m] = (m > 0) ? detJ * (gx[m] * SF[2] + gy[m] * SF[4] + SS[m][1]) : detJ * SS[m][1];
+    for (int m = 1; m < NP; ++m) {
+      Rz[m] = gx[m] * SF[0] + gy[m] * SF[3];
+      Rx[m] = fma(detJ, SS[m][0], gx[m] * SF[1] + gy[m] * SF[2]);
+      Ry[m] = fma(detJ, SS[m][1], gx[m] * SF[2] + gy[m] * SF[4]);
     }
   } else if constexpr (sizeof(T) == 4 && DG_PACKED_FLUX) {
     // FP32: the points in packed pairs (0,1), (2,3), (4,5), (6,7); point 7 has zero weight and zero
     // basis values (the mean state, finite) and adds exact zeros
     static_assert(NQ + 1 == MAXNQP, "one padding point");
+    // gradients of r and s: the barycentric gradients of vertices 1 and 2, times 2
+    const T h = T(-0.5) * idetJ, rx = h * G.lnx[2], ry = h * G.lny[2], sx = h * G.lnx[0], sy = h * G.lny[0];
     constexpr int NS = NP - 1;
     f2 Rz2[NP], Rx2[NP], Ry2[NP];
 #pragma unroll
@@ -508,6 +514,7 @@ __device__ __forceinline__ void tile_area(const Elem<P, Pol>& E, const Geo<Pol>&
       Ry[m] = Ry2[m].x + Ry2[m].y;
     }
   } else {
+    const T h = T(-0.5) * idetJ, rx = h * G.lnx[2], ry = h * G.lny[2], sx = h * G.lnx[0], sy = h * G.lny[0];
 #pragma unroll
     for (int m = 0; m < NP; ++m) Rz[m] = Rx[m] = Ry[m] = T(0);
 #pragma unroll
@@ -885,9 +892,12 @@ __device__ __forceinline__ void tile_edge(const StageArgs<Pol>& a, const ScenDev
 // one warp per tile, once per mesh: ownership of the tile's edges (boundary edges, edges to
 // out-of-tile neighbours and in-tile edges to a higher index belong to a lane's element; the lower
 // element index is the left side) and the order described at EDGE_INLINE
-template <class T>
-__global__ void __launch_bounds__(256) plan_kernel(const int4* nbr, const int4* tile_meta, int ntiles, uint4* plan,
+template <class Pol>
+__global__ void __launch_bounds__(256) plan_kernel(const int4* nbr, const uint4* geo, const int4* nodes, const double* xy,
+                                                   const int4* tile_meta, int ntiles, int rv, uint4* stat,
                                                    int32_t* plan_x) {
+  using T = typename Pol::T;
+  using L = TileLayout<1, Pol>;  // the static block does not depend on the degree
   const int tile = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (tile >= ntiles) return;
   const int4 meta = tile_meta[tile];
@@ -895,14 +905,22 @@ __global__ void __launch_bounds__(256) plan_kernel(const int4* nbr, const int4* 
   const int e0 = tile * TILE, e = e0 + lane;
   const int4 nb = valid ? nbr[e] : make_int4(-1, -1, -1, 0);
   const int code[3] = {nb.x, nb.y, nb.z};
-  const unsigned lt = (1u << lane) - 1u;
-  uint4* P = plan + (size_t)tile * plan_vec<T>();
+  uint4* B = stat + (size_t)tile * L::SVM;
+  for (int i = lane; i < TILE * L::GV; i += 32) B[i] = geo[(size_t)tile * TILE * L::GV + i];
+  {
+    const long long v = valid ? nodes[e].x : 0;
+    T* x0 = reinterpret_cast<T*>(B + L::S_XY) + 2 * lane;
+    x0[0] = valid ? (T)xy[2 * v] : T(0);
+    x0[1] = valid ? (T)xy[2 * v + 1] : T(0);
+  }
+  uint4* P = B + L::S_PLAN;
   unsigned* desc = reinterpret_cast<unsigned*>(P);
   int32_t* halo = reinterpret_cast<int32_t*>(P + EDGE_INLINE / 4);
   int32_t* over = plan_x + (size_t)tile * PLAN_X;
   for (int i = lane; i < EDGE_INLINE + HALO; i += 32) desc[i] = 0u;
   for (int i = lane; i < PLAN_X; i += 32) over[i] = 0;
   __syncwarp();
+  const unsigned lt = (1u << lane) - 1u;
   // halo slot of each edge to another tile
   int hs[3], nhalo = 0;
 #pragma unroll
@@ -912,8 +930,9 @@ __global__ void __launch_bounds__(256) plan_kernel(const int4* nbr, const int4* 
     const unsigned m = __ballot_sync(0xffffffffu, out);
     hs[j] = out ? nhalo + __popc(m & lt) : -1;
     if (out) {
-      if (hs[j] < HALO) halo[hs[j]] = n;
-      else over[hs[j]] = n;  // neighbour 32 and on, after the 32 edge words
+      const int32_t at = (int32_t)(((unsigned)n >> 5) * rv * 32 + (n & 31));
+      if (hs[j] < HALO) halo[hs[j]] = at;
+      else over[hs[j]] = at;  // neighbour 32 and on, after the 32 edge words
     }
     nhalo += __popc(m);
   }
@@ -978,8 +997,8 @@ DG_HD constexpr bool storm_regs() {
 // Phases 1-3 of one tile: the area integrals and rain of each lane's element, every edge of the tile
 // once, then the lift, stage combination and positive-depth operator; O is the element's new record.
 // halo_ready() makes the staged halo records readable; it is called once by the whole warp, before
-// the first round that has an edge to another tile; halo_more(n) replaces them by the records of the
-// element that each lane names (n < 0: none); release() is called once by the whole warp when the tile's static data is
+// the first round that has an edge to another tile; halo_more(mine, at) replaces them by the
+// records at the places that the lanes name; release() is called once by the whole warp when the tile's static data is
 // done with.  The step-initial record comes from shared memory (WNS) or from a.wn.
 template <int P, int FLUX, class Pol, int FT, bool WNS, class HaloReady, class HaloMore, class Release>
 __device__ __forceinline__ void tile_body(const StageArgs<Pol>& a, const ScenDev& S, double t64, int rain_kind, int press,
@@ -1070,7 +1089,7 @@ __device__ __forceinline__ void tile_body(const StageArgs<Pol>& a, const ScenDev
     if (r >= nr0) {  // further neighbours (rare): their records in place of the ones before, and their edges
       const int b = r - nr0, n = (more >> (8 * b)) & 255;
       __syncwarp();
-      halo_more(lane < n ? __ldg(over + 32 + HALO * b + lane) : -1);
+      halo_more(lane < n, (uint32_t)__ldg(over + 32 + HALO * b + lane));
       base = lim;
       lim += n;
     }
@@ -1095,7 +1114,7 @@ __device__ __forceinline__ void tile_body(const StageArgs<Pol>& a, const ScenDev
       for (int v = 0; v < RV; ++v) r.v[v] = own[v * TILE + lane];
       unpack<P>(r, E);
     }
-    Acc massout;  // edge mass outflow (volume per second), summed exactly over the three sides
+    T ms[3];  // edge mass outflows (volume per second)
     if constexpr (slots_sd<P, Pol>()) {
       // basis over an edge's two points: mean * S + difference / 2 * D, for phi_1 and phi_2 on edges 0, 1, 2
       constexpr float MID[3][2] = {{0.f, -1.f}, {0.8660254f, 0.5f}, {-0.8660254f, 0.5f}};
@@ -1119,7 +1138,7 @@ __device__ __forceinline__ void tile_body(const StageArgs<Pol>& a, const ScenDev
             Ry[m] = fma(-DIF[j][m - 1], y.y, Ry[m]);
           }
         }
-        massout = (j == 0) ? acc_make<Acc>(zx.x, T(0), zx.x) : acc_addr(massout, zx.x);
+        ms[j] = zx.x;
       }
     } else {
 #pragma unroll
@@ -1136,8 +1155,7 @@ __device__ __forceinline__ void tile_body(const StageArgs<Pol>& a, const ScenDev
             Ry[m] = fma(-ph_, vals[2 * NG + k], Ry[m]);
           }
         }
-        const T ms = side_mass<T, NG, L::MASSV>(vals);
-        massout = (j == 0) ? acc_make<Acc>(ms, T(0), ms) : acc_addr(massout, ms);
+        ms[j] = side_mass<T, NG, L::MASSV>(vals);
       }
     }
     if (E.flags & FLAG_DRY) {  // the momentum equations are not advanced on dry elements
@@ -1149,9 +1167,11 @@ __device__ __forceinline__ void tile_body(const StageArgs<Pol>& a, const ScenDev
     const Acc an = acc_make<Acc>(a.a_n_hi, a.a_n_lo, a.a_n);
     const Acc ain = acc_make<Acc>(a.a_in_hi, a.a_in_lo, a.a_in);
     const Acc bdt = acc_make<Acc>(S.bdt_hi[a.stage], S.bdt_lo[a.stage], S.bdt[a.stage]);
-    // mean rates: d(zeta_bar)/dt = R_e - massout / A;  d(q_bar)/dt = phi_0 R_0 / detJ
-    const Acc zrate = acc_addr(acc_neg(acc_mul(massout, G.invA)), Re);
-    const T xrate = tab.phi0 * Rx[0] * idetJ, yrate = tab.phi0 * Ry[0] * idetJ;
+    // increments of the means: beta dt (R_e - outflow / A) and beta dt phi_0 R_0 / detJ
+    const Acc massout = acc_sum3(ms[0], ms[1], ms[2], acc_make<Acc>(0.f, 0.f, 0.0));
+    const Acc dz = acc_increment(bdt, Re, massout, G.invA);
+    const T fR = acc_r(bdt) * idetJ;
+    const T dx = (tab.phi0 * fR) * Rx[0], dy = (tab.phi0 * fR) * Ry[0];
     O = E;
     Elem<P, Pol> Wn = E;
     if (a.has_n) {
@@ -1183,27 +1203,48 @@ __device__ __forceinline__ void tile_body(const StageArgs<Pol>& a, const ScenDev
           y = acc_add(y, acc_mul(an, Wn.yb));
         }
       }
-      O.zb = acc_addf(z, acc_mul(bdt, zrate));
-      O.xb = acc_addr(x, acc_r(bdt) * xrate);
-      O.yb = acc_addr(y, acc_r(bdt) * yrate);
+      O.zb = acc_addf(z, dz);
+      O.xb = acc_addr(x, dx);
+      O.yb = acc_addr(y, dy);
     }
-    const T bdt_r = acc_r(bdt);
+    // other modes: in FP32 two modes per packed operation
+    if constexpr (sizeof(T) == 4 && DG_PACKED_FLUX) {
+      const f2 f2R = p2(fR), ai2 = p2(ain_r), an2 = p2(an_r);
+      auto comb = [&](const T* w, const T* wn, const T* R, T* o) {
 #pragma unroll
-    for (int m = 0; m < NS; ++m) {
-      T z = ain_r * E.zs[m] + bdt_r * (Rz[m + 1] * idetJ);
-      T x = ain_r * E.xs[m] + bdt_r * (Rx[m + 1] * idetJ);
-      T y = ain_r * E.ys[m] + bdt_r * (Ry[m + 1] * idetJ);
-      if (a.has_n) {
-        z = fma(an_r, Wn.zs[m], z);
-        x = fma(an_r, Wn.xs[m], x);
-        y = fma(an_r, Wn.ys[m], y);
+        for (int m = 0; m + 1 < NS; m += 2) {
+          f2 v = fma2(f2R, make_float2(R[m + 1], R[m + 2]), mul2(ai2, make_float2(w[m], w[m + 1])));
+          if (a.has_n) v = fma2(an2, make_float2(wn[m], wn[m + 1]), v);
+          o[m] = v.x;
+          o[m + 1] = v.y;
+        }
+        if (NS % 2) {
+          T v = fma(fR, R[NS], ain_r * w[NS - 1]);
+          if (a.has_n) v = fma(an_r, wn[NS - 1], v);
+          o[NS - 1] = v;
+        }
+      };
+      comb(E.zs, Wn.zs, Rz, O.zs);
+      comb(E.xs, Wn.xs, Rx, O.xs);
+      comb(E.ys, Wn.ys, Ry, O.ys);
+    } else {
+#pragma unroll
+      for (int m = 0; m < NS; ++m) {
+        T z = fma(fR, Rz[m + 1], ain_r * E.zs[m]);
+        T x = fma(fR, Rx[m + 1], ain_r * E.xs[m]);
+        T y = fma(fR, Ry[m + 1], ain_r * E.ys[m]);
+        if (a.has_n) {
+          z = fma(an_r, Wn.zs[m], z);
+          x = fma(an_r, Wn.xs[m], x);
+          y = fma(an_r, Wn.ys[m], y);
+        }
+        O.zs[m] = z;
+        O.xs[m] = x;
+        O.ys[m] = y;
       }
-      O.zs[m] = z;
-      O.xs[m] = x;
-      O.ys[m] = y;
     }
     apply_positivity<P, Pol>(O, G, e, a, &a.ctl->err);
-    rain_acc = acc_addf(rain_acc, acc_mulr(G.A, Re));
+    rain_acc = acc_addmul(rain_acc, G.A, Re);
   }
 }
 
@@ -1234,7 +1275,7 @@ __global__ void DG_TILE_BOUNDS tile_kernel(const StageArgs<Pol> a) {
   using T = typename Pol::T;
   using Acc = typename Pol::Acc;
   using L = TileLayout<P, Pol, FT>;
-  constexpr int NP = np_of(P), NG = P + 1, RV = L::RV, GV = L::GV;
+  constexpr int NP = np_of(P), NG = P + 1, RV = L::RV;
   const RefTab<T>& tab = ctab<T, P>();
 
   // edge basis values, read at edge-dependent indices; in FP32 as rows of 16 bytes (side_traces)
@@ -1266,9 +1307,7 @@ __global__ void DG_TILE_BOUNDS tile_kernel(const StageArgs<Pol> a) {
   // the records' barrier when they are double-buffered too
   constexpr bool SD = L::NSTAT == 2;
   auto copy_static = [&](int t, uint4* to, uint32_t br) {
-    bulk_g2s(smem_u32(to + L::S_GEO), a.geo + (size_t)t * TILE * GV, 16u * TILE * GV, br);
-    bulk_g2s(smem_u32(to + L::S_PLAN), a.plan + (size_t)t * L::PV, 16u * L::PV, br);
-    if constexpr (L::XV > 0) bulk_g2s(smem_u32(to + L::S_XY), a.xy0 + (size_t)t * L::XV, 16u * L::XV, br);
+    bulk_g2s(smem_u32(to), a.stat + (size_t)t * L::SVM, 16u * L::SV, br);
   };
   auto issue = [&](int t, int b, bool stat, bool rec) {
     if (lane == 0) {
@@ -1355,9 +1394,9 @@ __global__ void DG_TILE_BOUNDS tile_kernel(const StageArgs<Pol> a) {
 
     // ---- the out-of-tile neighbours' records, one halo slot per lane, by the tile's plan
     if (lane < (meta.z >> 16)) {
-      const int n = reinterpret_cast<const int32_t*>(stat + L::S_HALO)[lane];
+      const uint4* from = a.in + reinterpret_cast<const uint32_t*>(stat + L::S_HALO)[lane];
 #pragma unroll
-      for (int v = 0; v < RV; ++v) cp_async16(halo + v * HALO + lane, a.in + rec_at<RV>(n, v));
+      for (int v = 0; v < RV; ++v) cp_async16(halo + v * HALO + lane, from + v * TILE);
     }
     cp_async_commit();
 
@@ -1369,11 +1408,11 @@ __global__ void DG_TILE_BOUNDS tile_kernel(const StageArgs<Pol> a) {
                                          cp_async_wait_all();
                                          __syncwarp();
                                        },
-                                       [&](int n) {
-                                         if (n >= 0) {
+                                       [&](bool mine, uint32_t at) {
+                                         if (mine) {
 #pragma unroll
                                            for (int v = 0; v < RV; ++v)
-                                             cp_async16(halo + v * HALO + lane, a.in + rec_at<RV>(n, v));
+                                             cp_async16(halo + v * HALO + lane, a.in + at + v * TILE);
                                          }
                                          cp_async_commit();
                                          cp_async_wait_all();

@@ -34,13 +34,14 @@ inline int tile_try_spec_occ<Mixed>(int p, int flux, int feat, int block) {
 
 #define DG_DEFINE_TILE_LAUNCHERS(POL)                                                                        \
   template <>                                                                                                \
-  cudaError_t launch_plan<POL>(const int4* nbr, const int4* meta, int ntiles, uint4* plan, int32_t* px, cudaStream_t s) { \
-    plan_kernel<POL::T><<<(ntiles + 7) / 8, 256, 0, s>>>(nbr, meta, ntiles, plan, px);                       \
+  cudaError_t launch_plan<POL>(const int4* nbr, const uint4* geo, const int4* nodes, const double* xy,       \
+                               const int4* meta, int ntiles, int rv, uint4* stat, int32_t* px, cudaStream_t s) { \
+    plan_kernel<POL><<<(ntiles + 7) / 8, 256, 0, s>>>(nbr, geo, nodes, xy, meta, ntiles, rv, stat, px);      \
     return cudaGetLastError();                                                                               \
   }                                                                                                          \
   template <>                                                                                                \
-  void plan_bytes<POL>(int ntiles, size_t& plan, size_t& px) {                                               \
-    plan = 16 * (size_t)plan_vec<POL::T>() * ntiles;                                                         \
+  void plan_bytes<POL>(int ntiles, size_t& stat, size_t& px) {                                               \
+    stat = 16 * (size_t)TileLayout<1, POL>::SVM * ntiles;                                                    \
     px = 4 * (size_t)PLAN_X * ntiles;                                                                        \
   }                                                                                                          \
   template <>                                                                                                \
