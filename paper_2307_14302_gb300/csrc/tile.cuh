@@ -81,6 +81,7 @@ struct TileLayout {
   static constexpr int NG = P + 1;
   static constexpr int RV = Pol::template RV<P>;
   static constexpr int GV = Pol::GV;
+  static constexpr int RVN = (sizeof(T) == 4 ? 6 + 3 * (np_of(P) - 1) + 3 : 2 * (3 * np_of(P)) + 3) / 4;  // vectors with modes
   // edge slot of one element side: Gz[NG], Gx[NG], Gy[NG] -- and the mass integral when NG is odd;
   // with an even NG the mass is the sum of the Gz, which is exactly antisymmetric across the edge
   // (the right side holds the negated values in reverse order) -- stored as pairs of T
@@ -1390,7 +1391,8 @@ __global__ void DG_TILE_BOUNDS tile_kernel(const StageArgs<Pol> a) {
     const ScenDev& S = *Sp;
     const int e0 = tile * TILE, e = e0 + lane;
     const bool valid = lane < present;
-    if (a.has_n && lane == 0) bulk_prefetch_l2(a.wn + (size_t)e0 * RV, 16u * TILE * RV);  // read in phase B
+    // step-initial modes, read in phase B (not the vectors that hold only depth, flag and bathymetry)
+    if (a.has_n && lane == 0) bulk_prefetch_l2(a.wn + (size_t)e0 * RV, 16u * TILE * L::RVN);
 
     // ---- the out-of-tile neighbours' records, one halo slot per lane, by the tile's plan
     if (lane < (meta.z >> 16)) {
