@@ -857,6 +857,8 @@ static cudaError_t enqueue_small(dgswe_h h, int n) {
     c.bw = h->stages[s].bw;
     split_ff(c.bw, c.bw_hi, c.bw_lo);
   }
+  st.same_bw = 1;
+  for (int s = 1; s < S; ++s) st.same_bw = st.same_bw && h->stages[s].bw == h->stages[0].bw;
   st.nstage = S;
   st.nsteps = n;
   st.nrec = S > 2 ? 3 : 2;

@@ -73,6 +73,7 @@ struct StepsArgs {
     double a_n, a_in, cst, bw;
   } st[MAXSTAGE];
   int nstage, nsteps, nrec;
+  int same_bw;  // every stage has the same ledger weight
 };
 
 }  // namespace dg

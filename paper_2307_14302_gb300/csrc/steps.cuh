@@ -141,7 +141,10 @@ __global__ void __maxnreg__(sizeof(typename Pol::T) == 4 ? (P == 1 ? 128 : 200) 
       }
       Storm<T> storm = {};
       if constexpr (storm_regs<P, FT>()) storm = storm_at<T>(S, t64);
-      Acc rain_acc = acc_make<Acc>(0.f, 0.f, 0.0), bdry_acc = acc_make<Acc>(0.f, 0.f, 0.0);
+      // equal stage weights (SSP(2,2), SSP(5,2)): the volumes accumulate over stages and steps as they
+      // are and take the weight at the end
+      const Acc zero = acc_make<Acc>(0.f, 0.f, 0.0);
+      Acc rain_acc = st.same_bw ? rain_tot : zero, bdry_acc = st.same_bw ? bdry_tot : zero;
       Elem<P, Pol> O;
       tile_body<P, FLUX, Pol, FT, true>(a, S, t64, rain_kind, press, rr, storm, tile, lane, valid, meta.z, meta.w,
                                         Wm + SL::REC + c.in * SL::RECS, halo, Wm + SL::GEO,
@@ -168,9 +171,14 @@ __global__ void __maxnreg__(sizeof(typename Pol::T) == 4 ? (P == 1 ? 128 : 200) 
         for (int v = 0; v < RV; ++v) to[v * TILE + lane] = ro.v[v];
       }
       // ledger: the stage's volume rates with its weight in the step
-      const Acc bw = acc_make<Acc>(c.bw_hi, c.bw_lo, c.bw);
-      rain_tot = acc_add(rain_tot, acc_mul(rain_acc, bw));
-      bdry_tot = acc_add(bdry_tot, acc_mul(bdry_acc, bw));
+      if (st.same_bw) {
+        rain_tot = acc_norm(rain_acc);
+        bdry_tot = bdry_acc;
+      } else {
+        const Acc bw = acc_make<Acc>(c.bw_hi, c.bw_lo, c.bw);
+        rain_tot = acc_add(rain_tot, acc_mul(rain_acc, bw));
+        bdry_tot = acc_add(bdry_tot, acc_mul(bdry_acc, bw));
+      }
       __syncwarp();
       cluster_arrive();
     }
@@ -184,8 +192,9 @@ __global__ void __maxnreg__(sizeof(typename Pol::T) == 4 ? (P == 1 ? 128 : 200) 
     warp_reduce2(rain_tot, bdry_tot);
     if (lane == 0) {
       double* Lg = a.ledger + 2 * ((long long)sc * a.wslots + tile);
-      Lg[0] += S.dt * acc_d(rain_tot);
-      Lg[1] += S.dt * acc_d(bdry_tot);
+      const double wdt = st.same_bw ? st.st[0].bw * S.dt : S.dt;
+      Lg[0] += wdt * acc_d(rain_tot);
+      Lg[1] += wdt * acc_d(bdry_tot);
     }
   }
   if (blockIdx.x == 0 && tid == 0) a.ctl->step = step0 + st.nsteps;  // every CTA has read it: the barriers passed
