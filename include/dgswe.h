@@ -319,7 +319,7 @@ int dgswe_get_tile_features(dgswe_h, int32_t* run, int32_t* kernel);
 
 /* No counterpart in the paper (device scheduling).  How dgswe_step enqueues its work: 1
  * (default) replays whole steps from CUDA graphs captured
- * once (1-step and 8-step graphs); 0 launches every kernel of every stage directly on the
+ * once (graphs of 1, 2, 4 ... 32 steps); 0 launches every kernel of every stage directly on the
  * stream.  Results are bit-identical; the direct form exists to measure what the graphs save
  * on small, launch-bound meshes.  Returns DGSWE_EINVAL for other values. */
 int dgswe_set_graphs(dgswe_h, int32_t on);

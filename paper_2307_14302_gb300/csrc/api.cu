@@ -5,7 +5,7 @@
 // one device layout: element records, static geometry, connectivity and per-scenario parameter
 // blocks, scenario element ranges aligned to 256 so tiles never straddle two scenarios.  A step
 // is one launch of the fused stage kernel per Runge-Kutta stage; steps are replayed from CUDA
-// graphs (1 step and 8 steps) captured on a private stream and launched on the caller's.
+// graphs (1, 2, 4 ... 32 steps) captured on a private stream and launched on the caller's.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -146,13 +146,19 @@ struct dgswe_ctx {
   int feat = FT_ALL;       // features of the run (Feature bits): selects the tile-kernel instantiation
   long long nn_total = 0;
   int grid = 0;
-  cudaGraphExec_t g1 = nullptr, gK = nullptr;
-  int K = 8;
+  static constexpr int NGRAPH = 6;
+  cudaGraphExec_t graph[NGRAPH] = {};  // graphs of 1, 2, 4, ... 32 steps, built when first needed
   long long launches = 0;
   Summary* sum = nullptr;          // page-locked: sums written by the device (summarise)
   char* bound = nullptr;           // caller memory holding the three record buffers (dgswe_bind_device)
   size_t bound_bytes = 0;
 
+  void drop_graphs() {
+    for (cudaGraphExec_t& g : graph) {
+      if (g) cudaGraphExecDestroy(g);
+      g = nullptr;
+    }
+  }
   ~dgswe_ctx() {
     DeviceGuard dg_(device);
     DevBuf* bufs[] = {&rec[0], &rec[1], &rec[2], &nbr, &geo, &nodes, &node_xy, &xy64, &hbn, &rain_e, &scen,
@@ -161,8 +167,7 @@ struct dgswe_ctx {
                       &rain_node, &node_scen, &lim, &rain_rec, &stat, &plan_x};
     for (DevBuf* b : bufs) b->alloc(0);
     if (sum) cudaFreeHost(sum);
-    if (g1) cudaGraphExecDestroy(g1);
-    if (gK) cudaGraphExecDestroy(gK);
+    drop_graphs();
     if (cap) cudaStreamDestroy(cap);
     if (own_stream && stream) cudaStreamDestroy(stream);
   }
@@ -682,8 +687,7 @@ static int fold_ledger(dgswe_h h) {
       }
     CU(cudaMemset(h->ledger.p, 0, 8 * part.size()));
   }
-  if (h->g1) { cudaGraphExecDestroy(h->g1); h->g1 = nullptr; }
-  if (h->gK) { cudaGraphExecDestroy(h->gK); h->gK = nullptr; }
+  h->drop_graphs();
   return 0;
 }
 
@@ -908,23 +912,23 @@ static int autotune(dgswe_h h) {
   return apply_launch(h, bb, bp, bs);
 }
 
-static int build_graphs(dgswe_h h) {
-  for (int which = 0; which < 2; ++which) {
-    const int nsteps = which == 0 ? 1 : h->K;
-    cudaGraph_t g;
-    CU(cudaStreamBeginCapture(h->cap, cudaStreamCaptureModeThreadLocal));
-    int rc = 0;
-    for (int k = 0; k < nsteps && !rc; ++k)
-      for (size_t s = 0; s < h->stages.size() && !rc; ++s) rc = launch_stage_once(h, (int)s, 0, h->cap);
-    cudaError_t ce = cudaStreamEndCapture(h->cap, &g);
-    if (rc) return rc;
-    if (ce != cudaSuccess) return fail(DGSWE_ECUDA, "graph capture: %s", cudaGetErrorString(ce));
-    h->launches -= nsteps * (long long)h->stages.size() * launches_per_stage(h);  // counted when the graph runs
-    cudaGraphExec_t ex;
-    ce = cudaGraphInstantiate(&ex, g, 0);
-    cudaGraphDestroy(g);
-    if (ce != cudaSuccess) return fail(DGSWE_ECUDA, "graph instantiate: %s", cudaGetErrorString(ce));
-    (which == 0 ? h->g1 : h->gK) = ex;
+// the graph of 2^k steps
+static int build_graph(dgswe_h h, int k) {
+  const int nsteps = 1 << k;
+  cudaGraph_t g;
+  CU(cudaStreamBeginCapture(h->cap, cudaStreamCaptureModeThreadLocal));
+  int rc = 0;
+  for (int i = 0; i < nsteps && !rc; ++i)
+    for (size_t s = 0; s < h->stages.size() && !rc; ++s) rc = launch_stage_once(h, (int)s, 0, h->cap);
+  cudaError_t ce = cudaStreamEndCapture(h->cap, &g);
+  if (rc) return rc;
+  if (ce != cudaSuccess) return fail(DGSWE_ECUDA, "graph capture: %s", cudaGetErrorString(ce));
+  h->launches -= nsteps * (long long)h->stages.size() * launches_per_stage(h);  // counted when the graph runs
+  ce = cudaGraphInstantiate(&h->graph[k], g, 0);
+  cudaGraphDestroy(g);
+  if (ce != cudaSuccess) {
+    h->graph[k] = nullptr;
+    return fail(DGSWE_ECUDA, "graph instantiate: %s", cudaGetErrorString(ce));
   }
   return 0;
 }
@@ -1260,11 +1264,16 @@ int dgswe_step(dgswe_h h, int64_t n) {
     }
     return 0;
   }
-  if (!h->g1)
-    if (int rc = build_graphs(h)) return rc;
+  // whole steps from graphs of 32, 16, ... 1 steps: a graph launch costs about 3 us of idle GPU, so few and
+  // large ones (20 steps as 16 + 4; with graphs of 8 and 1 they were six launches)
   const long long per = (long long)h->stages.size() * launches_per_stage(h);
-  for (int64_t i = 0; i < n / h->K; ++i) CU(cudaGraphLaunch(h->gK, h->stream));
-  for (int64_t i = 0; i < n % h->K; ++i) CU(cudaGraphLaunch(h->g1, h->stream));
+  int64_t left = n;
+  for (int k = dgswe_ctx::NGRAPH - 1; k >= 0; --k)
+    for (; left >= (1 << k); left -= 1 << k) {
+      if (!h->graph[k])
+        if (int rc = build_graph(h, k)) return rc;
+      CU(cudaGraphLaunch(h->graph[k], h->stream));
+    }
   h->launches += n * per;
   return 0;
 }
