@@ -102,11 +102,13 @@ struct DevBuf {
 
 struct DeviceGuard {
   int prev = -1;
+  bool changed = false;
   explicit DeviceGuard(int dev) {
     if (cudaGetDevice(&prev) != cudaSuccess) prev = -1;
-    if (prev != dev) cudaSetDevice(dev);
+    changed = prev != dev;
+    if (changed) cudaSetDevice(dev);
   }
-  ~DeviceGuard() { if (prev >= 0) cudaSetDevice(prev); }
+  ~DeviceGuard() { if (changed && prev >= 0) cudaSetDevice(prev); }
 };
 
 }  // namespace
@@ -743,6 +745,14 @@ static StageArgs<Pol> make_args(dgswe_h h, int stage, int tune) {
   return a;
 }
 
+// arguments of the kernels that write a state into the records w^n
+template <class Pol>
+static StageArgs<Pol> load_args(dgswe_h h) {
+  StageArgs<Pol> a = make_args<Pol>(h, 0, 1);
+  a.in = a.out = h->rec[0].as<uint4>();
+  return a;
+}
+
 static int edge_grid(dgswe_h h) {
   int sms = 0;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
@@ -1343,21 +1353,6 @@ static int gather_state(dgswe_h h, size_t s, double* z, double* x, double* y, bo
   return 0;
 }
 
-// after records [b, b + n) received a state: their mean depths and wet/dry flags from it, the
-// state kept as given (positive-depth pass in classify mode)
-static cudaError_t classify_loaded(dgswe_h h, long long b, long long n) {
-  if (mixed(h)) {
-    StageArgs<Mixed> a = make_args<Mixed>(h, 0, 1);
-    a.in = a.out = h->rec[0].as<uint4>();
-    a.classify_only = 1;
-    return launch_prepare<Mixed>(h->prm.p, a, b, b + n, h->stream);
-  }
-  StageArgs<Fp64> a = make_args<Fp64>(h, 0, 1);
-  a.in = a.out = h->rec[0].as<uint4>();
-  a.classify_only = 1;
-  return launch_prepare<Fp64>(h->prm.p, a, b, b + n, h->stream);
-}
-
 int dgswe_get_state(dgswe_h h, double* z, double* x, double* y) {
   if (int rc = check_handle(h)) return rc;
   if (!h->ready) return fail(DGSWE_ESTATE, "no state");
@@ -1394,11 +1389,10 @@ int dgswe_exchange_state(dgswe_h h, const double* zi, const double* xi, const do
   const double *dzi = (const double*)m[0], *dxi = (const double*)m[1], *dyi = (const double*)m[2];
   double *dzo = (double*)m[3], *dxo = (double*)m[4], *dyo = (double*)m[5];
   const int32_t* inv = h->einv.as<int32_t>() + b;
-  cudaError_t ce = mixed(h) ? launch_exchange<Mixed>(h->prm.p, h->rec[0].as<uint4>(), b, n, inv, dzi, dxi, dyi, dzo, dxo, dyo, h->stream)
-                            : launch_exchange<Fp64>(h->prm.p, h->rec[0].as<uint4>(), b, n, inv, dzi, dxi, dyi, dzo, dxo, dyo, h->stream);
-  if (ce == cudaSuccess) ce = classify_loaded(h, b, n);
+  cudaError_t ce = mixed(h) ? launch_exchange<Mixed>(h->prm.p, load_args<Mixed>(h), b, n, inv, dzi, dxi, dyi, dzo, dxo, dyo, h->stream)
+                            : launch_exchange<Fp64>(h->prm.p, load_args<Fp64>(h), b, n, inv, dzi, dxi, dyi, dzo, dxo, dyo, h->stream);
   if (ce != cudaSuccess) return fail(DGSWE_ECUDA, "exchange_state launch: %s", cudaGetErrorString(ce));
-  h->launches += 2;
+  h->launches++;
   CU(cudaStreamSynchronize(h->stream));
   return 0;
 }
@@ -1431,11 +1425,10 @@ int dgswe_load_state(dgswe_h h, const double* z, const double* x, const double* 
     sx = dz + cnt;
     sy = dz + 2 * cnt;
   }
-  cudaError_t ce = mixed(h) ? launch_scatter<Mixed>(h->prm.p, h->rec[0].as<uint4>(), b, n, h->einv.as<int32_t>() + b, sz, sx, sy, h->stream)
-                            : launch_scatter<Fp64>(h->prm.p, h->rec[0].as<uint4>(), b, n, h->einv.as<int32_t>() + b, sz, sx, sy, h->stream);
-  if (ce == cudaSuccess) ce = classify_loaded(h, b, n);
+  cudaError_t ce = mixed(h) ? launch_scatter<Mixed>(h->prm.p, load_args<Mixed>(h), b, n, h->einv.as<int32_t>() + b, sz, sx, sy, h->stream)
+                            : launch_scatter<Fp64>(h->prm.p, load_args<Fp64>(h), b, n, h->einv.as<int32_t>() + b, sz, sx, sy, h->stream);
   if (ce != cudaSuccess) return fail(DGSWE_ECUDA, "load_state launch: %s", cudaGetErrorString(ce));
-  h->launches += 2;
+  h->launches++;
   if (!direct) CU(cudaStreamSynchronize(h->stream));
   return 0;
 }

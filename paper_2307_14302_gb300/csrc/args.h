@@ -54,7 +54,6 @@ struct StageArgs {
   int stage;               // Shu-Osher stage index
   int last;                // 1 on the final stage of a step
   int tune;                // 1: timing run, no ledger or step bookkeeping
-  int classify_only;       // prepare pass: derive depth and dry flag, keep the state as given
   int friction;            // 0 Manning, 1 quadratic, 2 none
   int has_n;               // the stage combines with the step-initial state
   int pow2;                // a_n and a_in are 0 or powers of two (exact float-float scaling)
@@ -211,9 +210,10 @@ template <class Pol>
 cudaError_t launch_gather(int p, const uint4* rec, long long begin, long long n, const int32_t* inv, double* z,
                           double* x, double* y, cudaStream_t s);
 
-// modal state [Np][n] (caller order) into the records of [begin, begin + n), same conventions
+// modal state [Np][n] (caller order) into the records a.out of [begin, begin + n), same conventions;
+// their depths and wet/dry flags are derived from it
 template <class Pol>
-cudaError_t launch_scatter(int p, uint4* rec, long long begin, long long n, const int32_t* inv, const double* z,
-                           const double* x, const double* y, cudaStream_t s);
+cudaError_t launch_scatter(int p, const StageArgs<Pol>& a, long long begin, long long n, const int32_t* inv,
+                           const double* z, const double* x, const double* y, cudaStream_t s);
 
 }  // namespace dg

@@ -9,15 +9,15 @@ namespace dg {
 // Thread c takes caller element c (coalesced in the caller's arrays): it reads the element's
 // record, writes its modal coefficients out exactly as the unpacking kernel of dgswe_get_state
 // does (mode 0 of each variable is sqrt(2) times the element mean), then sets the coefficients
-// from the in arrays exactly as the packing kernel of dgswe_load_state does (bathymetry modes kept;
-// depth and wet/dry flag are derived by the positive-depth pass that follows) and stores the
-// record.  Each record is read and written by one thread only (inv is a permutation).
+// from the in arrays exactly as the packing kernel of dgswe_load_state does (bathymetry modes kept,
+// depth and wet/dry flag derived) and stores the record.  Each record is read and written by one thread only (inv is a permutation).
 template <int P, class Pol>
-__global__ void __launch_bounds__(256) exchange_kernel(uint4* rec, long long begin, long long n, const int32_t* inv,
+__global__ void __launch_bounds__(256) exchange_kernel(const StageArgs<Pol> a, long long begin, long long n, const int32_t* inv,
                                                        const double* zi, const double* xi, const double* yi,
                                                        double* zo, double* xo, double* yo) {
   constexpr int RV = Pol::template RV<P>, NS = np_of(P) - 1;
   using T = typename Pol::T;
+  uint4* rec = a.out;
   const double s2 = 1.4142135623730951, is2 = 0.7071067811865476;
   for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n; c += (long long)gridDim.x * blockDim.x) {
     const long long e = begin + inv[c];
@@ -52,24 +52,25 @@ __global__ void __launch_bounds__(256) exchange_kernel(uint4* rec, long long beg
       E.xs[m] = (T)xn[m];
       E.ys[m] = (T)yn[m];
     }
+    classify<P, Pol>(E, e, a);
     pack<P>(E, r);
     store_raw<RV>(rec, e, r);
   }
 }
 
 template <class Pol>
-cudaError_t launch_exchange(int p, uint4* rec, long long begin, long long n, const int32_t* inv, const double* zi,
+cudaError_t launch_exchange(int p, const StageArgs<Pol>& a, long long begin, long long n, const int32_t* inv, const double* zi,
                             const double* xi, const double* yi, double* zo, double* xo, double* yo, cudaStream_t s) {
   const long long g0 = (n + 255) / 256;
   const int g = (int)(g0 < 1 ? 1 : (g0 > 65535 * 8 ? 65535 * 8 : g0));
-  if (p == 1) exchange_kernel<1, Pol><<<g, 256, 0, s>>>(rec, begin, n, inv, zi, xi, yi, zo, xo, yo);
-  else exchange_kernel<2, Pol><<<g, 256, 0, s>>>(rec, begin, n, inv, zi, xi, yi, zo, xo, yo);
+  if (p == 1) exchange_kernel<1, Pol><<<g, 256, 0, s>>>(a, begin, n, inv, zi, xi, yi, zo, xo, yo);
+  else exchange_kernel<2, Pol><<<g, 256, 0, s>>>(a, begin, n, inv, zi, xi, yi, zo, xo, yo);
   return cudaGetLastError();
 }
 
-template cudaError_t launch_exchange<Mixed>(int, uint4*, long long, long long, const int32_t*, const double*,
+template cudaError_t launch_exchange<Mixed>(int, const StageArgs<Mixed>&, long long, long long, const int32_t*, const double*,
                                             const double*, const double*, double*, double*, double*, cudaStream_t);
-template cudaError_t launch_exchange<Fp64>(int, uint4*, long long, long long, const int32_t*, const double*,
+template cudaError_t launch_exchange<Fp64>(int, const StageArgs<Fp64>&, long long, long long, const int32_t*, const double*,
                                            const double*, const double*, double*, double*, double*, cudaStream_t);
 
 }  // namespace dg

@@ -1898,16 +1898,21 @@ __global__ void __launch_bounds__(256) prepare_kernel(const StageArgs<Pol> a, lo
     load_raw<RV>(a.in, e, r);
     Elem<P, Pol> E;
     unpack<P>(r, E);
-    Elem<P, Pol> O = E;
-    apply_positivity<P, Pol>(O, G, e, a, &a.ctl->err);
-    if (a.classify_only) {
-      E.Hb = O.Hb;
-      E.flags = O.flags;
-      O = E;
-    }
-    pack<P>(O, r);
+    apply_positivity<P, Pol>(E, G, e, a, &a.ctl->err);
+    pack<P>(E, r);
     store_raw<RV>(a.out, e, r);
   }
+}
+
+// mean depth and wet/dry flag of an element that has just received a state, which stays as given
+template <int P, class Pol>
+__device__ __forceinline__ void classify(Elem<P, Pol>& E, long long e, const StageArgs<Pol>& a) {
+  Geo<Pol> G;
+  load_geo(a.geo, e, make_int4(0, 0, 0, 0), G);
+  Elem<P, Pol> O = E;
+  apply_positivity<P, Pol>(O, G, e, a, &a.ctl->err);
+  E.Hb = O.Hb;
+  E.flags = O.flags;
 }
 
 __device__ __forceinline__ void neu_add(double& s, double& c, double v) {
@@ -2102,11 +2107,13 @@ __global__ void __launch_bounds__(256) gather_kernel(const uint4* rec, long long
 }
 
 // modal state [Np][n] in caller order -> records of elements [begin, begin + n) (thread c reads
-// caller element c, coalesced); bathymetry modes are kept, depth and flags are recomputed by the
-// positive-depth pass that follows
+// caller element c, coalesced); bathymetry modes are kept, depth and flags derived (a pass of its own
+// before: 9 us of a 50 us exchange on 30k triangles)
 template <int P, class Pol>
-__global__ void __launch_bounds__(256) scatter_kernel(uint4* rec, long long begin, long long n, const int32_t* inv,
-                                                      const double* z, const double* x, const double* y) {
+__global__ void __launch_bounds__(256) scatter_kernel(const StageArgs<Pol> a, long long begin, long long n,
+                                                      const int32_t* inv, const double* z, const double* x,
+                                                      const double* y) {
+  uint4* rec = a.out;
   constexpr int RV = Pol::template RV<P>, NS = np_of(P) - 1;
   const double is2 = 0.7071067811865476;  // mean = mode-0 coefficient / sqrt(2)
   for (long long c = blockIdx.x * (long long)blockDim.x + threadIdx.x; c < n; c += (long long)gridDim.x * blockDim.x) {
@@ -2124,6 +2131,7 @@ __global__ void __launch_bounds__(256) scatter_kernel(uint4* rec, long long begi
       E.xs[m] = (typename Pol::T)x[(m + 1) * n + c];
       E.ys[m] = (typename Pol::T)y[(m + 1) * n + c];
     }
+    classify<P, Pol>(E, e, a);
     pack<P>(E, r);
     store_raw<RV>(rec, e, r);
   }
@@ -2247,11 +2255,11 @@ static inline int grid_for(long long n, int block) {
     return cudaGetLastError();                                                                               \
   }                                                                                                          \
   template <>                                                                                                \
-  cudaError_t launch_scatter<POL>(int p, uint4* rec, long long b, long long n, const int32_t* inv,           \
+  cudaError_t launch_scatter<POL>(int p, const StageArgs<POL>& a, long long b, long long n, const int32_t* inv, \
                                   const double* z, const double* x, const double* y, cudaStream_t s) {       \
     int g = grid_for(n, 256);                                                                                \
-    if (p == 1) scatter_kernel<1, POL><<<g, 256, 0, s>>>(rec, b, n, inv, z, x, y);                           \
-    else scatter_kernel<2, POL><<<g, 256, 0, s>>>(rec, b, n, inv, z, x, y);                                  \
+    if (p == 1) scatter_kernel<1, POL><<<g, 256, 0, s>>>(a, b, n, inv, z, x, y);                             \
+    else scatter_kernel<2, POL><<<g, 256, 0, s>>>(a, b, n, inv, z, x, y);                                    \
     return cudaGetLastError();                                                                               \
   }
 
