@@ -528,28 +528,27 @@ __device__ __forceinline__ Trace<typename Pol::T> trace_p1(const Elem<1, Pol>& E
   return t;
 }
 
-// canonical flux across an edge with unit normal n from L to R; returns the mass flux and the
-// advective + dissipative momentum flux (the pressure part is added per side)
+// twice the canonical flux across an edge with unit normal n from L to R: the mass flux and the
+// advective + dissipative momentum flux (the pressure part is added per side).  Doubled, the averages
+// and the dissipation need no halves; the caller's edge weight takes them.
 template <int FLUX, class T>
-__device__ __forceinline__ void edge_flux(const Trace<T>& L, const Trace<T>& R, T dcRL, T nx, T ny, T g, T H0, T& fz,
-                                          T& fx, T& fy) {
-  // one inverse square root per side (as edge_flux_pair)
+__device__ __forceinline__ void edge_flux2(const Trace<T>& L, const Trace<T>& R, T dcRL, T nx, T ny, T g, T H0, T& fz,
+                                           T& fx, T& fy) {
+  // one inverse square root per side (as edge_flux_pair2)
   const T HsL = max_r(L.H, H0), HsR = max_r(R.H, H0);
   const T rL = frsqrt(HsL), rR = frsqrt(HsR);
   const T mL = L.qx * nx + L.qy * ny, mR = R.qx * nx + R.qy * ny;
   const T unL = mL * (rL * rL), unR = mR * (rR * rR);
   const T dz = (R.d - L.d) + dcRL;
   const T dqx = R.qx - L.qx, dqy = R.qy - L.qy;
-  const T cx = T(0.5) * (L.qx * unL + R.qx * unR);
-  const T cy = T(0.5) * (L.qy * unL + R.qy * unR);
-  const T cz = T(0.5) * (mL + mR);
+  const T sx = fma(L.qx, unL, R.qx * unR), sy = fma(L.qy, unL, R.qy * unR), sz = mL + mR;
   const T sL = HsL * rL, sR = HsR * rR;
   if (FLUX == 1) {  // local Lax-Friedrichs
     const T sg = fsqrt_pos(g);
-    const T lam = max_r(abs_r(unL) + sg * sL, abs_r(unR) + sg * sR);
-    fz = cz - T(0.5) * lam * dz;
-    fx = cx - T(0.5) * lam * dqx;
-    fy = cy - T(0.5) * lam * dqy;
+    const T lam = max_r(fma(sg, sL, abs_r(unL)), fma(sg, sR, abs_r(unR)));
+    fz = fma(-lam, dz, sz);
+    fx = fma(-lam, dqx, sx);
+    fy = fma(-lam, dqy, sy);
     return;
   }
   // Roe: averages (arithmetic depth, sqrt-depth-weighted velocity), eigen-decomposition
@@ -562,9 +561,18 @@ __device__ __forceinline__ void edge_flux(const Trace<T>& L, const Trace<T>& R, 
   const T w = (dqn - utn * dz) * ic;
   const T a1 = T(0.5) * (dz - w), a3 = T(0.5) * (dz + w), a2 = dqt - utt * dz;
   const T l1 = abs_r(utn - c) * a1, l2 = abs_r(utn) * a2, l3 = abs_r(utn + c) * a3;
-  fz = cz - T(0.5) * (l1 + l3);
-  fx = cx - T(0.5) * (l1 * (ut - c * nx) - l2 * ny + l3 * (ut + c * nx));
-  fy = cy - T(0.5) * (l1 * (vt - c * ny) + l2 * nx + l3 * (vt + c * ny));
+  fz = sz - (l1 + l3);
+  fx = fma(-l1, fma(-c, nx, ut), fma(l2, ny, fma(-l3, fma(c, nx, ut), sx)));
+  fy = fma(-l1, fma(-c, ny, vt), fma(-l2, nx, fma(-l3, fma(c, ny, vt), sy)));
+}
+// the flux itself
+template <int FLUX, class T>
+__device__ __forceinline__ void edge_flux(const Trace<T>& L, const Trace<T>& R, T dcRL, T nx, T ny, T g, T H0, T& fz,
+                                          T& fx, T& fy) {
+  edge_flux2<FLUX, T>(L, R, dcRL, nx, ny, g, H0, fz, fx, fy);
+  fz *= T(0.5);
+  fx *= T(0.5);
+  fy *= T(0.5);
 }
 
 #ifndef DG_PACKED_FLUX
@@ -588,19 +596,19 @@ struct Trace2 {
   f2 d, H, qx, qy;  // two edge points
 };
 
-// edge_flux for two points at once (FP32), written with packed operations and one reciprocal
+// edge_flux2 for two points at once (FP32), written with packed operations and one reciprocal
 // square root per side: with r = 1/sqrt(Hs), 1/Hs = r^2, sqrt(Hs) = Hs r, the Roe velocity is
 // (q_L r_L + q_R r_R) / (sqrt(Hs_L) + sqrt(Hs_R)), u.n = (q.n)/Hs, and the jump of q.n is the
-// difference of the sides' q.n (the same quantities as edge_flux, fewer operations)
-// per-side quantities of edge_flux_pair that the wall flux of a closed edge reuses: q.n, 1/Hs and
+// difference of the sides' q.n (the same quantities as edge_flux2)
+// per-side quantities of edge_flux_pair2 that the wall flux of a closed edge reuses: q.n, 1/Hs and
 // sqrt(Hs) of both sides
 struct FluxAux2 {
   f2 mL, mR, iL, iR, sL, sR;
 };
 template <int FLUX>
-__device__ __forceinline__ void edge_flux_pair(const Trace2& L, const Trace2& R, f2 dcRL, f2 nx, f2 ny, float g,
-                                               float H0, f2& fz, f2& fx, f2& fy, FluxAux2& ax) {
-  const f2 half = p2(0.5f), mhalf = p2(-0.5f);
+__device__ __forceinline__ void edge_flux_pair2(const Trace2& L, const Trace2& R, f2 dcRL, f2 nx, f2 ny, float g,
+                                                float H0, f2& fz, f2& fx, f2& fy, FluxAux2& ax) {
+  const f2 half = p2(0.5f);
   const f2 HsL = max2(L.H, p2(H0)), HsR = max2(R.H, p2(H0));
   const f2 rL = rsqrt2(HsL), rR = rsqrt2(HsR);
   const f2 iL = mul2(rL, rL), iR = mul2(rR, rR);
@@ -608,18 +616,17 @@ __device__ __forceinline__ void edge_flux_pair(const Trace2& L, const Trace2& R,
   const f2 unL = mul2(mL, iL), unR = mul2(mR, iR);
   const f2 dz = add2(sub2(R.d, L.d), dcRL);
   const f2 dqx = sub2(R.qx, L.qx), dqy = sub2(R.qy, L.qy);
-  const f2 cx = mul2(half, fma2(L.qx, unL, mul2(R.qx, unR)));
-  const f2 cy = mul2(half, fma2(L.qy, unL, mul2(R.qy, unR)));
-  const f2 cz = mul2(half, add2(mL, mR));
+  const f2 sx = fma2(L.qx, unL, mul2(R.qx, unR));
+  const f2 sy = fma2(L.qy, unL, mul2(R.qy, unR));
+  const f2 sz = add2(mL, mR);
   const f2 sL = mul2(HsL, rL), sR = mul2(HsR, rR);
   ax = {mL, mR, iL, iR, sL, sR};
   if (FLUX == 1) {  // local Lax-Friedrichs: sqrt(g Hs) = sqrt(g) sqrt(Hs)
     const f2 sg = p2(fsqrt_pos(g));
-    const f2 lam = max2(fma2(sg, sL, abs2(unL)), fma2(sg, sR, abs2(unR)));
-    const f2 hl = mul2(mhalf, lam);
-    fz = fma2(hl, dz, cz);
-    fx = fma2(hl, dqx, cx);
-    fy = fma2(hl, dqy, cy);
+    const f2 ml = neg2(max2(fma2(sg, sL, abs2(unL)), fma2(sg, sR, abs2(unR))));
+    fz = fma2(ml, dz, sz);
+    fx = fma2(ml, dqx, sx);
+    fy = fma2(ml, dqy, sy);
     return;
   }
   // Roe: averages (arithmetic depth, sqrt-depth-weighted velocity), eigen-decomposition
@@ -630,14 +637,12 @@ __device__ __forceinline__ void edge_flux_pair(const Trace2& L, const Trace2& R,
   const f2 utn = fma2(ut, nx, mul2(vt, ny)), utt = fma2(vt, nx, mul2(neg2(ut), ny));
   const f2 dqn = sub2(mR, mL), dqt = fma2(dqy, nx, mul2(neg2(dqx), ny));
   const f2 w = mul2(fma2(neg2(utn), dz, dqn), ic);
-  const f2 a1 = mul2(half, sub2(dz, w)), a3 = mul2(half, add2(dz, w)), a2 = fma2(neg2(utt), dz, dqt);
+  const f2 a1 = mul2(half, sub2(w, dz)), a3 = mul2(p2(-0.5f), add2(dz, w)), a2 = fma2(neg2(utt), dz, dqt);
+  // l1 and l3 negated
   const f2 l1 = mul2(abs2(sub2(utn, c)), a1), l2 = mul2(abs2(utn), a2), l3 = mul2(abs2(add2(utn, c)), a3);
-  const f2 D0 = add2(l1, l3);
-  const f2 D1 = fma2(l1, fma2(neg2(c), nx, ut), fma2(neg2(l2), ny, mul2(l3, fma2(c, nx, ut))));
-  const f2 D2 = fma2(l1, fma2(neg2(c), ny, vt), fma2(l2, nx, mul2(l3, fma2(c, ny, vt))));
-  fz = fma2(mhalf, D0, cz);
-  fx = fma2(mhalf, D1, cx);
-  fy = fma2(mhalf, D2, cy);
+  fz = add2(sz, add2(l1, l3));
+  fx = fma2(l1, fma2(neg2(c), nx, ut), fma2(l2, ny, fma2(l3, fma2(c, nx, ut), sx)));
+  fy = fma2(l1, fma2(neg2(c), ny, vt), fma2(neg2(l2), nx, fma2(l3, fma2(c, ny, vt), sy)));
 }
 
 // pressure difference P - P_c with P_c the pressure at the reference elevation c:
@@ -1731,10 +1736,10 @@ __global__ void DG_STAGE_BOUNDS stage_kernel(const StageArgs<Pol> a) {
                           make_float2(b0.qy, b1.qy)};
           f2 fz2, fx2, fy2;
           FluxAux2 ax;
-          edge_flux_pair<FLUX>(L2, R2, p2(dcRL), p2(sgn * nx), p2(sgn * ny), g, H0, fz2, fx2, fy2, ax);
-          fzc[0] = fz2.x; fzc[1] = fz2.y;
-          fxc[0] = fx2.x; fxc[1] = fx2.y;
-          fyc[0] = fy2.x; fyc[1] = fy2.y;
+          edge_flux_pair2<FLUX>(L2, R2, p2(dcRL), p2(sgn * nx), p2(sgn * ny), g, H0, fz2, fx2, fy2, ax);
+          fzc[0] = 0.5f * fz2.x; fzc[1] = 0.5f * fz2.y;
+          fxc[0] = 0.5f * fx2.x; fxc[1] = 0.5f * fx2.y;
+          fyc[0] = 0.5f * fy2.x; fyc[1] = 0.5f * fy2.y;
           if (river) fzc[0] = fzc[1] = -qr;
         } else {
 #pragma unroll

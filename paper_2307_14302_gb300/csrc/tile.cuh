@@ -611,6 +611,12 @@ __device__ __forceinline__ void side_traces(const Elem<P, Pol>& E, int j, const 
     }
 #pragma unroll
     for (int k = 0; k < NG; ++k) t[k].H = E.Hb + (t[k].d + h[k]);
+  } else if constexpr (P == 1) {
+#pragma unroll
+    for (int k = 0; k < NG; ++k) {
+      const T* ph = ephi[j][REV ? NG - 1 - k : k];
+      t[k] = trace_p1(E, ph[1], ph[2]);
+    }
   } else {
 #pragma unroll
     for (int k = 0; k < NG; ++k) t[k] = trace_at<P, Pol>(E, ephi[j][REV ? NG - 1 - k : k]);
@@ -695,6 +701,24 @@ __device__ __forceinline__ void store_sd(void* flx, int e, int j, f2 z, f2 x, f2
   reinterpret_cast<float2*>(reinterpret_cast<float4*>(flx) + 96)[j * 32 + e] = y;
 }
 
+// a point's (or a packed pair's) values for both sides from the doubled flux: w half the point's edge
+// weight, pq = w g / 2 for the pressure, the mean of the sides' g/2 d (2H - d) relative to each side's mean
+template <class V>
+__device__ __forceinline__ void side_points(V Ld, V LH, V Rd, V RH, V dc, V nx, V ny, V w, V pq, V fz, V fx, V fy,
+                                            V (&l)[3], V (&r)[3]) {
+  const V two = vbc<V>(2.f);
+  const V Fz = vmul(w, fz), Fx = vmul(w, fx), Fy = vmul(w, fy);
+  const V A = vmul(Ld, vfma(two, LH, vneg(Ld))), B = vmul(Rd, vfma(two, RH, vneg(Rd)));
+  const V R1 = vadd(Rd, dc), L1 = vadd(Ld, vneg(dc));
+  const V pL = vmul(pq, vfma(R1, vfma(two, RH, vneg(R1)), A)), pR = vmul(pq, vfma(L1, vfma(two, LH, vneg(L1)), B));
+  l[0] = Fz;
+  l[1] = vfma(pL, nx, Fx);
+  l[2] = vfma(pL, ny, Fy);
+  r[0] = vneg(Fz);
+  r[1] = vneg(vfma(pR, nx, Fx));
+  r[2] = vneg(vfma(pR, ny, Fy));
+}
+
 template <int P, int FLUX, class Pol, int FT>
 __device__ __forceinline__ void tile_edge(const StageArgs<Pol>& a, const ScenDev& S, uint32_t ownB, uint32_t halB,
                                           const uint4* geo, void* flx, unsigned ed,
@@ -766,31 +790,31 @@ __device__ __forceinline__ void tile_edge(const StageArgs<Pol>& a, const ScenDev
                     make_float2(tr[0].qy, tr[1].qy)};
     f2 fz2, fx2, fy2;
     FluxAux2 ax;  // per-side quantities for the wall flux
-    edge_flux_pair<FLUX>(L2, R2, p2(dcRL), p2(nx), p2(ny), g, H0, fz2, fx2, fy2, ax);
-    if (river) fz2 = p2(-qr);  // the specified normal flow is the mass flux
-    const f2 hl2 = p2(hl);
-    const f2 Fz = mul2(sum_diff(fz2), hl2);  // Fz.x: the mass integral along n
+    edge_flux_pair2<FLUX>(L2, R2, p2(dcRL), p2(nx), p2(ny), g, H0, fz2, fx2, fy2, ax);
+    if (river) fz2 = p2(-2.f * qr);  // the specified normal flow is the mass flux
+    const f2 hh2 = p2(0.5f * hl);    // half the edge weight: the fluxes are doubled
+    const f2 Fz = mul2(sum_diff(fz2), hh2);  // Fz.x: the mass integral along n
     // wet/dry closure: no water leaves a dry element (interior: either side; ocean/river: L)
     const bool closed = land || (dryL && Fz.x > 0.f) || (dryR && Fz.x < 0.f);
     if (!closed) {
-      const f2 Fx = mul2(sum_diff(fx2), hl2), Fy = mul2(sum_diff(fy2), hl2), dc = p2(dcRL), hq = p2(0.25f * g);
+      const f2 Fx = mul2(sum_diff(fx2), hh2), Fy = mul2(sum_diff(fy2), hh2), dc = p2(dcRL), pq = p2(0.25f * g * hl);
       if (srcL < TILE) {  // pressure: the mean of the sides' g/2 d (2H - d) relative to L's mean
         const f2 Rd = add2(R2.d, dc);
         const f2 pp = fma2(L2.d, fma2(p2(2.f), L2.H, neg2(L2.d)), mul2(Rd, fma2(p2(2.f), R2.H, neg2(Rd))));
-        const f2 Pd = mul2(sum_diff(mul2(hq, pp)), hl2);
+        const f2 Pd = mul2(sum_diff(pp), pq);
         store_sd(flx, srcL, jL, Fz, fma2(Pd, p2(nx), Fx), fma2(Pd, p2(ny), Fy));
         if (!interior) bdry_acc = acc_addr(bdry_acc, -Fz.x);  // inflow
       }
       if (interior && srcR < TILE) {  // relative to R's mean, along -n
         const f2 Ld = sub2(L2.d, dc);
         const f2 pp = fma2(R2.d, fma2(p2(2.f), R2.H, neg2(R2.d)), mul2(Ld, fma2(p2(2.f), L2.H, neg2(Ld))));
-        const f2 Pd = mul2(sum_diff(mul2(hq, pp)), hl2);
+        const f2 Pd = mul2(sum_diff(pp), pq);
         store_sd(flx, srcR, jR, make_float2(-Fz.x, Fz.y), fma2(Pd, make_float2(-nx, nx), make_float2(-Fx.x, Fx.y)),
                  fma2(Pd, make_float2(-ny, ny), make_float2(-Fy.x, Fy.y)));
       }
     } else {
       // wall: q.n (q.n / Hs + c) + pressure relative to the side's mean (LLF: (q.n + |q.n|) / Hs)
-      const f2 z = p2(0.f), sg = p2(fsqrt_pos(g)), hg = p2(0.5f * g);
+      const f2 z = p2(0.f), sg = p2(fsqrt_pos(g)), hg = p2(0.5f * g), hl2 = p2(hl);
       if (srcL < TILE) {
         const f2 un = (FLUX == 1) ? mul2(add2(ax.mL, abs2(ax.mL)), ax.iL) : mul2(ax.mL, ax.iL);
         const f2 w = fma2(ax.mL, fma2(sg, ax.sL, un), mul2(hg, mul2(L2.d, fma2(p2(2.f), L2.H, neg2(L2.d)))));
@@ -806,84 +830,80 @@ __device__ __forceinline__ void tile_edge(const StageArgs<Pol>& a, const ScenDev
       }
     }
   } else {
-    T fz[NG], fx[NG], fy[NG];
-    T ec = T(0);  // mass flux integral along n (L's outward normal)
-    bool closed = land;
-    if (!land) {
-      if constexpr (P == 2 && sizeof(T) == 4 && DG_PACKED_FLUX) {  // points 0 and 1 packed, point 2 alone
-        const Trace2 L2{make_float2(tl[0].d, tl[1].d), make_float2(tl[0].H, tl[1].H), make_float2(tl[0].qx, tl[1].qx),
-                        make_float2(tl[0].qy, tl[1].qy)};
-        const Trace2 R2{make_float2(tr[0].d, tr[1].d), make_float2(tr[0].H, tr[1].H), make_float2(tr[0].qx, tr[1].qx),
-                        make_float2(tr[0].qy, tr[1].qy)};
-        f2 fz2, fx2, fy2;
-        FluxAux2 ax2;
-        edge_flux_pair<FLUX>(L2, R2, p2(dcRL), p2(nx), p2(ny), g, H0, fz2, fx2, fy2, ax2);
-        fz[0] = fz2.x; fz[1] = fz2.y;
-        fx[0] = fx2.x; fx[1] = fx2.y;
-        fy[0] = fy2.x; fy[1] = fy2.y;
-        edge_flux<FLUX, T>(tl[NG - 1], tr[NG - 1], dcRL, nx, ny, g, H0, fz[NG - 1], fx[NG - 1], fy[NG - 1]);
-      } else {
+    // both sides' values at the points, in L's point order
+    T lv[NG][3], rv[NG][3];
+    const T hh = T(0.5) * hl, hp = T(0.5) * g;
+    if constexpr (P == 2 && sizeof(T) == 4 && DG_PACKED_FLUX) {  // points 0 and 1 packed, point 2 alone
+      const Trace2 L2{make_float2(tl[0].d, tl[1].d), make_float2(tl[0].H, tl[1].H), make_float2(tl[0].qx, tl[1].qx),
+                      make_float2(tl[0].qy, tl[1].qy)};
+      const Trace2 R2{make_float2(tr[0].d, tr[1].d), make_float2(tr[0].H, tr[1].H), make_float2(tr[0].qx, tr[1].qx),
+                      make_float2(tr[0].qy, tr[1].qy)};
+      f2 fz2, fx2, fy2, l2v[3], r2v[3];
+      FluxAux2 ax2;
+      edge_flux_pair2<FLUX>(L2, R2, p2(dcRL), p2(nx), p2(ny), g, H0, fz2, fx2, fy2, ax2);
+      if (river) fz2 = p2(-2.f * qr);
+      const f2 w = mul2(make_float2(tab.gw[0], tab.gw[1]), p2(hh));
+      side_points<f2>(L2.d, L2.H, R2.d, R2.H, p2(dcRL), p2(nx), p2(ny), w, mul2(w, p2(hp)), fz2, fx2, fy2, l2v, r2v);
+      T fz, fx, fy;
+      edge_flux2<FLUX, T>(tl[2], tr[2], dcRL, nx, ny, g, H0, fz, fx, fy);
+      if (river) fz = -2.f * qr;
+      const T w2 = tab.gw[2] * hh;
+      side_points<T>(tl[2].d, tl[2].H, tr[2].d, tr[2].H, dcRL, nx, ny, w2, w2 * hp, fz, fx, fy, lv[2], rv[2]);
 #pragma unroll
-        for (int k = 0; k < NG; ++k) edge_flux<FLUX, T>(tl[k], tr[k], dcRL, nx, ny, g, H0, fz[k], fx[k], fy[k]);
+      for (int v = 0; v < 3; ++v) {
+        lv[0][v] = l2v[v].x;
+        lv[1][v] = l2v[v].y;
+        rv[0][v] = r2v[v].x;
+        rv[1][v] = r2v[v].y;
       }
-      if (river) {
+    } else {
 #pragma unroll
-        for (int k = 0; k < NG; ++k) fz[k] = -qr;  // the specified normal flow is the mass flux
+      for (int k = 0; k < NG; ++k) {
+        T fz, fx, fy;
+        edge_flux2<FLUX, T>(tl[k], tr[k], dcRL, nx, ny, g, H0, fz, fx, fy);
+        if (river) fz = T(-2) * qr;  // the specified normal flow is the mass flux
+        const T w = P == 1 ? hh : tab.gw[k] * hh;  // both Gauss weights are 1 at p = 1
+        side_points<T>(tl[k].d, tl[k].H, tr[k].d, tr[k].H, dcRL, nx, ny, w, w * hp, fz, fx, fy, lv[k], rv[k]);
       }
+    }
+    T ec = lv[0][0];  // mass flux integral along n (L's outward normal)
 #pragma unroll
-      for (int k = 0; k < NG; ++k) ec = fma(tab.gw[k], fz[k], ec);
-      ec = ec * hl;
-      // wet/dry closure: no water leaves a dry element (interior: either side; ocean/river: L)
-      closed = (dryL && ec > T(0)) || (dryR && ec < T(0));
+    for (int k = 1; k < NG; ++k) ec += lv[k][0];
+    // wet/dry closure: no water leaves a dry element (interior: either side; ocean/river: L)
+    const bool closed = land || (dryL && ec > T(0)) || (dryR && ec < T(0));
+    if (closed) {  // walls, each side from its own trace
+      ec = T(0);
+#pragma unroll
+      for (int k = 0; k < NG; ++k) {
+        const T w = tab.gw[k] * hl;
+        const T cl = w * wall_coef<FLUX, T>(tl[k], nx, ny, g, H0), cr = w * wall_coef<FLUX, T>(tr[k], -nx, -ny, g, H0);
+        lv[k][0] = rv[k][0] = T(0);
+        lv[k][1] = cl * nx;
+        lv[k][2] = cl * ny;
+        rv[k][1] = -(cr * nx);
+        rv[k][2] = -(cr * ny);
+      }
     }
     T vals[NV + 1];
     if (srcL < TILE) {  // L's slot, in L's point order
-      if (!closed) {
 #pragma unroll
-        for (int k = 0; k < NG; ++k) {
-          const T p = T(0.5) * (pdev(tl[k].d, tl[k].H, g) + pdev(tr[k].d + dcRL, tr[k].H, g));
-          const T wk = tab.gw[k] * hl;
-          vals[k] = wk * fz[k];
-          vals[NG + k] = wk * (fx[k] + p * nx);
-          vals[2 * NG + k] = wk * (fy[k] + p * ny);
-        }
-        if (MASSV) vals[3 * NG] = ec;
-      } else {
-#pragma unroll
-        for (int k = 0; k < NG; ++k) {
-          const T cw = tab.gw[k] * hl * wall_coef<FLUX, T>(tl[k], nx, ny, g, H0);
-          vals[k] = T(0);
-          vals[NG + k] = cw * nx;
-          vals[2 * NG + k] = cw * ny;
-        }
-        if (MASSV) vals[3 * NG] = T(0);
+      for (int k = 0; k < NG; ++k) {
+        vals[k] = lv[k][0];
+        vals[NG + k] = lv[k][1];
+        vals[2 * NG + k] = lv[k][2];
       }
+      if (MASSV) vals[3 * NG] = ec;
       store_side<T, NPR, NV>(flx, srcL, jL, vals);
-      if (!interior && !closed) bdry_acc = acc_addr(bdry_acc, -side_mass<T, NG, MASSV>(vals));  // inflow
+      if (!interior && !closed) bdry_acc = acc_addr(bdry_acc, -ec);  // inflow
     }
     if (interior && srcR < TILE) {  // R's slot, in R's point order (its point k is L's NG-1-k)
-      if (!closed) {
 #pragma unroll
-        for (int kr = 0; kr < NG; ++kr) {
-          const int k = NG - 1 - kr;
-          const T p = T(0.5) * (pdev(tr[k].d, tr[k].H, g) + pdev(tl[k].d - dcRL, tl[k].H, g));
-          const T wk = tab.gw[kr] * hl;
-          vals[kr] = -(wk * fz[k]);
-          vals[NG + kr] = -(wk * (fx[k] + p * nx));
-          vals[2 * NG + kr] = -(wk * (fy[k] + p * ny));
-        }
-        if (MASSV) vals[3 * NG] = -ec;
-      } else {
-#pragma unroll
-        for (int kr = 0; kr < NG; ++kr) {
-          const int k = NG - 1 - kr;
-          const T cw = tab.gw[kr] * hl * wall_coef<FLUX, T>(tr[k], -nx, -ny, g, H0);
-          vals[kr] = T(0);
-          vals[NG + kr] = -(cw * nx);
-          vals[2 * NG + kr] = -(cw * ny);
-        }
-        if (MASSV) vals[3 * NG] = T(0);
+      for (int k = 0; k < NG; ++k) {
+        vals[k] = rv[NG - 1 - k][0];
+        vals[NG + k] = rv[NG - 1 - k][1];
+        vals[2 * NG + k] = rv[NG - 1 - k][2];
       }
+      if (MASSV) vals[3 * NG] = -ec;
       store_side<T, NPR, NV>(flx, srcR, jR, vals);
     }
   }
