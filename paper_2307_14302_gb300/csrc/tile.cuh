@@ -7,33 +7,31 @@
 //      pressure set-up) and the element rain of Eq. rain;
 //   2. edge phase: every edge touching the tile is evaluated ONCE (Sec. 2.3: Roe or LLF flux at
 //      p+1 Gauss points, land/ocean/river ghost states, the wet/dry closure of Sec. 2.4), about 60
-//      edges per tile, one per lane and round.  Both sides' records come from shared memory: the
-//      tile's own records, and the records of the ~23 out-of-tile neighbours staged there with
-//      cp.async while phase 1 runs.  The flux values at the Gauss points, scaled by the Gauss
-//      weight and half the edge length, go into per-(element, local edge) slots in shared memory,
-//      each side in its own point order, with the pressure relative to that side's own mean;
+//      edges per tile, one per lane and round, as the tile's plan lists them.  Both sides' records
+//      come from shared memory: the tile's own records, and the records of the ~23 out-of-tile
+//      neighbours staged there with cp.async while phase 1 runs.  The flux values at the Gauss points,
+//      scaled by the Gauss weight and half the edge length, go into per-(element, local edge) slots in
+//      shared memory, each side as seen along its own edge, with the pressure relative to that side's
+//      own mean;
 //   3. element phase B: each lane lifts its three edge slots into the modal right-hand side,
 //      applies the diagonal inverse mass matrix (Eq. dubiner), the Shu-Osher combination, the
 //      positive-depth operator M Pi_h (Sec. 2.4), stores its record and books its rain volume.
 // Interior edges are oriented canonically (the lower element index is "left"), so an edge on the
 // border of two tiles gives the same bits in both, and the two sides of every edge receive
 // exactly opposite mass fluxes: mass is conserved to rounding of the element means.
+// The three phases are one routine, tile_body, which the small-mesh kernel (steps.cuh) shares.
 //
-// Memory pipeline (per warp): the tile's records, static geometry, neighbour codes, first vertices
-// and metadata arrive in shared memory by TMA bulk copies
-// (cp.async.bulk, one per array, completing on an mbarrier), double-buffered: the next tile's
-// copies are in flight while this tile is computed.  The tile's step-initial records are
-// prefetched into L2 by a bulk prefetch at the start of the tile and read in phase 3; the
-// out-of-tile neighbour records are gathered with 16-byte cp.async.  Every mbarrier wait is
-// bounded: a wait that runs out sets ERR_TIMEOUT in the device error word and the kernel returns.
+// Memory pipeline (per warp): a tile's records and its static block (geometry, plan, first vertices)
+// arrive in shared memory by two TMA bulk copies (cp.async.bulk completing on an mbarrier); the next
+// tile's records, and where the static buffer is doubled its static block too, are in flight while
+// this tile is computed.  The modes of the tile's step-initial records are prefetched into L2 by a
+// bulk prefetch at the start of the tile and read in phase 3; the out-of-tile neighbour records are
+// gathered with 16-byte cp.async.  Every mbarrier wait is bounded: a wait that runs out sets
+// ERR_TIMEOUT in the device error word and the kernel returns.
 //
 // Records are vector-major in shared memory ([RV][32], as in the tile-blocked device array), so
 // the 16-byte reads of a warp, at its own slots or at any mix of neighbour slots, spread over
-// the banks.  Shared memory per warp: the two buffers, the halo records [RV][32], the edge
-// descriptors [96] {left side, right side, left normal} and the edge slots [3][pairs][32], which
-// overlay the consumed static part of the current buffer (about 12 KB in the mixed p = 1 path).
-// Neighbours beyond 32 halo slots (none on Hilbert-ordered meshes; kept for generality) are read
-// from global memory.
+// the banks.  Shared memory per warp: TileLayout.
 //
 // The kernel takes a set of Feature bits (args.h): the generic instantiation has all of them;
 // the specialised ones (tile_spec.cu) leave out the code of the features a run does not have.
