@@ -850,7 +850,7 @@ static bool plan_small(dgswe_h h) {
 }
 
 template <class Pol>
-static cudaError_t enqueue_small(dgswe_h h, int n) {
+static cudaError_t enqueue_small(dgswe_h h, int n, cudaStream_t stream) {
   StepsArgs st;
   std::memset(&st, 0, sizeof st);
   const int S = (int)h->stages.size();
@@ -876,7 +876,7 @@ static cudaError_t enqueue_small(dgswe_h h, int n) {
   st.nstage = S;
   st.nsteps = n;
   st.nrec = S > 2 ? 3 : 2;
-  return launch_steps<Pol>(h->prm.p, h->prm.flux, h->feat, make_args<Pol>(h, S - 1, 0), st, h->s_ctas, h->s_wpc, h->stream);
+  return launch_steps<Pol>(h->prm.p, h->prm.flux, h->feat, make_args<Pol>(h, S - 1, 0), st, h->s_ctas, h->s_wpc, stream);
 }
 
 // time whole steps (every stage; timing runs write only the two scratch records) for each form
@@ -928,12 +928,15 @@ static int build_graph(dgswe_h h, int k) {
   cudaGraph_t g;
   CU(cudaStreamBeginCapture(h->cap, cudaStreamCaptureModeThreadLocal));
   int rc = 0;
-  for (int i = 0; i < nsteps && !rc; ++i)
+  cudaError_t se = cudaSuccess;
+  if (h->small) se = mixed(h) ? enqueue_small<Mixed>(h, nsteps, h->cap) : enqueue_small<Fp64>(h, nsteps, h->cap);
+  for (int i = 0; i < nsteps && !rc && !h->small; ++i)
     for (size_t s = 0; s < h->stages.size() && !rc; ++s) rc = launch_stage_once(h, (int)s, 0, h->cap);
   cudaError_t ce = cudaStreamEndCapture(h->cap, &g);
   if (rc) return rc;
+  if (se != cudaSuccess) return fail(DGSWE_ECUDA, "small-mesh launch: %s", cudaGetErrorString(se));
   if (ce != cudaSuccess) return fail(DGSWE_ECUDA, "graph capture: %s", cudaGetErrorString(ce));
-  h->launches -= nsteps * (long long)h->stages.size() * launches_per_stage(h);  // counted when the graph runs
+  if (!h->small) h->launches -= nsteps * (long long)h->stages.size() * launches_per_stage(h);  // counted when the graph runs
   ce = cudaGraphInstantiate(&h->graph[k], g, 0);
   cudaGraphDestroy(g);
   if (ce != cudaSuccess) {
@@ -1265,10 +1268,21 @@ int dgswe_step(dgswe_h h, int64_t n) {
         if (int rc = launch_stage_once(h, (int)s, 0, h->stream)) return rc;
     return 0;
   }
+  // a single step of a small mesh from a graph: a caller that steps one at a time is bound by the host,
+  // and replaying the launch costs it less than forming it (4.5 us with its kilobyte of arguments; with
+  // it the 400-triangle step and read-out took 38-41 us in a host-bound loop against 35 for a graph of
+  // two tile kernels).  Longer calls are bound by the GPU.
+  if (h->small && n == 1) {
+    if (!h->graph[0])
+      if (int rc = build_graph(h, 0)) return rc;
+    CU(cudaGraphLaunch(h->graph[0], h->stream));
+    h->launches++;
+    return 0;
+  }
   if (h->small) {  // at most 1024 steps (a few milliseconds) per launch
     for (int64_t i = 0; i < n; i += 1024) {
       const int k = (int)std::min<int64_t>(1024, n - i);
-      const cudaError_t e = mixed(h) ? enqueue_small<Mixed>(h, k) : enqueue_small<Fp64>(h, k);
+      const cudaError_t e = mixed(h) ? enqueue_small<Mixed>(h, k, h->stream) : enqueue_small<Fp64>(h, k, h->stream);
       if (e != cudaSuccess) return fail(DGSWE_ECUDA, "small-mesh launch: %s", cudaGetErrorString(e));
       h->launches++;
     }

@@ -134,3 +134,31 @@ def test_a_larger_mesh_in_the_same_context():
     t.step(3)
     t.sync()
     assert np.array_equal(s.state(), t.state())
+
+
+@pytest.mark.parametrize("prec", [D.FP64, D.MIXED])
+def test_single_steps_equal_a_longer_call(prec):
+    """Steps taken one by one (replayed from a graph) give the bits of one call, also after the records
+    have moved to other memory and after a new state."""
+    import torch
+
+    w = _basin(9, 5)
+    a, b = (D.from_workload(w, precision=prec) for _ in range(2))
+    for s in (a, b):
+        s.step(1)
+    mem = torch.empty(a.record_bytes(), dtype=torch.uint8, device="cuda")
+    a.bind_device(mem.data_ptr(), mem.numel())
+    for _ in range(4):
+        a.step(1)
+    b.step(4)
+    for s in (a, b):
+        s.sync()
+    assert np.array_equal(a.state(), b.state()) and a.ledger()["steps"] == b.ledger()["steps"] == 5
+    for s in (a, b):
+        s.set_state(w.zeta0)
+    a.step(1)
+    a.step(1)
+    b.step(2)
+    for s in (a, b):
+        s.sync()
+    assert np.array_equal(a.state(), b.state())
