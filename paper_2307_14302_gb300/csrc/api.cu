@@ -630,13 +630,15 @@ static int build_layout(dgswe_h h) {
   if (mx) plan_bytes<Mixed>(h->ntiles, pb, pxb);
   else plan_bytes<Fp64>(h->ntiles, pb, pxb);
   if (h->stat.alloc(pb) || h->plan_x.alloc(pxb)) return fail(DGSWE_ENOMEM, "device allocation failed");
-  CU(cudaDeviceSynchronize());  // the uploads above ran on the default stream, this stream does not wait for it
+  CU(cudaMemcpy(h->scen.p, sd.data(), sizeof(ScenDev) * ns, cudaMemcpyHostToDevice));
+  // every upload above ran on the default stream and may not have landed (a copy from pageable memory
+  // returns before its transfer); the kernels below read them on a stream that does not wait for it
+  CU(cudaDeviceSynchronize());
   CU((mx ? launch_plan<Mixed> : launch_plan<Fp64>)(h->nbr.as<int4>(), h->geo.as<uint4>(), h->nodes.as<int4>(),
                                                    h->xy64.as<double>(), h->tile_meta.as<int4>(), h->ntiles, h->rv,
                                                    h->stat.as<uint4>(), h->plan_x.as<int32_t>(), h->stream));
   h->launches++;
   h->wcur = 0;
-  CU(cudaMemcpy(h->scen.p, sd.data(), sizeof(ScenDev) * ns, cudaMemcpyHostToDevice));
   for (size_t s = 0; s < ns; ++s) {
     if (!sd[s].rrec) continue;
     cudaError_t ce = mx ? launch_rain_records<Mixed>(h->scen.as<ScenDev>(), (int)s, h->nodes.as<int4>(), h->xy64.as<double>(),

@@ -1,0 +1,61 @@
+"""Order between the default stream and the library's own stream, on the CPU.
+
+The library's stream is non-blocking, so nothing orders it against uploads on the default stream but a
+synchronisation.  A stand-in for the CUDA runtime (order_cudart.cpp, loaded before the real one in a child
+process) follows the calls of a few programs and reports every order that CUDA does not promise."""
+import os
+import subprocess
+import sys
+
+import pytest
+
+from paper_2307_14302_gb300 import build as B
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+ROOT = os.path.dirname(HERE)
+
+PRELUDE = """
+import ctypes, sys
+import numpy as np
+from paper_2307_14302_gb300 import dgswe as D
+from paper_2307_14302_gb300 import workloads as W
+
+def basin(nx, ny, grid=False):
+    w = W.basin_c1(nx=nx, ny=ny)
+    if grid:
+        w.rain_nodal = None
+        w.rain_grid = W.RainGrid(3, 2, 4, 0.0, 0.0, 5e3, 5e3, 0.0, 600.0, np.ones((4, 2, 3), np.float32))
+    return w
+"""
+EPILOGUE = """
+r = ctypes.CDLL(None).order_report
+r.restype = ctypes.c_char_p
+sys.stdout.write(r().decode())
+"""
+
+PROGRAMS = {
+    "gridded_rain": """
+s = D.from_workload(basin(9, 5, grid=True), dt=1.0, precision=PREC, block=64, split=2)
+s.sync()
+""",
+}
+
+
+@pytest.fixture(scope="module")
+def runtime(tmp_path_factory):
+    B.build()
+    so = tmp_path_factory.mktemp("order") / "order_cudart.so"
+    inc = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(B._nvcc()))), "include")
+    subprocess.run(["g++", "-std=c++17", "-O1", "-shared", "-fPIC", f"-I{inc}", "-o", str(so),
+                    os.path.join(HERE, "order_cudart.cpp")], check=True)
+    return so
+
+
+@pytest.mark.parametrize("prec", ["D.FP64", "D.MIXED"])
+@pytest.mark.parametrize("program", list(PROGRAMS))
+def test_no_unordered_work(program, prec, runtime):
+    code = PRELUDE + f"PREC = {prec}\n" + PROGRAMS[program] + EPILOGUE
+    env = dict(os.environ, LD_PRELOAD=str(runtime), PYTHONPATH=ROOT)
+    r = subprocess.run([sys.executable, "-c", code], env=env, capture_output=True, text=True, timeout=600)
+    assert r.returncode == 0, r.stderr[-2000:]
+    assert r.stdout == ""
