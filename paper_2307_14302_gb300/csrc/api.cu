@@ -657,10 +657,12 @@ static int build_layout(dgswe_h h) {
   return 0;
 }
 
-// fill the per-scenario time-step fields once dt is known
+// fill the per-scenario time-step fields once dt is known (on the context's stream: the first step
+// follows there, and nothing else orders it behind a copy on the default stream)
 static int upload_dt(dgswe_h h) {
   std::vector<ScenDev> sd(h->sc.size());
-  CU(cudaMemcpy(sd.data(), h->scen.p, sizeof(ScenDev) * sd.size(), cudaMemcpyDeviceToHost));
+  CU(cudaMemcpyAsync(sd.data(), h->scen.p, sizeof(ScenDev) * sd.size(), cudaMemcpyDeviceToHost, h->stream));
+  CU(cudaStreamSynchronize(h->stream));
   for (size_t s = 0; s < sd.size(); ++s) {
     ScenDev& D = sd[s];
     D.dt = h->sc[s].dt;
@@ -674,7 +676,8 @@ static int upload_dt(dgswe_h h) {
       D.bw[k] = h->stages[k].bw;
     }
   }
-  CU(cudaMemcpy(h->scen.p, sd.data(), sizeof(ScenDev) * sd.size(), cudaMemcpyHostToDevice));
+  CU(cudaMemcpyAsync(h->scen.p, sd.data(), sizeof(ScenDev) * sd.size(), cudaMemcpyHostToDevice, h->stream));
+  CU(cudaStreamSynchronize(h->stream));  // sd is gone after this
   return 0;
 }
 

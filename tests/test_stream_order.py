@@ -38,6 +38,12 @@ PROGRAMS = {
 s = D.from_workload(basin(9, 5, grid=True), dt=1.0, precision=PREC, block=64, split=2)
 s.sync()
 """,
+    # the time step's upload, then the first step at once in a shape that is not timed
+    "fixed_shape": """
+s = D.from_workload(basin(9, 5), precision=PREC, block=64, split=2)
+s.step(3)
+s.sync()
+""",
 }
 
 
