@@ -681,18 +681,20 @@ static int upload_dt(dgswe_h h) {
   return 0;
 }
 
-// launch shape change: fold the ledger slots of the old shape into the host accumulators
+// launch shape change: fold the ledger slots of the old shape into the host accumulators, on the
+// context's stream: steps in flight book their volumes before they are read, later ones after the clear
 static int fold_ledger(dgswe_h h) {
   if (h->wcur > 0) {
     const size_t ns = h->sc.size();
     std::vector<double> part(2 * (size_t)h->wslots * ns);
-    CU(cudaMemcpy(part.data(), h->ledger.p, 8 * part.size(), cudaMemcpyDeviceToHost));
+    CU(cudaMemcpyAsync(part.data(), h->ledger.p, 8 * part.size(), cudaMemcpyDeviceToHost, h->stream));
+    CU(cudaStreamSynchronize(h->stream));
     for (size_t s = 0; s < ns; ++s)
       for (int w = 0; w < h->wcur; ++w) {
         h->led_rain[s] += part[2 * (s * h->wslots + w)];
         h->led_bdry[s] += part[2 * (s * h->wslots + w) + 1];
       }
-    CU(cudaMemset(h->ledger.p, 0, 8 * part.size()));
+    CU(cudaMemsetAsync(h->ledger.p, 0, 8 * part.size(), h->stream));
   }
   h->drop_graphs();
   return 0;

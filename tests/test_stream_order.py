@@ -44,6 +44,27 @@ s = D.from_workload(basin(9, 5), precision=PREC, block=64, split=2)
 s.step(3)
 s.sync()
 """,
+    # the ledger of the shape before is folded, then the first launch books into it
+    "cluster": """
+s = D.from_workload(basin(9, 5), precision=PREC)
+s.step(3)
+s.sync()
+""",
+    # a choice of shape asked for while steps are in flight
+    "retuned": """
+s = D.from_workload(basin(9, 5), precision=PREC, block=256, split=1)
+s.step(50)
+s.set_launch(0)
+s.step(1)
+s.sync()
+""",
+    "retuned_large": """
+s = D.from_workload(basin(90, 50), precision=PREC, block=256, split=1)
+s.step(50)
+s.set_launch(0)
+s.step(1)
+s.sync()
+""",
 }
 
 
