@@ -350,6 +350,7 @@ static int run_features(dgswe_h h, const std::vector<int32_t>& nbr) {
 
 static int build_layout(dgswe_h h) {
   DeviceGuard dg_(h->device);
+  CU(cudaStreamSynchronize(h->stream));  // steps of the state before may still run on what is replaced here
   const int p = h->prm.p, np = np_of(p);
   const bool mx = mixed(h);
   h->np = np;

@@ -65,6 +65,41 @@ s.set_launch(0)
 s.step(1)
 s.sync()
 """,
+    # a new state, and a new mesh, while steps are in flight
+    "new_state": """
+w, v = basin(9, 5), basin(13, 7, grid=True)
+s = D.from_workload(w, precision=PREC)
+s.step(50)
+s.set_state(w.zeta0)
+s.step(50)
+s.set_mesh(v.mesh)
+s.set_fields(v.hb, v.manning)
+s.set_rain_grid(v.rain_grid)
+s.set_state(v.zeta0)
+s.step(1)
+s.sync()
+""",
+    "read_outs": """
+s = D.from_workload(basin(90, 50), precision=PREC, dt=1.0)
+s.step(50)
+s.ledger()
+s.step(1)
+s.volume()
+s.step(1)
+s.dry()
+s.step(1)
+a = s.state_arrays()
+s.step(1)
+s.load_state(*a)
+s.step(1)
+s.exchange(*a)
+e = D.Ensemble([s, D.from_workload(basin(9, 5), precision=PREC)])
+e.step(3)
+e.ledger(1)
+e.step(1)
+e.state(0)
+e.sync()
+""",
 }
 
 
