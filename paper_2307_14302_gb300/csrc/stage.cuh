@@ -119,6 +119,26 @@ __device__ __forceinline__ ff acc_addmul(ff s, ff a, float b) {
 }
 __device__ __forceinline__ double acc_norm(double a) { return a; }
 __device__ __forceinline__ ff acc_norm(ff a) { return quick_two_sum(a.hi, a.lo); }
+// sum of very many values: doubles, or pairs of floats in three words (the roundings of the first two are
+// kept, so that equal addends do not round the same way every time)
+struct fff {
+  float a, b, c;
+};
+template <class Acc>
+struct LongSum {
+  using type = double;
+};
+template <>
+struct LongSum<ff> {
+  using type = fff;
+};
+__device__ __forceinline__ void long_add(double& s, double v) { s += v; }
+__device__ __forceinline__ void long_add(fff& s, ff v) {
+  const ff t = two_sum(s.a, v.hi), u = two_sum(s.b, v.lo), w = two_sum(u.hi, t.lo);
+  s = {t.hi, w.hi, __fadd_rn(s.c, __fadd_rn(u.lo, w.lo))};
+}
+__device__ __forceinline__ double long_d(double s) { return s; }
+__device__ __forceinline__ double long_d(fff s) { return (double)s.a + ((double)s.b + (double)s.c); }
 // a - b rounded to the working precision (float: within an ulp, from the words' differences)
 __device__ __forceinline__ double acc_sub_r(double a, double b) { return a - b; }
 __device__ __forceinline__ float acc_sub_r(ff a, ff b) { return __fadd_rn(__fsub_rn(a.hi, b.hi), __fsub_rn(a.lo, b.lo)); }
