@@ -1185,7 +1185,9 @@ __device__ __forceinline__ RainRec<T> rain_records(const ScenDev& S, double t) {
   return {r, S.gnt > 1 ? r + S.rstride : r, (T)(gt - (double)it)};
 }
 template <class T>
-__device__ __forceinline__ T rain_blend(T v0, T v1, T f) { return fma(f, v1 - v0, v0); }
+__device__ __forceinline__ T rain_blend(T v0, T v1, T f) {
+  return fma(f, v1, (T(1) - f) * v0);  // each record exactly where it alone counts: no rounding of v1 - v0
+}
 
 // element means of every grid record (in FP64, stored in the path's type): thread e forms its
 // vertices' cells and weights once and walks the records
