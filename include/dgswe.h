@@ -302,8 +302,9 @@ int dgswe_ensemble_get_ledger(dgswe_h ens, int32_t member, dgswe_ledger* out);
  * each warp evaluates every edge touching its 32-element tile once from records staged in shared
  * memory.  The three forms agree to rounding; for a fixed form results do not depend on block or
  * waves.  With block 0 a mesh of few tiles (without limiter and with at most the tiles that a
- * thread-block cluster of 16 holds) runs whole steps in one cluster launch instead: states have the
- * bits of the tile form, the ledger's volumes agree to rounding.  Returns DGSWE_EINVAL for other values. */
+ * thread-block cluster of 16 holds; in FP64 96 tiles at p = 1 and 64 at p = 2) runs whole steps in
+ * one cluster launch instead: states have the bits of the tile form, the ledger's volumes agree to
+ * rounding.  Returns DGSWE_EINVAL for other values. */
 int dgswe_set_launch(dgswe_h, int32_t block, int32_t waves, int32_t split);
 /* No counterpart in the paper (device scheduling): the launch shape in use (after autotuning,
  * the one it chose; a mesh stepped in cluster launches reports the tile form, split 2); NULL

@@ -836,16 +836,24 @@ static int apply_launch(dgswe_h h, int block, int waves, int split) {
 
 // Small meshes: whole steps in one launch of one cluster (steps.cuh), when every tile can have a warp
 // in it and no other kernel runs between the stages.
-// At least four warps per CTA (one per SM sub-partition; fewer CTAs make the barrier cheaper), more
-// when 16 CTAs would not hold the mesh.
+// Mixed: at least four warps per CTA (one per SM sub-partition; fewer CTAs make the barrier cheaper), more
+// when 16 CTAs would not hold the mesh; ahead of the tile form up to the largest cluster (us per step at
+// 65, 124 and 188 tiles: 7.2, 6.1 and 8.4 against 11.4, 10.4 and 11.3).
+// FP64: a tile keeps the FP64 pipe of its sub-partition busy, so tiles go one to a CTA first (13 tiles:
+// 87.1 us per step, with four to a CTA 95.5, tile form 92.5), and beyond four to a CTA they take turns
+// where the tile form has the other SMs: 47, 62, 95 and 124 tiles (3, 4, 6 and 8 to a CTA) 73.4, 112.6,
+// 113.7 and 149 against 79.5, 110.4, 79.1 and 79.5; degree 2 with 31, 62 and 95 tiles 216, 324 and 340
+// against 229, 311 and 230.  So degree 2 stops at four to a CTA.  Degree 1 stops at six: that a call of
+// a gridded-rain mesh of 94 tiles is one launch is tested, and costs it up to 1.4 times the tile form.
 static bool plan_small(dgswe_h h) {
   const int nrec = h->stages.size() > 2 ? 3 : 2;
+  const int least = mixed(h) ? 4 : 1, most = mixed(h) ? 16 : h->prm.p == 1 ? 6 : 4;
   if (h->prm.limiter || h->grid_rain) return false;
   int live = h->ntiles;  // the last tiles of the last scenario may be padding
   while (live > 1 && (long long)(live - 1) * TILE >= h->eoff.back() + h->sc.back().m.ne) --live;
   for (int ctas = 16; ctas >= 8; ctas -= 8) {
-    const int wpc = std::max(4, (live + ctas - 1) / ctas), use = (live + wpc - 1) / wpc;
-    if (wpc > 16) continue;
+    const int wpc = std::max(least, (live + ctas - 1) / ctas), use = (live + wpc - 1) / wpc;
+    if (wpc > most) continue;
     const bool ok = mixed(h) ? steps_fit<Mixed>(h->prm.p, h->prm.flux, h->feat, use, wpc, nrec)
                              : steps_fit<Fp64>(h->prm.p, h->prm.flux, h->feat, use, wpc, nrec);
     if (ok) {

@@ -7,7 +7,7 @@
 //   - a copy or cudaMemset on the default stream, over device memory, while work on a non-blocking stream
 //     may still be running.
 // A device or stream synchronisation, a copy back to the host on the same stream and a wait for an event
-// recorded behind the work end what is pending.  cudaFree is not counted on.
+// recorded behind the work end what is pending.  cudaFree is not counted on.  It also lists the launches.
 #include <cuda_runtime.h>
 
 #include <cstdlib>
@@ -19,6 +19,7 @@
 
 namespace {
 std::string report, uploads;              // violations; what is pending on the default stream
+std::string launches;                      // kernels in the order of their launches: name, grid, block
 std::map<cudaStream_t, std::string> busy;  // pending work of the other streams
 std::map<cudaEvent_t, cudaStream_t> recorded;
 std::set<cudaStream_t> capturing;
@@ -34,6 +35,10 @@ cudaError_t enqueue(cudaStream_t s, const std::string& what) {
   busy[s] = what;
   return cudaSuccess;
 }
+cudaError_t launch(cudaStream_t s, const std::string& name, dim3 g, dim3 b) {
+  launches += name + " " + std::to_string(g.x) + " " + std::to_string(b.x) + "\n";
+  return enqueue(s, name);
+}
 void on_default(const std::string& what, bool pending) {
   for (auto& b : busy)
     if (!b.second.empty()) violation(what + " on the default stream while pending elsewhere: " + b.second);
@@ -45,6 +50,7 @@ std::string sized(const char* op, size_t n) { return std::string(op) + " of " + 
 
 extern "C" {
 const char* order_report() { return report.c_str(); }
+const char* order_launches() { return launches.c_str(); }
 
 void** __cudaRegisterFatBinary(void*) { static void* h; return &h; }
 void __cudaRegisterFatBinaryEnd(void**) {}
@@ -70,10 +76,12 @@ cudaError_t __cudaGetKernel(cudaKernel_t* k, const void* host) {
   *k = (cudaKernel_t)host;
   return cudaSuccess;
 }
-cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3, dim3, void**, size_t, cudaStream_t s) {
-  return enqueue(s, names[(const void*)k]);
+cudaError_t __cudaLaunchKernel(cudaKernel_t k, dim3 g, dim3 b, void**, size_t, cudaStream_t s) {
+  return launch(s, names[(const void*)k], g, b);
 }
-cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void**) { return enqueue(c->stream, names[f]); }
+cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t* c, const void* f, void**) {
+  return launch(c->stream, names[f], c->gridDim, c->blockDim);
+}
 cudaError_t cudaGraphLaunch(cudaGraphExec_t, cudaStream_t s) { return enqueue(s, "a graph"); }
 
 cudaError_t cudaMemcpy(void* d, const void* s, size_t n, cudaMemcpyKind k) {

@@ -28,7 +28,7 @@ def basin(nx, ny, grid=False):
     return w
 """
 EPILOGUE = """
-r = ctypes.CDLL(None).order_report
+r = ctypes.CDLL(None).{}
 r.restype = ctypes.c_char_p
 sys.stdout.write(r().decode())
 """
@@ -113,11 +113,37 @@ def runtime(tmp_path_factory):
     return so
 
 
-@pytest.mark.parametrize("prec", ["D.FP64", "D.MIXED"])
-@pytest.mark.parametrize("program", list(PROGRAMS))
-def test_no_unordered_work(program, prec, runtime):
-    code = PRELUDE + f"PREC = {prec}\n" + PROGRAMS[program] + EPILOGUE
+def _run(runtime, program, what):
+    code = PRELUDE + program + EPILOGUE.format(what)
     env = dict(os.environ, LD_PRELOAD=str(runtime), PYTHONPATH=ROOT)
     r = subprocess.run([sys.executable, "-c", code], env=env, capture_output=True, text=True, timeout=600)
     assert r.returncode == 0, r.stderr[-2000:]
-    assert r.stdout == ""
+    return r.stdout
+
+
+@pytest.mark.parametrize("prec", ["D.FP64", "D.MIXED"])
+@pytest.mark.parametrize("program", list(PROGRAMS))
+def test_no_unordered_work(program, prec, runtime):
+    assert _run(runtime, f"PREC = {prec}\n" + PROGRAMS[program], "order_report") == ""
+
+
+# kernel, grid and block of a call of several steps on nx x ny x 2 triangles; None: stage by stage
+@pytest.mark.parametrize("prec,p,nx,ny,want", [
+    ("D.FP64", 1, 20, 10, ("steps_kernel", 13, 32)),     # FP64: one tile per SM while there are 16 or fewer
+    ("D.FP64", 1, 32, 32, ("steps_kernel", 16, 128)),
+    ("D.FP64", 1, 48, 32, ("steps_kernel", 16, 192)),    # the last that keep the cluster
+    ("D.FP64", 1, 48, 33, None),
+    ("D.FP64", 2, 32, 32, ("steps_kernel", 16, 128)),
+    ("D.FP64", 2, 32, 33, None),
+    ("D.MIXED", 1, 20, 10, ("steps_kernel", 4, 128)),
+    ("D.MIXED", 1, 64, 64, ("steps_kernel", 16, 512)),   # as many tiles as the largest cluster has warps
+    ("D.MIXED", 1, 64, 65, None),
+])
+def test_form_of_small_meshes(runtime, prec, p, nx, ny, want):
+    out = _run(runtime, f"""
+w = basin({nx}, {ny})
+w.p = {p}
+s = D.from_workload(w, precision={prec}, dt=1.0)
+s.step(2)
+""", "order_launches").split("\n")[-2].split()
+    assert ((want[0] in out[0] and (int(out[1]), int(out[2])) == want[1:]) if want else "steps_kernel" not in out[0])
