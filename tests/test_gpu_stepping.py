@@ -1,4 +1,5 @@
-"""Ways of stepping at the edges of their ranges."""
+"""Ways of stepping at the edges of their ranges: the largest cluster, long graphs, and ensembles whose
+members have different kinds of rain."""
 import numpy as np
 import pytest
 
@@ -40,3 +41,52 @@ def test_the_largest_clusters(prec, p, nx, ny, cluster):
     b.sync()
     if a.launch()[2] == 2:  # the same form: the same bits
         assert np.array_equal(a.state(), b.state())
+
+
+@pytest.mark.parametrize("limiter", [False, True])
+@pytest.mark.parametrize("prec", [D.FP64, D.MIXED])
+def test_every_graph_length_equals_direct_launches(prec, limiter):
+    """63 steps are one graph each of 32, 16, 8, 4, 2 and 1 steps."""
+    w = W.coastal_c2(12_000, seed=23, fast_mesh=True)
+    w.cfl = 0.1
+    a, b = (D.from_workload(w, precision=prec, block=128, waves=1, split=2, limiter=limiter) for _ in range(2))
+    b.set_graphs(False)
+    for s in (a, b):
+        n0 = s.launch_count()
+        s.step(63)
+        assert s.launch_count() - n0 == 63 * 2 * (2 if limiter else 1)
+        s.sync()
+    assert np.array_equal(a.state(), b.state()) and a.ledger() == b.ledger()
+
+
+def _gridded(nx, ny, nt, seed):
+    w = W.basin_c1(nx=nx, ny=ny, seed=seed)
+    w.rain_nodal = None
+    f = np.random.default_rng(seed).uniform(0, 100, (nt, 3, 4)).astype(np.float32)
+    w.rain_grid = W.RainGrid(4, 3, nt, 0.0, 0.0, 3e3, 2e3, 0.0, 7.0, f)
+    return w
+
+
+@pytest.mark.parametrize("k", [1, 6])
+def test_an_ensemble_of_different_rains(k):
+    """Gridded (two grids), storm, nodal and no rain side by side, in a cluster and stage by stage: in FP64,
+    where one instantiation serves every run, the bits of the members' solo runs."""
+    coastal = W.coastal_c2(500 * k * k, seed=23, fast_mesh=True)
+    coastal.cfl = 0.1
+    dry = W.basin_c1(nx=5 * k, ny=3 * k)
+    dry.rain_nodal = None
+    ws = [_gridded(6 * k, 4 * k, 5, 1), coastal, W.basin_c1(nx=7 * k, ny=3 * k), _gridded(5 * k, 5 * k, 2, 2), dry]
+    solo = [D.from_workload(w, precision=D.FP64, block=64, waves=1, split=2) for w in ws]
+    ens = D.Ensemble([D.from_workload(w, precision=D.FP64) for w in ws])
+    ens.step(1)
+    n0 = ens.launch_count()
+    ens.step(6)
+    assert (ens.launch_count() - n0 == 1) == (k == 1)
+    ens.sync()
+    same = ens.launch()[2] == 2
+    for i, s in enumerate(solo):
+        s.step(7)
+        s.sync()
+        want = s.state()
+        assert np.array_equal(ens.state(i), want) if same else np.abs(ens.state(i) - want).max() <= 1e-11 * np.abs(want).max()
+        assert ens.ledger(i)["rel_err"] < 1e-12
