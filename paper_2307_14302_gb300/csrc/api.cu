@@ -774,8 +774,8 @@ static int launch_stage_once(dgswe_h h, int stage, int tune, cudaStream_t s) {
   const int grid = h->grid;
   cudaError_t e = cudaSuccess;
   if (h->grid_rain) {  // nodal gridded rain at this stage's time
-    e = mixed(h) ? launch_node_rain<Mixed>(make_args<Mixed>(h, stage, tune), h->nn_total, s)
-                 : launch_node_rain<Fp64>(make_args<Fp64>(h, stage, tune), h->nn_total, s);
+    e = mixed(h) ? launch_node_rain<Mixed>(make_args<Mixed>(h, stage, tune), h->xy64.as<double>(), h->nn_total, s)
+                 : launch_node_rain<Fp64>(make_args<Fp64>(h, stage, tune), h->xy64.as<double>(), h->nn_total, s);
     if (e != cudaSuccess) return fail(DGSWE_ECUDA, "node rain launch: %s", cudaGetErrorString(e));
     h->launches++;
   }

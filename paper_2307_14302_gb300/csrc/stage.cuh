@@ -1140,33 +1140,8 @@ __global__ void __launch_bounds__(256) edge_kernel(const StageArgs<Pol> a) {
   }
 }
 
-// gridded rain (mm/h records, bilinear in space, linear in time, clamped to the grid) at a
-// point and time, in m/s (Sec. 2.5)
-template <class T>
-__device__ __forceinline__ T grid_rain(const ScenDev& S, const ForcingT<T>& F, T px, T py, T t) {
-  T gx = (px - F.grid[0]) * F.grid[2], gy = (py - F.grid[1]) * F.grid[3];
-  T gt = (t - F.grid[4]) * F.grid[5];
-  gx = fmin(fmax(gx, T(0)), T(S.gnx - 1));
-  gy = fmin(fmax(gy, T(0)), T(S.gny - 1));
-  gt = fmin(fmax(gt, T(0)), T(S.gnt - 1));
-  const int ix = min(max((int)floor(gx), 0), max(S.gnx - 2, 0));
-  const int iy = min(max((int)floor(gy), 0), max(S.gny - 2, 0));
-  const int it = min(max((int)floor(gt), 0), max(S.gnt - 2, 0));
-  const T fx = gx - T(ix), fy = gy - T(iy), ft = gt - T(it);
-  const int ix1 = S.gnx > 1 ? ix + 1 : ix, iy1 = S.gny > 1 ? iy + 1 : iy;
-  T val[2];
-#pragma unroll
-  for (int qq = 0; qq < 2; ++qq) {
-    const int kk = S.gnt > 1 ? it + qq : 0;
-    const float* Gr = S.grid + (size_t)kk * S.gnx * S.gny;
-    const T v00 = Gr[(size_t)iy * S.gnx + ix], v10 = Gr[(size_t)iy * S.gnx + ix1];
-    const T v01 = Gr[(size_t)iy1 * S.gnx + ix], v11 = Gr[(size_t)iy1 * S.gnx + ix1];
-    val[qq] = (T(1) - fy) * ((T(1) - fx) * v00 + fx * v10) + fy * ((T(1) - fx) * v01 + fx * v11);
-  }
-  return ((T(1) - ft) * val[0] + ft * val[1]) * T(1.0 / 3.6e6);
-}
-
-// Gridded rain from per-element records.  Eq. rain's element rate (mean of three nodal rates) and
+// Gridded rain (mm/h records, bilinear in space, linear in time, clamped to the grid, Sec. 2.5) from
+// per-element records.  Eq. rain's element rate (mean of three nodal rates) and
 // the bilinear interpolation are linear in the grid's values, so the element mean of every record
 // can be formed once, when the state is set, and a stage only blends the two records around its
 // time: two coalesced loads per element.  Before, each stage interpolated the grid to the nodes in
@@ -1189,6 +1164,26 @@ __device__ __forceinline__ T rain_blend(T v0, T v1, T f) {
   return fma(f, v1, (T(1) - f) * v0);  // each record exactly where it alone counts: no rounding of v1 - v0
 }
 
+// a point's cell of a scenario's rain grid (coordinates outside the grid take its edge): place of the lower
+// corner in a record, steps to the next column and row (0 on a grid of one), position in the cell
+struct GridCell {
+  long long at, dx, dy;
+  double fx, fy;
+};
+__device__ __forceinline__ GridCell grid_cell(const ScenDev& S, double x, double y) {
+  const double gx = fmin(fmax((x - S.d.grid[0]) * S.d.grid[2], 0.0), (double)(S.gnx - 1));
+  const double gy = fmin(fmax((y - S.d.grid[1]) * S.d.grid[3], 0.0), (double)(S.gny - 1));
+  const int ix = min((int)gx, max(S.gnx - 2, 0)), iy = min((int)gy, max(S.gny - 2, 0));
+  return {(long long)iy * S.gnx + ix, S.gnx > 1 ? 1 : 0, S.gny > 1 ? S.gnx : 0, gx - ix, gy - iy};
+}
+// a record at that place
+template <class V>
+__device__ __forceinline__ V cell_value(const float* g, const GridCell& c, V fx, V fy) {
+  const V lo = (V(1) - fx) * g[0] + fx * g[c.dx];
+  const V hi = (V(1) - fx) * g[c.dy] + fx * g[c.dy + c.dx];
+  return (V(1) - fy) * lo + fy * hi;
+}
+
 // element means of every grid record (in FP64, stored in the path's type): thread e forms its
 // vertices' cells and weights once and walks the records
 template <class T>
@@ -1198,46 +1193,39 @@ __global__ void __launch_bounds__(256) rain_record_kernel(const ScenDev* scen, i
   for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < ne; e += (long long)gridDim.x * blockDim.x) {
     const int4 nd = nodes[S.elem_begin + e];
     const int v[3] = {nd.x, nd.y, nd.z};
-    long long at[3], dx[3], dy[3];
-    double fx[3], fy[3];
+    GridCell c[3];
 #pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      const double gx = fmin(fmax((xy64[2 * (long long)v[i]] - S.d.grid[0]) * S.d.grid[2], 0.0), (double)(S.gnx - 1));
-      const double gy = fmin(fmax((xy64[2 * (long long)v[i] + 1] - S.d.grid[1]) * S.d.grid[3], 0.0), (double)(S.gny - 1));
-      const int ix = min((int)gx, max(S.gnx - 2, 0)), iy = min((int)gy, max(S.gny - 2, 0));
-      fx[i] = gx - ix;
-      fy[i] = gy - iy;
-      at[i] = (long long)iy * S.gnx + ix;
-      dx[i] = S.gnx > 1 ? 1 : 0;
-      dy[i] = S.gny > 1 ? S.gnx : 0;
-    }
+    for (int i = 0; i < 3; ++i) c[i] = grid_cell(S, xy64[2 * (long long)v[i]], xy64[2 * (long long)v[i] + 1]);
     const float* G = S.grid;
     for (int k = 0; k < S.gnt; ++k, G += (size_t)S.gnx * S.gny) {
       double sum = 0.0;
 #pragma unroll
-      for (int i = 0; i < 3; ++i) {
-        const float* g = G + at[i];
-        const double lo = (1.0 - fx[i]) * g[0] + fx[i] * g[dx[i]];
-        const double hi = (1.0 - fx[i]) * g[dy[i]] + fx[i] * g[dy[i] + dx[i]];
-        sum += (1.0 - fy[i]) * lo + fy[i] * hi;
-      }
+      for (int i = 0; i < 3; ++i) sum += cell_value<double>(G + c[i].at, c[i], c[i].fx, c[i].fy);
       rrec[(size_t)k * stride + e] = (T)(sum * (1.0 / (3.0 * 3.6e6)));
     }
   }
 }
 
 // node kernel, for records whose element means would not fit in memory: the gridded rain of every
-// node at this stage's time, once per node instead of once per (element, vertex)
+// node at this stage's time, once per node instead of once per (element, vertex).  Places in the grid and
+// in time are formed in FP64 and the values blended in the path's type, so that both ways agree to rounding
+// (in FP32 a place was 3e-4 of a record off 250,000 s into 60 s records).
 template <class Pol>
-__global__ void __launch_bounds__(256) node_rain_kernel(const StageArgs<Pol> a, long long nn) {
+__global__ void __launch_bounds__(256) node_rain_kernel(const StageArgs<Pol> a, const double* xy64, long long nn) {
   using T = typename Pol::T;
   const double stepd = (double)a.ctl->step + a.cst;
   for (long long n = (long long)blockIdx.x * blockDim.x + threadIdx.x; n < nn; n += (long long)gridDim.x * blockDim.x) {
     const ScenDev& S = a.scen[a.node_scen[n]];
     if (S.rain_kind != 3 || S.rrec) continue;
-    const ForcingT<T>& F = forcing<T>(S);
-    const T t = (T)(S.d.t0 + stepd * S.d.dt);  // stage time, formed in FP64
-    a.rain_node[n] = grid_rain<T>(S, F, a.node_xy[2 * n], a.node_xy[2 * n + 1], t);
+    const GridCell c = grid_cell(S, xy64[2 * n], xy64[2 * n + 1]);
+    const double gt = fmin(fmax((S.d.t0 + stepd * S.d.dt - S.d.grid[4]) * S.d.grid[5], 0.0), (double)(S.gnt - 1));
+    const int it = min((int)gt, max(S.gnt - 2, 0));
+    const size_t rec = (size_t)S.gnx * S.gny;
+    const float* g0 = S.grid + rec * it + c.at;
+    const float* g1 = S.gnt > 1 ? g0 + rec : g0;
+    const T fx = (T)c.fx, fy = (T)c.fy;
+    a.rain_node[n] = rain_blend<T>(cell_value<T>(g0, c, fx, fy), cell_value<T>(g1, c, fx, fy), (T)(gt - (double)it)) *
+                     T(1.0 / 3.6e6);
   }
 }
 
@@ -2239,8 +2227,8 @@ static inline int grid_for(long long n, int block) {
     return launch_pdl(limit_kernel<POL>, grid_for(ne, 256), 256, 0, s, a, ne);                               \
   }                                                                                                          \
   template <>                                                                                                \
-  cudaError_t launch_node_rain<POL>(const StageArgs<POL>& a, long long nn, cudaStream_t s) {                 \
-    node_rain_kernel<POL><<<grid_for(nn, 256), 256, 0, s>>>(a, nn);                                          \
+  cudaError_t launch_node_rain<POL>(const StageArgs<POL>& a, const double* xy64, long long nn, cudaStream_t s) { \
+    node_rain_kernel<POL><<<grid_for(nn, 256), 256, 0, s>>>(a, xy64, nn);                                    \
     return cudaGetLastError();                                                                               \
   }                                                                                                          \
   template <>                                                                                                \

@@ -35,3 +35,27 @@ def test_after_a_storm_the_last_record_holds(prec, bound, launch):
     s.sync()
     want = 20 * 0.5 * _area(w.mesh).sum() * float(f[1, 0, 0]) * W.MMH
     assert abs(s.ledger()["rain_in"] / want - 1) <= bound
+
+
+def test_the_node_kernel_agrees_to_rounding():
+    """4,400 records on 500k triangles (8.8 GB of element means) go through the node kernel; the two around
+    the run's time, as a grid of their own, through records.  250,000 s into 60 s records, 10 and 90 mm/h in
+    turn.  Both hold FP32 values: a blend and a mean of four roundings each, and the stored rates."""
+    w = W.coastal_c2(500_000, seed=3, fast_mesh=True)
+    w.storm = None
+    f = np.empty((4400, 1, 1), np.float32)
+    f[0::2], f[1::2] = 10.0, 90.0
+    t0 = 250_000.3
+    k = int(t0 // 60.0)
+    rain = []
+    for first, rec in ((0, f), (k, f[k:k + 2])):
+        w.rain_grid = W.RainGrid(1, 1, len(rec), 0.0, 0.0, 1.0, 1.0, 60.0 * first, 60.0, rec)
+        dev = D.from_workload(w, dt=0.2, block=64, waves=1, split=2)
+        dev.set_state(w.zeta0, t0=t0)
+        n0 = dev.launch_count()
+        dev.step(1)
+        assert dev.launch_count() - n0 == (4 if first == 0 else 2)
+        dev.sync()
+        rain.append(dev.ledger()["rain_in"])
+        dev.close()
+    assert abs(rain[0] / rain[1] - 1) <= 10 * 2.0**-24
