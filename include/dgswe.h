@@ -150,7 +150,10 @@ int dgswe_set_rain_nodal(dgswe_h, const double* r_nodal); /* constant in time [n
 /* The moving rain cell of dgswe_storm (the parametric rainfall of Sec. 2.5), copied. */
 int dgswe_set_rain_parametric(dgswe_h, const dgswe_storm* storm);
 /* Gridded records [nt][ny][nx] float32 in mm/h on x0 + i dx, y0 + j dy, times t0 + k dt_rec:
- * bilinear in space, linear in time, clamped at the grid and record ends (Sec. 2.5). */
+ * bilinear in space, linear in time, clamped at the grid and record ends (Sec. 2.5).  The element means of
+ * every record are formed when the state is set, up to 8 GiB of them; beyond that, or where they and the
+ * staging of a state do not fit in memory, the grid is interpolated at every stage, with the same rain to
+ * rounding. */
 int dgswe_set_rain_grid(dgswe_h, int32_t nx, int32_t ny, int32_t nt, double x0, double y0, double dx, double dy,
                         double t0, double dt_rec, const float* mm_per_h);
 

@@ -348,9 +348,38 @@ static int run_features(dgswe_h h, const std::vector<int32_t>& nbr) {
   return f;
 }
 
+// gridded rain: memory for the element means of every record, up to 8 GiB (25 hourly records of 8M
+// triangles are 0.8 GB); else a node kernel interpolates the grid at every stage.  The size decides,
+// not what happens to be free, so that a run repeats; only where the records and the staging of a state
+// exceed what is left after everything else does the node kernel, whose rain agrees to rounding, step in.
+static int alloc_rain_records(dgswe_h h, std::vector<ScenDev>& sd) {
+  const size_t word = mixed(h) ? 4 : 8;
+  size_t need = 0, staging = 0, free_b = 0, total_b = 0;
+  std::vector<size_t> at(sd.size(), 0);
+  for (size_t s = 0; s < sd.size(); ++s) {
+    staging = std::max(staging, 3 * sizeof(double) * (size_t)h->np * h->sc[s].m.ne);
+    if (sd[s].rain_kind != 3) continue;
+    at[s] = need;
+    need += word * sd[s].gnt * (size_t)h->sc[s].m.ne;
+  }
+  h->grid_rain = need > 0;
+  if (need == 0 || need > (size_t)8 << 30) return 0;
+  CU(cudaMemGetInfo(&free_b, &total_b));
+  if (need + staging > free_b) return 0;
+  if (h->rain_rec.alloc(need)) {
+    cudaGetLastError();  // the node kernel takes over
+    return 0;
+  }
+  h->grid_rain = false;
+  for (size_t s = 0; s < sd.size(); ++s)
+    if (sd[s].rain_kind == 3) sd[s].rrec = h->rain_rec.as<char>() + at[s];
+  return 0;
+}
+
 static int build_layout(dgswe_h h) {
   DeviceGuard dg_(h->device);
   CU(cudaStreamSynchronize(h->stream));  // steps of the state before may still run on what is replaced here
+  h->rain_rec.alloc(0);
   const int p = h->prm.p, np = np_of(p);
   const bool mx = mixed(h);
   h->np = np;
@@ -544,21 +573,6 @@ static int build_layout(dgswe_h h) {
     }
   }
   h->nn_total = N;
-  // gridded rain: element means of every record, where they fit (at most 8 GiB and a quarter of the
-  // free memory: 25 hourly records of 8M triangles are 0.8 GB); else a node kernel interpolates the
-  // grid at every stage
-  size_t rr_elems = 0, free_b = 0, total_b = 0;
-  std::vector<size_t> rr_off(ns, 0);
-  for (size_t s = 0; s < ns; ++s)
-    if (h->sc[s].rain_kind == 3) {
-      rr_off[s] = rr_elems;
-      rr_elems += (size_t)h->sc[s].gnt * h->sc[s].m.ne;
-    }
-  const size_t rr_bytes = (mx ? 4 : 8) * rr_elems;
-  CU(cudaMemGetInfo(&free_b, &total_b));
-  const bool records = rr_elems > 0 && rr_bytes <= std::min<size_t>((size_t)8 << 30, free_b / 4);
-  if (h->rain_rec.alloc(records ? rr_bytes : 0)) return fail(DGSWE_ENOMEM, "device allocation of %zu bytes failed", rr_bytes);
-  h->grid_rain = rr_elems > 0 && !records;
   CU(cudaMemset(h->ctl.p, 0, sizeof(Ctl)));
   CU(cudaMemset(h->scratch.p, 0, h->scratch.n));
   // per-scenario parameter blocks (dt filled in later)
@@ -573,7 +587,6 @@ static int build_layout(dgswe_h h) {
     D.rain_kind = S.rain_kind;
     D.gnx = S.gnx; D.gny = S.gny; D.gnt = S.gnt;
     D.grid = S.rain_kind == 3 ? h->grids.as<float>() + grid_off[s] : nullptr;
-    D.rrec = (records && S.rain_kind == 3) ? static_cast<const void*>(h->rain_rec.as<char>() + (mx ? 4 : 8) * rr_off[s]) : nullptr;
     D.rstride = S.m.ne;
     D.nseg = (int32_t)S.tamp.size();
     D.rnseg = S.rnseg;
@@ -631,6 +644,7 @@ static int build_layout(dgswe_h h) {
   if (mx) plan_bytes<Mixed>(h->ntiles, pb, pxb);
   else plan_bytes<Fp64>(h->ntiles, pb, pxb);
   if (h->stat.alloc(pb) || h->plan_x.alloc(pxb)) return fail(DGSWE_ENOMEM, "device allocation failed");
+  if (int rc = alloc_rain_records(h, sd)) return rc;
   CU(cudaMemcpy(h->scen.p, sd.data(), sizeof(ScenDev) * ns, cudaMemcpyHostToDevice));
   // every upload above ran on the default stream and may not have landed (a copy from pageable memory
   // returns before its transfer); the kernels below read them on a stream that does not wait for it
@@ -642,10 +656,11 @@ static int build_layout(dgswe_h h) {
   h->wcur = 0;
   for (size_t s = 0; s < ns; ++s) {
     if (!sd[s].rrec) continue;
+    void* to = const_cast<void*>(sd[s].rrec);
     cudaError_t ce = mx ? launch_rain_records<Mixed>(h->scen.as<ScenDev>(), (int)s, h->nodes.as<int4>(), h->xy64.as<double>(),
-                                                     h->sc[s].m.ne, sd[s].rstride, h->rain_rec.as<float>() + rr_off[s], h->stream)
+                                                     h->sc[s].m.ne, sd[s].rstride, static_cast<float*>(to), h->stream)
                         : launch_rain_records<Fp64>(h->scen.as<ScenDev>(), (int)s, h->nodes.as<int4>(), h->xy64.as<double>(),
-                                                    h->sc[s].m.ne, sd[s].rstride, h->rain_rec.as<double>() + rr_off[s], h->stream);
+                                                    h->sc[s].m.ne, sd[s].rstride, static_cast<double*>(to), h->stream);
     if (ce != cudaSuccess) return fail(DGSWE_ECUDA, "rain record launch: %s", cudaGetErrorString(ce));
     h->launches++;
   }

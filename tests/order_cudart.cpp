@@ -45,6 +45,10 @@ void on_default(const std::string& what, bool pending) {
   if (pending) uploads += (uploads.empty() ? "" : ", ") + what;
   else uploads.clear();
 }
+size_t free_bytes() {  // free device memory, as long as the test says so
+  const char* e = getenv("ORDER_FREE");
+  return e ? strtoull(e, nullptr, 10) : (size_t)200 << 30;
+}
 std::string sized(const char* op, size_t n) { return std::string(op) + " of " + std::to_string(n) + " bytes"; }
 }  // namespace
 
@@ -122,13 +126,17 @@ cudaError_t cudaEventRecord(cudaEvent_t e, cudaStream_t s) {
 cudaError_t cudaEventSynchronize(cudaEvent_t e) { return cudaStreamSynchronize(recorded[e]); }
 
 cudaError_t cudaMalloc(void** p, size_t n) {
-  *p = aligned_alloc(256, (n + 255) / 256 * 256);
+  *p = n > free_bytes() ? nullptr : aligned_alloc(256, (n + 255) / 256 * 256);
   return *p ? cudaSuccess : cudaErrorMemoryAllocation;
 }
 cudaError_t cudaFree(void* p) { free(p); return cudaSuccess; }
 cudaError_t cudaHostAlloc(void** p, size_t n, unsigned) { *p = calloc(1, n); return cudaSuccess; }
 cudaError_t cudaFreeHost(void* p) { free(p); return cudaSuccess; }
-cudaError_t cudaMemGetInfo(size_t* f, size_t* t) { *f = *t = (size_t)200 << 30; return cudaSuccess; }
+cudaError_t cudaMemGetInfo(size_t* f, size_t* t) {
+  *f = free_bytes();
+  *t = (size_t)280 << 30;
+  return cudaSuccess;
+}
 cudaError_t cudaGetSymbolAddress(void** p, const void* s) { *p = const_cast<void*>(s); return cudaSuccess; }
 cudaError_t cudaPointerGetAttributes(cudaPointerAttributes* a, const void*) {
   memset(a, 0, sizeof *a);

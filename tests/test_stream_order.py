@@ -147,3 +147,18 @@ s = D.from_workload(w, precision={prec}, dt=1.0)
 s.step(2)
 """, "order_launches").split("\n")[-2].split()
     assert ((want[0] in out[0] and (int(out[1]), int(out[2])) == want[1:]) if want else "steps_kernel" not in out[0])
+
+
+@pytest.mark.parametrize("free,node", [(200 << 30, False), (1 << 30, False), (100 << 20, True)])
+def test_rain_path_follows_the_size(runtime, free, node, monkeypatch):
+    """360 MB of rain records: element records whatever else the device holds, the node kernel only where
+    they do not fit."""
+    monkeypatch.setenv("ORDER_FREE", str(free))
+    out = _run(runtime, """
+w = basin(9, 5)
+w.rain_nodal = None
+w.rain_grid = W.RainGrid(2, 1, 1_000_000, 0.0, 0.0, 1e4, 1e4, 0.0, 60.0, np.ones((1_000_000, 1, 2), np.float32))
+s = D.from_workload(w, dt=1.0, block=64, split=2)
+s.step(1)
+""", "order_launches")
+    assert ("node_rain_kernel" in out) == node and ("rain_record_kernel" in out) != node
