@@ -237,9 +237,10 @@ __device__ __forceinline__ float frsqrt(float x) { return mufu_rsqrt(x); }  // x
 __device__ __forceinline__ double frsqrt(double x) { return hh_rsqrt(x); }
 __device__ __forceinline__ float fsqrt_pos(float x) { return x * mufu_rsqrt(x); }  // x > 0
 __device__ __forceinline__ double fsqrt_pos(double x) { return x * hh_rsqrt(x); }
-// sqrt(x) for x >= 0 (a squared speed or distance): below 1e-30, where it is negligible, at most 1e-15
+// sqrt(x) for x >= 0 (a squared speed or distance): below 1e-30 (FP64: 1e-290), where it is negligible, at
+// most 1e-15 (0); not a number of a run that has blown up stays one
 __device__ __forceinline__ float fsqrt0(float x) { return x * mufu_rsqrt(fmaxf(x, 1e-30f)); }
-__device__ __forceinline__ double fsqrt0(double x) { return x > 1e-290 ? x * hh_rsqrt(x) : 0.0; }
+__device__ __forceinline__ double fsqrt0(double x) { return x <= 1e-290 ? 0.0 : x * hh_rsqrt(x); }
 // H^{-4/3} = 2^(-4/3 log2 H)
 __device__ __forceinline__ float fpowm43(float h) { return mufu_ex2(-1.3333333f * mufu_lg2(h)); }
 // 1/H, and the depth factor of the friction law: H^{-4/3} (friction 0) or 1/H.  FP64 takes both from
