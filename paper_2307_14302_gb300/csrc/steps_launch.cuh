@@ -20,11 +20,9 @@ const StepsKernel<Pol>& steps_find(int p, int flux, int feat) {
   static const StepsKernel<Pol> generic[4] = {steps_entry<Pol, 1, 0, FT_ALL>(), steps_entry<Pol, 1, 1, FT_ALL>(),
                                               steps_entry<Pol, 2, 0, FT_ALL>(), steps_entry<Pol, 2, 1, FT_ALL>()};
   if constexpr (sizeof(typename Pol::T) == 4) {
-    static const StepsKernel<Pol> spec[] = {
-        steps_entry<Pol, 1, 0, FT_WALL_NODAL>(), steps_entry<Pol, 1, 0, FT_TIDE_STORM>(),
-        steps_entry<Pol, 1, 0, FT_TIDE_GRID>(), steps_entry<Pol, 2, 0, FT_TIDE_STORM_SETUP>(),
-        steps_entry<Pol, 1, 0, FT_TIDE_STORM | FT_GENSSP>(), steps_entry<Pol, 1, 0, FT_TIDE_GRID | FT_GENSSP>(),
-        steps_entry<Pol, 1, 1, FT_TIDE_STORM | FT_GENSSP>(), steps_entry<Pol, 1, 1, FT_TIDE_GRID | FT_GENSSP>()};
+#define DG_STEPS_SPEC(P, FLUX, FT) steps_entry<Pol, P, FLUX, FT>(),
+    static const StepsKernel<Pol> spec[] = {DG_SPECIALISED(DG_STEPS_SPEC)};
+#undef DG_STEPS_SPEC
     const int ft = tile_spec_features(p, flux, feat);
     for (const auto& k : spec)
       if (k.p == p && k.flux == flux && k.ft == ft) return k;

@@ -22,19 +22,9 @@ template <int P, int FLUX, int FT>
 constexpr Spec spec() {
   return {P, FLUX, FT, tile_kernel<P, FLUX, Mixed, FT>, tile_smem_bytes<P, Mixed, FT>(32)};
 }
-const Spec kSpecs[] = {
-    spec<1, 0, FT_WALL_NODAL>(),
-    spec<1, 0, FT_TIDE_STORM>(),
-    spec<1, 0, FT_TIDE_GRID>(),
-    spec<2, 0, FT_TIDE_STORM_SETUP>(),
-    // the other Runge-Kutta schemes and the LLF flux on the same families (LLF with five stages is the
-    // scheme of the paper's production runs): hurricane 500k LLF SSP(5,2) 168 -> 154 us per step against
-    // the generic instantiation
-    spec<1, 0, FT_TIDE_STORM | FT_GENSSP>(),
-    spec<1, 0, FT_TIDE_GRID | FT_GENSSP>(),
-    spec<1, 1, FT_TIDE_STORM | FT_GENSSP>(),
-    spec<1, 1, FT_TIDE_GRID | FT_GENSSP>(),
-};
+#define DG_SPEC(P, FLUX, FT) spec<P, FLUX, FT>(),
+const Spec kSpecs[] = {DG_SPECIALISED(DG_SPEC)};
+#undef DG_SPEC
 
 int bits(int x) {
   int n = 0;

@@ -4,6 +4,7 @@ The library's stream is non-blocking, so nothing orders it against uploads on th
 synchronisation.  A stand-in for the CUDA runtime (order_cudart.cpp, loaded before the real one in a child
 process) follows the calls of a few programs and reports every order that CUDA does not promise."""
 import os
+import re
 import subprocess
 import sys
 
@@ -162,3 +163,18 @@ s = D.from_workload(w, dt=1.0, block=64, split=2)
 s.step(1)
 """, "order_launches")
     assert ("node_rain_kernel" in out) == node and ("rain_record_kernel" in out) != node
+
+
+@pytest.mark.parametrize("workload,options", [
+    ("basin(9, 5)", ""), ("basin(9, 5)", "ssp_stages=3"), ("W.coastal_c2(800, seed=1, fast_mesh=True)", ""),
+    ("W.coastal_c2(800, seed=1, fast_mesh=True)", "ssp_stages=5, flux=D.FLUX_LLF"), ("W.inclined_plane('A', sim_s=1.0)", ""),
+    ("W.inclined_plane('A', sim_s=1.0)", "ssp_stages=3"), ("W.graded_c3(800)", ""), ("W.river_basin(nx=8, ny=4)", ""),
+])
+def test_both_kernels_take_the_same_instantiation(runtime, workload, options):
+    """The small-mesh kernel and the tile kernel of a run: equal template arguments."""
+    out = [_run(runtime, f"""
+s = D.from_workload({workload}, dt=1.0{launch}{options and ", " + options})
+s.step(2)
+""", "order_launches").split("\n")[-2] for launch in ("", ", block=64, split=2")]
+    args = [re.search(kernel + r"(I.*?5MixedE.*?E)Ev", o) for kernel, o in zip(("steps_kernel", "tile_kernel"), out)]
+    assert args[0] and args[1] and args[0].group(1) == args[1].group(1)
