@@ -204,6 +204,12 @@ struct Summary {
   long long wet;
   unsigned long long step;
 };
+constexpr int SUM_BLOCKS = 304;  // blocks of a summary launch at most: two per SM
+constexpr int SUM_WORDS = 9;     // partials of a block: four compensated sums and a count
+constexpr int DT_BLOCKS = 1024;  // blocks of a time-step launch at most
+// the scratch array of both, in doubles: partials, then the summary's block counter
+constexpr int SCRATCH = SUM_WORDS * SUM_BLOCKS + 1;
+static_assert(DT_BLOCKS < SCRATCH, "the time step's partials end before the counter");
 template <class Pol>
 cudaError_t launch_summary(int p, bool depth, const uint4* rec, const uint4* geo, long long begin, long long end,
                            const double* led, int nled, const Ctl* ctl, double* partials, unsigned* ticket, Summary* out,

@@ -1995,7 +1995,7 @@ __global__ void __launch_bounds__(SUM_BLOCK) summary_kernel(const uint4* rec, co
     const double a2 = __shfl_down_sync(0xffffffffu, a, o), b2 = __shfl_down_sync(0xffffffffu, b, o);
     neu_merge(a, b, a2, b2);
   }
-  double* part = partials + 9 * (long long)blockIdx.x;
+  double* part = partials + SUM_WORDS * (long long)blockIdx.x;
   if (lane == 0) {
     part[2 * w] = a;
     part[2 * w + 1] = b;
@@ -2013,7 +2013,7 @@ __global__ void __launch_bounds__(SUM_BLOCK) summary_kernel(const uint4* rec, co
   __threadfence();
   a = b = 0.0;
   for (int k = lane; k < (int)gridDim.x; k += 32)
-    neu_merge(a, b, __ldcg(partials + 9 * (long long)k + 2 * w), __ldcg(partials + 9 * (long long)k + 2 * w + 1));
+    neu_merge(a, b, __ldcg(partials + SUM_WORDS * (long long)k + 2 * w), __ldcg(partials + SUM_WORDS * (long long)k + 2 * w + 1));
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
     const double a2 = __shfl_down_sync(0xffffffffu, a, o), b2 = __shfl_down_sync(0xffffffffu, b, o);
@@ -2022,7 +2022,7 @@ __global__ void __launch_bounds__(SUM_BLOCK) summary_kernel(const uint4* rec, co
   if (lane == 0) out->sum[w] = a + b;
   if (w == 0) {
     long long n = 0;
-    for (int k = lane; k < (int)gridDim.x; k += 32) n += (long long)__ldcg(partials + 9 * (long long)k + 8);
+    for (int k = lane; k < (int)gridDim.x; k += 32) n += (long long)__ldcg(partials + SUM_WORDS * (long long)k + 8);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) n += __shfl_down_sync(0xffffffffu, n, o);
     if (lane == 0) {

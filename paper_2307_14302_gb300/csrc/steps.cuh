@@ -65,7 +65,7 @@ __global__ void __maxnreg__(sizeof(typename Pol::T) == 4 ? (P == 1 ? 128 : 200) 
   __shared__ float4 s_ephi4[P == 1 ? 3 : 15];
   extern __shared__ uint4 tsm[];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  for (int i = tid; i < 3 * NG * NP; i += blockDim.x) {
+  for (int i = tid; sizeof(T) == 8 && i < 3 * NG * NP; i += blockDim.x) {
     const int j = i / (NG * NP), k = (i / NP) % NG, m = i % NP;
     s_ephi[j][k][m] = tab.ephi[j][k][m];
   }

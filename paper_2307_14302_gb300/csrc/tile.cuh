@@ -42,7 +42,6 @@ namespace dg {
 
 constexpr int HALO = 32;    // staged out-of-tile neighbour records per tile
 static_assert(HALO == TILE, "own and halo records share one vector stride in shared memory");
-constexpr int TE_MAX = 96;  // edges touching a 32-element tile (3 per element at most)
 
 // The tile plan: what the neighbour codes say about a tile's edges, laid out once per mesh by
 // plan_kernel (the connectivity never changes) and copied with the tile's other data.  One 32-bit
@@ -1297,12 +1296,12 @@ __global__ void DG_TILE_BOUNDS tile_kernel(const StageArgs<Pol> a) {
   constexpr int NP = np_of(P), NG = P + 1, RV = L::RV;
   const RefTab<T>& tab = ctab<T, P>();
 
-  // edge basis values, read at edge-dependent indices; in FP32 as rows of 16 bytes (side_traces)
+  // edge basis values, read at edge-dependent indices; in FP32 as rows of 16 bytes alone (side_traces)
   __shared__ T s_ephi[3][NG][NP];
   __shared__ float4 s_ephi4[P == 1 ? 3 : 15];
   extern __shared__ uint4 tsm[];
   const int tid = threadIdx.x;
-  for (int i = tid; i < 3 * NG * NP; i += blockDim.x) {
+  for (int i = tid; sizeof(T) == 8 && i < 3 * NG * NP; i += blockDim.x) {
     const int j = i / (NG * NP), k = (i / NP) % NG, m = i % NP;
     s_ephi[j][k][m] = tab.ephi[j][k][m];
   }
