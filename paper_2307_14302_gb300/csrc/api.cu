@@ -127,7 +127,7 @@ struct dgswe_ctx {
   int np = 0, rv = 0, gv = 0;      // modes, record and geometry sizes (16-byte units)
   long long E = 0, N = 0;          // padded element count, node count
   std::vector<long long> eoff, noff;
-  DevBuf rec[3], nbr, geo, nodes, node_xy, xy64, hbn, rain_e, rain_node, node_scen, lim, rain_rec, scen, tile_scen, tile_meta, stat, plan_x,
+  DevBuf rec[3], nbr, geo, nodes, node_xy, xy64, hbn, rain_e, rain_node, node_scen, lim, rain_rec, rain_place, scen, tile_scen, tile_meta, stat, plan_x,
       ledger, ctl,
       einv, grids, rivers, scratch,
       gather_buf, edges, slots;
@@ -166,7 +166,7 @@ struct dgswe_ctx {
     DevBuf* bufs[] = {&rec[0], &rec[1], &rec[2], &nbr, &geo, &nodes, &node_xy, &xy64, &hbn, &rain_e, &scen,
                       &tile_scen, &tile_meta, &ledger, &ctl, &einv, &grids, &rivers, &scratch, &gather_buf,
                       &edges, &slots,
-                      &rain_node, &node_scen, &lim, &rain_rec, &stat, &plan_x};
+                      &rain_node, &node_scen, &lim, &rain_rec, &rain_place, &stat, &plan_x};
     for (DevBuf* b : bufs) b->alloc(0);
     if (sum) cudaFreeHost(sum);
     drop_graphs();
@@ -363,16 +363,20 @@ static int alloc_rain_records(dgswe_h h, std::vector<ScenDev>& sd) {
     need += word * sd[s].gnt * (size_t)h->sc[s].m.ne;
   }
   h->grid_rain = need > 0;
-  if (need == 0 || need > (size_t)8 << 30) return 0;
-  CU(cudaMemGetInfo(&free_b, &total_b));
-  if (need + staging > free_b) return 0;
-  if (h->rain_rec.alloc(need)) {
-    cudaGetLastError();  // the node kernel takes over
-    return 0;
+  if (need == 0) return 0;
+  bool fits = need <= (size_t)8 << 30;
+  if (fits) {
+    CU(cudaMemGetInfo(&free_b, &total_b));
+    fits = need + staging <= free_b;
   }
-  h->grid_rain = false;
-  for (size_t s = 0; s < sd.size(); ++s)
+  if (fits && h->rain_rec.alloc(need)) {
+    cudaGetLastError();  // the node kernel takes over
+    fits = false;
+  }
+  h->grid_rain = !fits;
+  for (size_t s = 0; fits && s < sd.size(); ++s)
     if (sd[s].rain_kind == 3) sd[s].rrec = h->rain_rec.as<char>() + at[s];
+  if (!fits && mixed(h) && h->rain_place.alloc(16 * (size_t)h->N)) return fail(DGSWE_ENOMEM, "device allocation failed");
   return 0;
 }
 
@@ -380,6 +384,7 @@ static int build_layout(dgswe_h h) {
   DeviceGuard dg_(h->device);
   CU(cudaStreamSynchronize(h->stream));  // steps of the state before may still run on what is replaced here
   h->rain_rec.alloc(0);
+  h->rain_place.alloc(0);
   const int p = h->prm.p, np = np_of(p);
   const bool mx = mixed(h);
   h->np = np;
@@ -654,6 +659,11 @@ static int build_layout(dgswe_h h) {
                                                    h->stat.as<uint4>(), h->plan_x.as<int32_t>(), h->stream));
   h->launches++;
   h->wcur = 0;
+  if (h->rain_place.p) {
+    CU(launch_node_places<Mixed>(h->scen.as<ScenDev>(), h->node_scen.as<int32_t>(), h->xy64.as<double>(), N, h->rain_place.p,
+                                 h->stream));
+    h->launches++;
+  }
   for (size_t s = 0; s < ns; ++s) {
     if (!sd[s].rrec) continue;
     void* to = const_cast<void*>(sd[s].rrec);
@@ -789,8 +799,8 @@ static int launch_stage_once(dgswe_h h, int stage, int tune, cudaStream_t s) {
   const int grid = h->grid;
   cudaError_t e = cudaSuccess;
   if (h->grid_rain) {  // nodal gridded rain at this stage's time
-    e = mixed(h) ? launch_node_rain<Mixed>(make_args<Mixed>(h, stage, tune), h->xy64.as<double>(), h->nn_total, s)
-                 : launch_node_rain<Fp64>(make_args<Fp64>(h, stage, tune), h->xy64.as<double>(), h->nn_total, s);
+    e = mixed(h) ? launch_node_rain<Mixed>(make_args<Mixed>(h, stage, tune), h->xy64.as<double>(), h->rain_place.p, h->nn_total, s)
+                 : launch_node_rain<Fp64>(make_args<Fp64>(h, stage, tune), h->xy64.as<double>(), nullptr, h->nn_total, s);
     if (e != cudaSuccess) return fail(DGSWE_ECUDA, "node rain launch: %s", cudaGetErrorString(e));
     h->launches++;
   }

@@ -192,7 +192,12 @@ template <class Pol>
 cudaError_t launch_limiter(const StageArgs<Pol>& a, long long ne, cudaStream_t s);
 // gridded rain (rain_kind 3) interpolated to every node at the stage time: a.rain_node[0, nn)
 template <class Pol>
-cudaError_t launch_node_rain(const StageArgs<Pol>& a, const double* xy64, long long nn, cudaStream_t s);
+cudaError_t launch_node_rain(const StageArgs<Pol>& a, const double* xy64, const void* place, long long nn,
+                             cudaStream_t s);
+// mixed path: every node's cell of its scenario's rain grid and the position in it, 16 bytes per node
+template <class Pol>
+cudaError_t launch_node_places(const ScenDev* scen, const int32_t* node_scen, const double* xy64, long long nn,
+                               void* place, cudaStream_t s);
 // gridded rain of every record averaged to the elements of one scenario: rrec[record][element], m/s
 template <class Pol>
 cudaError_t launch_rain_records(const ScenDev* scen, int sc, const int4* nodes, const double* xy64, long long ne,

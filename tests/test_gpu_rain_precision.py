@@ -59,3 +59,33 @@ def test_the_node_kernel_agrees_to_rounding():
         rain.append(dev.ledger()["rain_in"])
         dev.close()
     assert abs(rain[0] / rain[1] - 1) <= 10 * 2.0**-24
+
+
+@pytest.mark.parametrize("prec", [D.FP64, D.MIXED])
+def test_members_of_an_ensemble_keep_their_own_grids_in_the_node_kernel(prec):
+    """Two small gridded members beside one whose records are beyond 8 GiB: nodes of different scenarios
+    share blocks.  Their rain is that of their solo runs, which go through records."""
+    big = W.coastal_c2(500_000, seed=3, fast_mesh=True)
+    big.storm = None
+    nt = 4400 if prec == D.MIXED else 2200
+    big.rain_grid = W.RainGrid(1, 1, nt, 0.0, 0.0, 1.0, 1.0, 0.0, 60.0, np.full((nt, 1, 1), 5.0, np.float32))
+    ws = []
+    for k in (2, 3):
+        w = W.basin_c1(nx=5 * k, ny=4)
+        w.rain_nodal = None
+        f = np.random.default_rng(k).uniform(0, 100, (k, 3, 4)).astype(np.float32)
+        w.rain_grid = W.RainGrid(4, 3, k, 0.0, 0.0, 3e3, 2e3, 0.0, 0.7 * k, f)
+        ws.append(w)
+    ens = D.Ensemble([D.from_workload(w, precision=prec, dt=0.2, block=64, split=2) for w in [ws[0], big, ws[1]]])
+    ens.set_launch(64, 1, 2)
+    n0 = ens.launch_count()
+    ens.step(5)
+    assert ens.launch_count() - n0 == 20  # a node launch per stage
+    ens.sync()
+    for i, w in ((0, ws[0]), (2, ws[1])):
+        s = D.from_workload(w, precision=prec, dt=0.2, block=64, waves=1, split=2)
+        s.step(5)
+        s.sync()
+        assert abs(ens.ledger(i)["rain_in"] / s.ledger()["rain_in"] - 1) <= (10 * 2.0**-24 if prec == D.MIXED else 1e-13)
+        s.close()
+    ens.close()
