@@ -117,8 +117,6 @@ __device__ __forceinline__ ff acc_addmul(ff s, ff a, float b) {
   const ff t = two_sum(s.hi, p);
   return {t.hi, __fadd_rn(s.lo, __fadd_rn(t.lo, __fmaf_rn(a.lo, b, __fmaf_rn(a.hi, b, -p))))};
 }
-__device__ __forceinline__ double acc_norm(double a) { return a; }
-__device__ __forceinline__ ff acc_norm(ff a) { return quick_two_sum(a.hi, a.lo); }
 // sum of very many values: doubles, or pairs of floats in three words (the roundings of the first two are
 // kept, so that equal addends do not round the same way every time)
 struct fff {

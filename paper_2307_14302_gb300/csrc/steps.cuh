@@ -99,14 +99,14 @@ __global__ void __maxnreg__(sizeof(typename Pol::T) == 4 ? (P == 1 ? 128 : 200) 
   const unsigned long long step0 = a.ctl->step;
   const int rain_kind = ft_rain(FT) >= 0 ? ft_rain(FT) : S.rain_kind;
   const int press = (FT & FT_PRESS) ? S.press : 0;
-  // ledger: the lane's volumes of a step in the path's accumulation type, those of the launch in three
-  // floats (mixed): a pair over the whole launch rounds a steady rain's equal addends the same way every
-  // time, 2e-12 of the volume after 1,000 steps of SSP(5,2), where the tile form, which books in FP64
-  // after every stage, keeps 1e-14.  Flume: 6.52 us per step with a pair, 6.57 with three words, 6.92
-  // with an FP64 sum.
+  // ledger: a lane's volumes of the launch in three floats (mixed).  A pair over the whole launch rounds a
+  // steady rain's equal addends the same way every time, 2e-12 of the volume after 1,000 steps of
+  // SSP(5,2), where the tile form, which books in FP64 after every stage, keeps 1e-14.  us per step with a
+  // pair and so: 400 triangles 5.0 and 4.9, flume 6.5 and 6.3, 4.8k river LLF SSP(5,2) 21.6 and 22.0 (445
+  // and 460 us per 20 steps); an FP64 sum per step took the flume to 6.9, three floats per step instead of
+  // per stage the 400 triangles to 5.45.
   typename LongSum<Acc>::type rain_sum = {}, bdry_sum = {};
   for (int n = 0; n < st.nsteps; ++n) {
-    Acc rain_tot = acc_make<Acc>(0.f, 0.f, 0.0), bdry_tot = acc_make<Acc>(0.f, 0.f, 0.0);
     for (int s = 0; s < st.nstage; ++s) {
       const StepsArgs::Stage& c = st.st[s];
       const uint32_t rin = 16u * SL::RECS * c.in;
@@ -147,10 +147,8 @@ __global__ void __maxnreg__(sizeof(typename Pol::T) == 4 ? (P == 1 ? 128 : 200) 
       }
       Storm<T> storm = {};
       if constexpr (storm_regs<P, FT>()) storm = storm_at<T>(S, t64);
-      // equal stage weights (SSP(2,2), SSP(5,2)): the volumes accumulate over stages as they are and take
-      // the weight at the end of the launch
       const Acc zero = acc_make<Acc>(0.f, 0.f, 0.0);
-      Acc rain_acc = st.same_bw ? rain_tot : zero, bdry_acc = st.same_bw ? bdry_tot : zero;
+      Acc rain_acc = zero, bdry_acc = zero;
       Elem<P, Pol> O;
       tile_body<P, FLUX, Pol, FT, true>(a, S, t64, rain_kind, press, rr, storm, tile, lane, valid, meta.z, meta.w,
                                         Wm + SL::REC + c.in * SL::RECS, halo, Wm + SL::GEO,
@@ -176,20 +174,18 @@ __global__ void __maxnreg__(sizeof(typename Pol::T) == 4 ? (P == 1 ? 128 : 200) 
 #pragma unroll
         for (int v = 0; v < RV; ++v) to[v * TILE + lane] = ro.v[v];
       }
-      // ledger: the stage's volume rates with its weight in the step
-      if (st.same_bw) {
-        rain_tot = acc_norm(rain_acc);
-        bdry_tot = bdry_acc;
-      } else {
-        const Acc bw = acc_make<Acc>(c.bw_hi, c.bw_lo, c.bw);
-        rain_tot = acc_add(rain_tot, acc_mul(rain_acc, bw));
-        bdry_tot = acc_add(bdry_tot, acc_mul(bdry_acc, bw));
-      }
       __syncwarp();
       cluster_arrive();
+      // the stage's volume rates with its weight in the step; equal weights (SSP(2,2), SSP(5,2)) come at the
+      // end of the launch
+      if (!st.same_bw) {
+        const Acc bw = acc_make<Acc>(c.bw_hi, c.bw_lo, c.bw);
+        rain_acc = acc_mul(rain_acc, bw);
+        bdry_acc = acc_mul(bdry_acc, bw);
+      }
+      long_add(rain_sum, rain_acc);
+      long_add(bdry_sum, bdry_acc);
     }
-    long_add(rain_sum, rain_tot);
-    long_add(bdry_sum, bdry_tot);
   }
   cluster_wait();  // no CTA leaves while another reads its records
   if (present > 0) {
